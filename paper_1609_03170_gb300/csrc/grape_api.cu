@@ -277,6 +277,8 @@ struct grape_problem {
     int fold = 0;                    // Hermitian kernel: own-entry coefficients cached in shared memory
     int jcache = 0;                  // Hermitian kernel: jump coefficients cached per entry
     int defer = 0;                   // Hermitian kernel: cluster wait after the compute
+    int raw = 0;                     // prop_s_kernel: A0 and every A_k in shared memory
+    int dconst = 0;                  // no control has an offset-0 band
     int omax = 0;                    // largest band offset of either Lindbladian
     int hb_h = 0;                    // lower entries the Hermitian stencil reads
     std::map<int, int *> htabs;      // Hermitian tables per cluster width
@@ -657,6 +659,23 @@ std::vector<int> hermitian_table(int d, int ncl, int omax, int hb, int *maxwin, 
     tab.insert(tab.end(), lists.begin(), lists.end());
     tab.insert(tab.end(), kf.begin(), kf.end());
     tab.insert(tab.end(), kl.begin(), kl.end());
+    // window slots peers write each stage: slot (r, c) of CTA k's window holds
+    // the upper entry (r, c), c >= r, or the mirror of (c, r); its writer is
+    // the owner of that upper entry, so a row's slots from the diagonal on
+    // are consecutive entries of which k owns a range
+    for (int k = 0; k < ncl; ++k) {
+        const long long u0 = head[4 * k], u1 = head[4 * k + 1];
+        long long n = 0;
+        for (int r = wr0[k]; r <= wr1[k]; ++r) {
+            const long long a = row_start(r), b = a + d - r;
+            n += (b - a) - std::max(0LL, std::min(b, u1) - std::max(a, u0));
+            for (int c = cs(r); c < r; ++c) {
+                const long long u = row_start(c) + (r - c);
+                if (u < u0 || u >= u1) ++n;
+            }
+        }
+        tab.push_back((int)n);
+    }
     *maxwin = mw;
     *cu = c;
     *rt_rows = rt;
@@ -704,8 +723,49 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
                         (size_t)rt_rows * (2 * ncl + 1) * sizeof(uint32_t) +
                         (size_t)cu * (2 * nb + nt + 1) * sizeof(short);
     const int sh = shape_id(P);
-    const int variant = (P->variant & 1) | 2 | (sh << 2) | ((sh && cu <= threads) ? 16 : 0);
-    {
+    // Options of prop_h_kernel, each kept only when the tile still fits
+    // (the same values, so the same bits, either way): the own-entry
+    // coefficients cached per slice (16 B per owned entry) instead of
+    // recomputed every stage; the next values of the owned entries kept in a
+    // row (16 B per owned entry) so that the cluster wait before the pushes
+    // comes after the compute; the jump coefficients of real jump tables
+    // cached per entry (8 B per term with an offset and owned entry).
+    bool want_fold = true, want_defer = false, want_jc = (P->variant & 1) != 0;
+    if (const char *env = std::getenv("GRAPE_FOLD")) want_fold = std::atoi(env) != 0;
+    if (const char *env = std::getenv("GRAPE_DEFER")) want_defer = std::atoi(env) != 0;   // off: measured slower
+    if (const char *env = std::getenv("GRAPE_JCACHE")) want_jc = want_jc && std::atoi(env) != 0;
+    // prop_s_kernel for the known shapes wherever its tile fits: the
+    // operators' tables in shared memory for the per-slice rebuild when there
+    // is room for them, else read from global memory.
+    size_t use = 0;
+    int variant = 0;
+    bool found = false, fold = false, defer = false, jcache = false, raw = false;
+    if (sh && want_fold && want_jc && !want_defer) {
+        const size_t wbytes = (size_t)(maxwin + 1) * sizeof(double2);
+        const bool one = cu <= threads && wbytes <= GRAPE_WOFF, small = one && wbytes <= GRAPE_WOFF_SMALL;
+        const size_t pbase = (one ? (small ? GRAPE_WOFF_SMALL : GRAPE_WOFF) : wbytes) + wbytes +
+                             (size_t)8 * d * sizeof(double2) + tab.size() * sizeof(int) +
+                             (size_t)rt_rows * (2 * ncl + 1) * sizeof(uint32_t) +
+                             (one ? 0 : (size_t)cu * (2 * sizeof(double2) + (2 + nt) * sizeof(double) + sizeof(int2) +
+                                                      (2 * (nb - 1) + 1 + nt) * sizeof(short)));
+        variant = (P->variant & 1) | 2 | (sh << 2) | (one ? 16 : 0) | 32 | (small ? 64 : 0);
+        const cudaError_t e = P->prec == GRAPE_PREC_FP64
+                                  ? grape_prepare_prop_f64(variant, (size_t)max_smem, 16)
+                                  : grape_prepare_prop_df(variant, (size_t)max_smem, 16);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return fail(GRAPE_ECUDA, std::string("hermitian kernel attributes: ") + cudaGetErrorString(e));
+        }
+        for (int with_raw = 1; with_raw >= 0 && !found; --with_raw) {
+            const size_t sm = pbase + (with_raw ? (size_t)(1 + P->R) * nb * d * sizeof(double2) : 0);
+            if (sm + 1024 > (size_t)max_smem || !cluster_fits(P, variant, threads, sm, ncl)) continue;
+            use = sm;
+            raw = with_raw != 0;
+            found = true;
+        }
+    }
+    if (!found) variant = (P->variant & 1) | 2 | (sh << 2);
+    if (!found) {
         const cudaError_t e = P->prec == GRAPE_PREC_FP64
                                   ? grape_prepare_prop_f64(variant, (size_t)max_smem_optin(P), 16)
                                   : grape_prepare_prop_df(variant, (size_t)max_smem_optin(P), 16);
@@ -714,18 +774,6 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
             return fail(GRAPE_ECUDA, std::string("hermitian kernel attributes: ") + cudaGetErrorString(e));
         }
     }
-    // Options, each kept only when the tile still fits (the same values, so
-    // the same bits, either way): the own-entry coefficients cached per slice
-    // (16 B per owned entry) instead of recomputed every stage; the next
-    // values of the owned entries kept in a row (16 B per owned entry) so
-    // that the cluster wait before the pushes comes after the compute; the
-    // jump coefficients of real jump tables cached per entry (8 B per term
-    // with an offset and owned entry).
-    bool want_fold = true, want_defer = false, want_jc = (variant & 1) != 0;
-    if (const char *env = std::getenv("GRAPE_FOLD")) want_fold = std::atoi(env) != 0;
-    if (const char *env = std::getenv("GRAPE_DEFER")) want_defer = std::atoi(env) != 0;   // off: measured slower
-    if (variant & 16) want_defer = false;        // one entry per thread: the wait stays before the compute
-    if (const char *env = std::getenv("GRAPE_JCACHE")) want_jc = want_jc && std::atoi(env) != 0;
     int njt = 0;
     for (int q = 0; q < P->tab[0].nt; ++q) njt += ((P->tab[0].jdiag >> q) & 1) ? 0 : 1;
     int njt_d = 0;
@@ -734,9 +782,8 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
     struct Opt { bool fold, defer, jc; };
     const Opt opts[] = {{true, true, true}, {true, true, false}, {true, false, true}, {true, false, false},
                         {false, true, false}, {false, false, false}};
-    size_t use = 0;
-    bool found = false, fold = false, defer = false, jcache = false;
     for (const Opt &o : opts) {
+        if (found) break;
         if ((o.fold && !want_fold) || (o.defer && !want_defer) || (o.jc && !want_jc)) continue;
         const size_t sm = base + 2 * (size_t)(maxwin + 1) * sizeof(double2) +
                           (o.fold ? (size_t)cu * sizeof(double2) : 0) +
@@ -748,7 +795,6 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
         defer = o.defer;
         jcache = o.jc;
         found = true;
-        break;
     }
     if (!found) {
         const size_t least = base + 2 * (size_t)(maxwin + 1) * sizeof(double2);
@@ -775,6 +821,7 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
 
     P->jcache = jcache ? 1 : 0;
     P->defer = defer ? 1 : 0;
+    P->raw = raw ? 1 : 0;
     P->threads = threads;
     P->chunk = cu;
     P->halo = 0;
@@ -935,6 +982,7 @@ grape_status choose_geometry_grid(grape_problem *P) {
 }
 
 void rk_coefficients(double h, bool adjoint, PropArgs *a) {
+    a->unit_g = adjoint ? 0 : 1;
     if (!adjoint) {
         const double g[4] = {1.0, 1.0, 1.0, 1.0};
         const double w[4] = {h / 6, h / 3, h / 3, h / 6};
@@ -947,6 +995,15 @@ void rk_coefficients(double h, bool adjoint, PropArgs *a) {
         const double b[4] = {0.0, h, h / 2, h / 2};
         for (int s = 0; s < 4; ++s) { a->g[s] = g[s]; a->a[s] = 1.0; a->b[s] = b[s]; a->store_map[s] = 3 - s; }
     }
+    auto ffs = [](const double (&v)[4], float2 (&o)[4]) {
+        for (int s = 0; s < 4; ++s) {
+            const grape_num::ff f = grape_num::ff_from_double(v[s]);
+            o[s] = make_float2(f.h, f.l);
+        }
+    };
+    ffs(a->g, a->gf);
+    ffs(a->a, a->af);
+    ffs(a->b, a->bf);
 }
 
 PropArgs base_args(const grape_problem *P, int dir, const double *u) {
@@ -974,6 +1031,8 @@ PropArgs base_args(const grape_problem *P, int dir, const double *u) {
 
     a.jcache = ((P->variant & 2) || P->grid) ? P->jcache : 0;
     a.defer = (P->variant & 2) ? P->defer : 0;
+    a.raw = P->raw;
+    a.dconst = P->dconst;
     a.src = P->penalty ? P->d_src : nullptr;
     a.gbuf = P->d_gbuf;
     a.gbar = P->d_gbar;
@@ -1764,6 +1823,8 @@ grape_status grape_problem_create(const grape_problem_desc *desc, grape_problem_
     bool placed = false;
     P->omax = omax;
     P->hb_h = hb;
+    P->dconst = 1;
+    for (const Bands &B : Ak) P->dconst = P->dconst && !B.count(0);
     if (kern != "grid" && herm) {
         st = choose_geometry_h(P);
         if (st != GRAPE_OK && st != GRAPE_EINVAL) return bail(st);

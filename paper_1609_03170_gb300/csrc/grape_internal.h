@@ -12,6 +12,8 @@
 #define GRAPE_MAXDO 8    // distinct band offsets among the control bands
 #define GRAPE_MAXST 4    // sandwich terms of dissipators whose rate is a control
 #define GRAPE_PROP_THREADS 512   // threads per CTA of the propagation kernel
+#define GRAPE_WOFF_SMALL 8192    // bytes between prop_s_kernel's two windows, one entry per thread
+#define GRAPE_WOFF 32768
 
 // One direction of the Lindblad action in the common form
 //   W = -i (A X - X A^+) + sum_t vL_t[i] conj(vR_t[j]) X[i + oL_t][j + oR_t]
@@ -57,6 +59,9 @@ struct PropArgs {
     long long sub_begin, sub_end;       // substep range
     int reverse;
     double g[4], a[4], b[4];
+    float2 gf[4], af[4], bf[4];         // the same as double-float numbers (hi, lo)
+    int unit_g;                         // g is 1 in every stage (an integer: a comparison of doubles
+                                        // in the kernels would be repeated, on the FP64 pipe)
     int store_map[4];                   // stage s -> slot of the stage store
     // state buffers are in the kernel's storage format (16 bytes per complex
     // entry: double2 for FP64, float4 hi/lo pairs for double-float)
@@ -79,6 +84,8 @@ struct PropArgs {
                                         // jump terms cached per owned entry
     int defer;                          // Hermitian kernel: next values kept until the cluster
                                         // wait before the pushes (hides its latency)
+    int raw;                            // prop_s_kernel: A0 and every A_k kept in shared memory
+    int dconst;                         // prop_s_kernel: own-entry coefficients the same in every slice
     const double *src;                  // adjoint source on the diagonal per row (App. B), or null
     // grid kernel (stage values in global memory, windows loaded per stage;
     // ncl = CTAs per state, htab/maxwin/cu/hb as for the Hermitian kernel)
@@ -99,6 +106,7 @@ struct PropArgs {
 //   [4 ncl + k]            start of CTA k's row-offset list (k = 0..ncl)
 //   [row-offset lists]     CTA k: nrows_k + 1 cumulative window offsets
 //   [kfirst[d], klast[d]]  first and last CTA whose window holds row r
+//   [ncl]                  window slots of CTA k that its peers write each stage
 #define GRAPE_HTAB_CTA(k) (4 * (k))
 #define GRAPE_HTAB_LISTS(ncl) (4 * (ncl))
 

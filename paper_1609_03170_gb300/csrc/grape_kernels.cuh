@@ -8,9 +8,10 @@
 //                 cluster, upper triangle only (every stage value is
 //                 Hermitian); the state stays in the cluster's shared memory
 //                 as compact row windows, halo values are pushed with st.async
-//                 and counted on the receiving window's mbarrier.  The default
-//                 kernel; specialised on the band/jump layout (Shape) and on
-//                 one entry per thread.
+//                 and counted on the receiving window's mbarrier.  Any band and
+//                 jump layout.
+//  prop_s_kernel  the same for the band/jump layouts known at compile time
+//                 (Shape), with few instructions per entry; the default.
 //  prop_kernel    the same over contiguous chunks of the full matrix (when the
 //                 Hermitian windows do not fit).
 //  prop_g_kernel  the Hermitian kernel's arithmetic over CTAs of the whole
@@ -387,47 +388,19 @@ using ShapeR = Shape<3, 0, 1>;   // resonator drives only: bands 0, +-Q; jump a
 template <class SH> __device__ __forceinline__ int sh_nb(const PropTables &t) { return SH::NB ? SH::NB : t.nb; }
 template <class SH> __device__ __forceinline__ int sh_nt(const PropTables &t) { return SH::NB ? SH::NT : t.nt; }
 
-// The Hamiltonian bands: the first t.nbr are real for every control value
-// (real multiply-adds: the same bits as the complex ones with a zero
-// imaginary part, half the work), the offset-0 band is last and excluded
-// (it is part of the own-entry coefficient).  x1(b), x2(b): the neighbours
-// (i + o_b, j) and (i, j + o_b).  The A X terms and the X A^+ terms go to
-// two accumulators (two independent dependency chains), added at the end
-// (four, real and complex bands apart, measured 3 % slower).
-template <class Num, class SH, class X1, class X2>
-__device__ __forceinline__ typename Num::acc band_terms(const PropTables &t, const typename Num::store_t *A,
-                                                        int i, int j, int d, X1 &&x1, X2 &&x2) {
-    typename Num::acc wa = Num::acc_zero(), wb = Num::acc_zero();
-    if constexpr (SH::NB > 0) {
-#pragma unroll
-        for (int b = 0; b < SH::NBR; ++b) {
-            Num::mac_real(wa, Num::load_re(A[b * d + i]), x1(b));
-            Num::mac_real(wb, Num::neg_real(Num::load_re(A[b * d + j])), x2(b));
-        }
-#pragma unroll
-        for (int b = SH::NBR; b < SH::NB - 1; ++b) {
-            Num::mac(wa, Num::load(A[b * d + i]), x1(b));
-            Num::mac_conj_neg(wb, Num::load(A[b * d + j]), x2(b));
-        }
-    } else {
-        const int nbo = (t.b0 >= 0) ? t.nb - 1 : t.nb;
-#pragma unroll 1
-        for (int b = 0; b < t.nbr; ++b) {
-            Num::mac_real(wa, Num::load_re(A[b * d + i]), x1(b));
-            Num::mac_real(wb, Num::neg_real(Num::load_re(A[b * d + j])), x2(b));
-        }
-#pragma unroll 2
-        for (int b = t.nbr; b < nbo; ++b) {
-            Num::mac(wa, Num::load(A[b * d + i]), x1(b));
-            Num::mac_conj_neg(wb, Num::load(A[b * d + j]), x2(b));
-        }
-    }
-    return Num::acc_add(wa, wb);
-}
-
+// W = Op(z) at an owned upper entry, W = U + i T: every product has a real
+// coefficient, U sums those of the real parts and T those of the imaginary
+// parts of the coefficients, in the order written here (the Hermitian
+// kernels all keep it, so they give the same bits):
+//   bands with real values (the first t.nbr):  T -= A_b[i] x1,  T += A_b[j] x2
+//   other bands (the offset-0 band is last and excluded, it is part of the
+//   own-entry coefficient):  U += im A_b[i] x1,  T -= re A_b[i] x1,
+//                            U += im A_b[j] x2,  T += re A_b[j] x2
+//   own entry:  U += re D_ij x,  T += im D_ij x;  jump terms with an offset.
+// x1 and x2 are the neighbours (i + o_b, j) and (i, j + o_b).
 // jc: null, or the entry's cached coefficients of the jump terms with an
 // offset (real tables only), jc[q' * jstride] for the q'-th such term
-template <class Num, bool REALJ, class SH, bool JQ = false>
+template <class Num, bool REALJ, class SH>
 __device__ __forceinline__ typename Num::val lindblad_h_at(const typename Num::store_t *cur,
                                                            const short *nb_ad, int i, int j, int d,
                                                            const PropTables &t,
@@ -439,39 +412,37 @@ __device__ __forceinline__ typename Num::val lindblad_h_at(const typename Num::s
                                                            const typename Num::real_t *jc, int jstride) {
     // neighbours outside the matrix point at the window's zero slot, so
     // every term is accumulated without a branch (adding 0 changes no bit).
-    // The terms on the entry itself - the offset-0 band and the jump terms
-    // with both offsets 0 - come as one coefficient D_ij (diag_coef).
+    using V = typename Num::val;
     const int nb = sh_nb<SH>(t), nt = sh_nt<SH>(t);
-    typename Num::acc w = band_terms<Num, SH>(t, A, i, j, d, [&](int b) { return Num::load(cur[nb_ad[2 * b]]); },
-                                              [&](int b) { return Num::load(cur[nb_ad[2 * b + 1]]); });
-    w = Num::acc_minus_i(w);
-    Num::mac(w, dij, Num::load(cur[nb_ad[2 * nb + nt]]));
-    if (REALJ && jc) {
-        int qq = 0;
-        auto term = [&](int q) {
-            if ((t.jdiag >> q) & 1) return;
-            // JQ: coefficient q of a per-term array (registers); else the
-            // qq-th term with an offset in the per-entry cache
-            Num::mac_real(w, jc[(JQ ? q : qq) * jstride], Num::load(cur[nb_ad[2 * nb + q]]));
-            ++qq;
-        };
-        if constexpr (SH::NB > 0) {
+    typename Num::acc U = Num::acc_zero(), T = Num::acc_zero();
+    auto real_band = [&](int b) {
+        Num::mac_real(T, Num::neg_real(Num::load_re(A[b * d + i])), Num::load(cur[nb_ad[2 * b]]));
+        Num::mac_real(T, Num::load_re(A[b * d + j]), Num::load(cur[nb_ad[2 * b + 1]]));
+    };
+    auto band = [&](int b) {
+        const V ai = Num::load(A[b * d + i]), aj = Num::load(A[b * d + j]);
+        const V x1 = Num::load(cur[nb_ad[2 * b]]), x2 = Num::load(cur[nb_ad[2 * b + 1]]);
+        Num::mac_real(U, Num::im(ai), x1);
+        Num::mac_real(T, Num::neg_real(Num::re(ai)), x1);
+        Num::mac_real(U, Num::im(aj), x2);
+        Num::mac_real(T, Num::re(aj), x2);
+    };
+    if constexpr (SH::NB > 0) {
 #pragma unroll
-            for (int q = 0; q < SH::NT; ++q) term(q);
-        } else {
+        for (int b = 0; b < SH::NBR; ++b) real_band(b);
+#pragma unroll
+        for (int b = SH::NBR; b < SH::NB - 1; ++b) band(b);
+    } else {
+        const int nbo = (t.b0 >= 0) ? t.nb - 1 : t.nb;
 #pragma unroll 1
-            for (int q = 0; q < nt; ++q) term(q);
-        }
-        return Num::raw(w);
+        for (int b = 0; b < t.nbr; ++b) real_band(b);
+#pragma unroll 2
+        for (int b = t.nbr; b < nbo; ++b) band(b);
     }
-    auto jumps = [&](auto rate) {
-        constexpr bool RT = decltype(rate)::value;
-        auto term = [&](int q) {
-            if ((t.jdiag >> q) & 1) return;
-            const int aJ = nb_ad[2 * nb + q];
-            if (REALJ) Num::mac_real(w, jump_real<Num, RT>(t, q, i, j, d, vL, vR, uj), Num::load(cur[aJ]));
-            else Num::mac(w, jump_cplx<Num, RT>(t, q, i, j, d, vL, vR, uj), Num::load(cur[aJ]));
-        };
+    const V x = Num::load(cur[nb_ad[2 * nb + nt]]);
+    Num::mac_real(U, Num::re(dij), x);
+    Num::mac_real(T, Num::im(dij), x);
+    auto each_jump = [&](auto &&term) {
         if constexpr (SH::NB > 0) {
 #pragma unroll
             for (int q = 0; q < SH::NT; ++q) term(q);
@@ -480,9 +451,45 @@ __device__ __forceinline__ typename Num::val lindblad_h_at(const typename Num::s
             for (int q = 0; q < nt; ++q) term(q);
         }
     };
-    if (!REALJ && t.jrate) jumps(std::true_type{});
-    else jumps(std::false_type{});
-    return Num::raw(w);
+    if (REALJ && jc) {
+        int qq = 0;
+        each_jump([&](int q) {
+            if ((t.jdiag >> q) & 1) return;
+            Num::mac_real(U, jc[qq * jstride], Num::load(cur[nb_ad[2 * nb + q]]));
+            ++qq;
+        });
+    } else {
+        auto jumps = [&](auto rate) {
+            constexpr bool RT = decltype(rate)::value;
+            each_jump([&](int q) {
+                if ((t.jdiag >> q) & 1) return;
+                const V xq = Num::load(cur[nb_ad[2 * nb + q]]);
+                if (REALJ) {
+                    Num::mac_real(U, jump_real<Num, RT>(t, q, i, j, d, vL, vR, uj), xq);
+                } else {
+                    const V c = jump_cplx<Num, RT>(t, q, i, j, d, vL, vR, uj);
+                    Num::mac_real(U, Num::re(c), xq);
+                    Num::mac_real(T, Num::im(c), xq);
+                }
+            });
+        };
+        if (!REALJ && t.jrate) jumps(std::true_type{});
+        else jumps(std::false_type{});
+    }
+    return Num::raw(Num::acc_add(U, Num::acc_times_i(T)));
+}
+
+// row and column of packed upper entry u (row i starts at i d - i (i - 1) / 2):
+// a float estimate of the row, corrected in integers.  (In FP64, with 2
+// lanes per cycle and SM, the same formula cost the kernels' set-up about
+// 15 us per use.)
+__device__ __forceinline__ int2 upper_entry(int u, int d) {
+    const float b2 = 2.0f * (float)d + 1.0f;
+    int i = (int)(0.5f * (b2 - sqrtf(fmaxf(b2 * b2 - 8.0f * (float)u, 0.0f))));
+    i = max(0, min(d - 1, i));
+    while (i > 0 && i * d - i * (i - 1) / 2 > u) --i;
+    while (i + 1 < d && (i + 1) * d - (i + 1) * i / 2 <= u) ++i;
+    return make_int2(i, i + (u - (i * d - i * (i - 1) / 2)));
 }
 
 // full-matrix store of upper entry (i, j) and its conjugate mirror
@@ -630,16 +637,14 @@ __device__ __forceinline__ void hpush_async(const uint32_t *rowtab, int rstride,
 // to 2, later waits are skipped and the results are invalid (the host
 // reports GRAPE_ETIMEOUT).  A one-CTA cluster pushes only into itself and
 // needs only the CTA barrier.
-// SH: the band and jump layout (ShapeAny: from the tables); ONE: every
-// thread owns at most one upper entry (cu <= threads), so the entry's
-// neighbour indices stay in registers for the whole launch.
-template <class Num, bool REALJ, class SH, bool ONE>
+// SH: the band and jump layout (ShapeAny: from the tables).
+template <class Num, bool REALJ, class SH>
 __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const PropArgs p) {
     using S = typename Num::store_t;
     using V = typename Num::val;
     using R = typename Num::real_t;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_count, s_err;
+    __shared__ int s_err;
     const int d = p.d, d2 = d * d;
     const int NU = d * (d + 1) / 2;
     const int nbd = p.tab.nb * d;
@@ -680,7 +685,6 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
     const uint32_t mbar_sa = smem_u32(mbar);
 
     if (threadIdx.x == 0) {
-        s_count = 0;
         s_err = 0;
         // per phase: the announcing arrival (expect_tx) and one arrival of
         // every thread after its pushes into the window
@@ -714,13 +718,9 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
     // i d - i (i - 1) / 2), their neighbours' window addresses and, for real
     // jump tables, their jump coefficients (fixed for the whole sweep)
     for (int u = u0 + threadIdx.x; u < u1; u += nth) {
-        const double b2 = 2.0 * d + 1.0;
-        int i = (int)floor(0.5 * (b2 - sqrt(b2 * b2 - 8.0 * (double)u)));
-        i = max(0, min(d - 1, i));
-        while (i > 0 && (long long)i * d - (long long)i * (i - 1) / 2 > u) --i;
-        while (i + 1 < d && (long long)(i + 1) * d - (long long)(i + 1) * i / 2 <= u) ++i;
-        const int j = i + (int)(u - ((long long)i * d - (long long)i * (i - 1) / 2));
-        rc[u - u0] = make_int2(i, j);
+        const int2 e = upper_entry(u, d);
+        const int i = e.x, j = e.y;
+        rc[u - u0] = e;
         short *na = nbad + (size_t)(u - u0) * nstride;
         const int own = ofs[i - wr0] + (j - cs_of(i, hb));
         na[ns] = (short)own;
@@ -744,36 +744,12 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
             }
         }
     }
-    // window slots written by peers each stage (16 B each): slot (r, c) of
-    // the window holds the upper entry (r, c), c >= r, or the mirror of
-    // (c, r); its writer is the owner of that upper entry
-    if (clu) {
-        const int cu = p.cu;
-        int cnt = 0;
-        for (int lr = threadIdx.x; lr < nrows; lr += nth) {
-            const int r = wr0 + lr;
-            for (int c = cs_of(r, hb); c < d; ++c) {
-                const int ur = c >= r ? r * d - r * (r - 1) / 2 + (c - r) : c * d - c * (c - 1) / 2 + (r - c);
-                if (ur / cu != rank) ++cnt;
-            }
-        }
-        if (cnt) atomicAdd(&s_count, cnt);
-    }
     // push targets of the rows this CTA writes: its own rows and, for the
     // mirrors, up to hb rows below
     int rfirst = 0, rlast = -1;
     if (u1 > u0) {
-        // rows of the first and last owned entries (same formula as above)
-        auto row_of = [&](int u) {
-            const double b2 = 2.0 * d + 1.0;
-            int i = (int)floor(0.5 * (b2 - sqrt(b2 * b2 - 8.0 * (double)u)));
-            i = max(0, min(d - 1, i));
-            while (i > 0 && (long long)i * d - (long long)i * (i - 1) / 2 > u) --i;
-            while (i + 1 < d && (long long)(i + 1) * d - (long long)(i + 1) * i / 2 <= u) ++i;
-            return i;
-        };
-        rfirst = row_of(u0);
-        rlast = min(d - 1, row_of(u1 - 1) + hb);
+        rfirst = upper_entry(u0, d).x;
+        rlast = min(d - 1, upper_entry(u1 - 1, d).x + hb);
     }
     const uint32_t buf0_sa = smem_u32(buf0);
     for (int r = rfirst + threadIdx.x; r <= rlast; r += nth) {
@@ -797,7 +773,8 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
         e[0] = (uint32_t)n;
     }
     cluster_sync_all();   // every CTA runs, windows zeroed, mbarriers initialised, tables built
-    const uint32_t expect = (uint32_t)s_count * (uint32_t)sizeof(S);
+    // bytes peers push into this CTA's window each stage
+    const uint32_t expect = (uint32_t)kfl[2 * d + rank] * (uint32_t)sizeof(S);
     const long long limit = 1LL << 31;          // SM cycles a window wait may take
     const uint32_t boff1 = (uint32_t)(wst * (int)sizeof(S));
 
@@ -818,36 +795,7 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
     }
     __syncthreads();
 
-    const bool unit_g = (p.g[1] == 1.0 && p.g[2] == 1.0 && p.g[3] == 1.0);   // forward RK4
-    constexpr int NSC = SH::NB ? 2 * SH::NB + SH::NT + 1 : 1;
-    constexpr int NJQ = SH::NB ? SH::NT : 1;
-    // ONE: the entry's neighbour indices, row and column, base value, RK
-    // accumulator, own-entry coefficient and jump coefficients in registers
-    short nreg[NSC];
-    int2 ijr = make_int2(0, 0);
-    V xr = Num::zero(), ar = Num::zero(), dr = Num::zero();
-    R jreg[NJQ];
-#pragma unroll
-    for (int q = 0; q < NJQ; ++q) jreg[q] = Num::real_const(0.0);
-    if constexpr (ONE) {
-        const bool mine = u0 + (int)threadIdx.x < u1;
-        const short *na0 = nbad + (size_t)threadIdx.x * nstride;
-#pragma unroll
-        for (int k = 0; k < NSC; ++k) nreg[k] = mine ? na0[k] : (short)0;
-        if (mine) {
-            ijr = rc[threadIdx.x];
-            xr = Num::load(xs[threadIdx.x]);
-            if (jcache) {
-                int qq = 0;
-#pragma unroll
-                for (int q = 0; q < NJQ; ++q) {
-                    if ((p.tab.jdiag >> q) & 1) continue;
-                    jreg[q] = jc[qq * p.cu + threadIdx.x];
-                    ++qq;
-                }
-            }
-        }
-    }
+    const bool unit_g = p.unit_g != 0;            // forward RK4
     int tb = 0;
     uint32_t g = 0;                              // stages done in this launch
     bool dfresh = true;                          // D table to (re)build for this slice
@@ -882,41 +830,29 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
 #pragma unroll 1
             for (int u = u0 + threadIdx.x; u < u1; u += nth) {
                 const int li = u - u0;
-                const int2 ij = ONE ? ijr : rc[li];
-                const short *na;
-                if constexpr (ONE) na = nreg;
-                else na = nbad + (size_t)li * nstride;
+                const int2 ij = rc[li];
+                const short *na = nbad + (size_t)li * nstride;
                 if (st) st[u] = cur[na[ns]];     // the stage input itself, packed
                 // own-entry coefficient: cached per slice (the entry is thread-private,
                 // so no barrier is needed) or recomputed when there is no room
                 V dij;
-                if constexpr (ONE) {
-                    if (s == 0 && dfresh) dr = diag_coef<Num, REALJ>(ij.x, ij.y, d, p.tab, A, vL, vR, uj);
-                    dij = dr;
-                } else if (p.fold) {
+                if (p.fold) {
                     if (s == 0 && dfresh) Dt[li] = Num::store(diag_coef<Num, REALJ>(ij.x, ij.y, d, p.tab, A, vL, vR, uj));
                     dij = Num::load(Dt[li]);
                 } else {
                     dij = diag_coef<Num, REALJ>(ij.x, ij.y, d, p.tab, A, vL, vR, uj);
                 }
-                V w;
-                if constexpr (ONE)
-                    w = lindblad_h_at<Num, REALJ, SH, true>(cur, na, ij.x, ij.y, d, p.tab, A, vL, vR, dij, uj,
-                                                            jcache ? jreg : nullptr, 1);
-                else
-                    w = lindblad_h_at<Num, REALJ, SH>(cur, na, ij.x, ij.y, d, p.tab, A, vL, vR, dij, uj,
-                                                      jcache ? jc + li : nullptr, p.cu);
-                const V x = ONE ? xr : Num::load(xs[li]);
-                const V acc = Num::axpy(as_, w, s == 0 ? x : (ONE ? ar : Num::load(as[li])));
+                const V w = lindblad_h_at<Num, REALJ, SH>(cur, na, ij.x, ij.y, d, p.tab, A, vL, vR, dij, uj,
+                                                          jcache ? jc + li : nullptr, p.cu);
+                const V x = Num::load(xs[li]);
+                const V acc = Num::axpy(as_, w, s == 0 ? x : Num::load(as[li]));
                 V z;
                 if (s < 3) {
-                    if constexpr (ONE) ar = acc;
-                    else as[li] = Num::store(acc);
+                    as[li] = Num::store(acc);
                     z = unit_g ? Num::axpy(cb[s + 1], w, x) : Num::lin2(cg[s + 1], x, cb[s + 1], w);
                 } else {
                     const V nx = with_source<Num>(p, n, ij.x, ij.y, acc);
-                    xs[li] = Num::store(nx);         // kept for the boundary and final stores
-                    if constexpr (ONE) xr = nx;
+                    xs[li] = Num::store(nx);
                     z = Num::scale(cg[0], nx);
                 }
                 if (p.defer) {
@@ -976,6 +912,502 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
     }
     for (int u = u0 + threadIdx.x; u < u1; u += nth)
         store_herm<Num>(x_out + soff, d, rc[u - u0].x, rc[u - u0].y, xs[u - u0]);
+}
+
+// ---------------------------------------------------------------------------
+// The Hermitian cluster kernel for the band and jump layouts known at compile
+// time (real jump tables), written for few instructions per entry and stage.
+//
+// What bounds it: at d=120 on 16 CTAs (454 entries per SM) the arithmetic of a
+// stage keeps the FP32 pipe busy for about 0.85 us (two issue cycles per
+// paired instruction), the exchange needs about 0.5 us (0.27 us for the two
+// barriers, 16 B per cycle and SM through distributed shared memory), and
+// everything else is instruction issue: prop_h_kernel spends 555 instructions
+// per entry and stage, 228 of them arithmetic, and 2.44 us.  So
+//  - the two windows lie a compile-time distance apart (WOFF) and the four
+//    stages are unrolled, so a neighbour is one load at a register plus an
+//    immediate;
+//  - every product has a real coefficient: the sums with real and with
+//    imaginary coefficients are kept apart, W = U + i T, so no operand is
+//    swapped or rotated before the end;
+//  - the band coefficients of one index are one 48-byte row (conflict-free
+//    across consecutive indices), three 16-byte loads per side;
+//  - RK coefficients are kernel parameters in the number type, and the entry's
+//    addresses, own-entry and jump coefficients, RK state and push targets are
+//    registers for the whole launch.
+// Measured (GB300, 2070 MHz, against prop_h_kernel with one entry per thread
+// in registers): d=120 on 16 CTAs 2.44 -> 1.69 us per stage, 376 instructions;
+// the d=120 gradient 81.1 -> 60.4 ms; d=20 on one CTA 1.28 -> 0.85 us.  Two
+// lanes per entry, which halves each thread's dependent chain, measured
+// 2.35 us at d=120: it doubles the instructions that are not arithmetic.
+//
+// Ownership, windows, pushes and the two mbarriers are prop_h_kernel's; each
+// warp arrives once (lane 0, after the warp's pushes).  The band rows of the
+// next slice are built at the last stage of a slice and published by the same
+// arrival, so the rebuild needs no barrier; A0 and every A_k stay in shared
+// memory (p.raw) and the slice's controls are fetched at its first stage.
+// WOFF > 0: at most one entry per thread (cu <= threads) and windows within
+// WOFF bytes; WOFF = 0: any tile, with the entries' data in shared memory.
+//
+// Shared memory: buf0, buf1 [maxwin + 1] (buf1 at WOFF when that is set); the
+// band rows [2][d][48 B]; the offset-0 band [2][d]; raw [1 + R][nb][d] when
+// p.raw; and with WOFF = 0 the base values and accumulators [cu] each (16 B),
+// tail coefficients [NTL][cu] (8 B), rc [cu] (int2); the window table; the row
+// push table; with WOFF = 0 the neighbour slots [NA][cu] (i16).
+
+// bounded wait on a window's mbarrier; gives up early once *stop is set
+__device__ __forceinline__ bool mbar_wait_window(uint32_t mbar, uint32_t parity, long long cycles,
+                                                 volatile int *stop) {
+    long long t0 = 0;
+    for (bool first = true;; first = false) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done)
+                     : "r"(mbar), "r"(parity)
+                     : "memory");
+        if (done) return true;
+        if (first) t0 = clock64();
+        else if (*stop || clock64() - t0 > cycles) return false;
+    }
+}
+
+template <class Num> struct RkConst;             // RK coefficients in the number type
+template <> struct RkConst<NumF> {
+    static __device__ __forceinline__ ff g(const PropArgs &p, int s) { return {p.gf[s].x, p.gf[s].y}; }
+    static __device__ __forceinline__ ff a(const PropArgs &p, int s) { return {p.af[s].x, p.af[s].y}; }
+    static __device__ __forceinline__ ff b(const PropArgs &p, int s) { return {p.bf[s].x, p.bf[s].y}; }
+};
+template <> struct RkConst<NumD> {
+    static __device__ __forceinline__ double g(const PropArgs &p, int s) { return p.g[s]; }
+    static __device__ __forceinline__ double a(const PropArgs &p, int s) { return p.a[s]; }
+    static __device__ __forceinline__ double b(const PropArgs &p, int s) { return p.b[s]; }
+};
+
+// two real coefficients in one 16-byte load
+template <class R>
+struct alignas(16) RealPair {
+    R u, t;
+};
+
+template <class Num, class SH, int WOFF>
+__global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const PropArgs p) {
+    using S = typename Num::store_t;
+    using V = typename Num::val;
+    using A = typename Num::acc;
+    using R = typename Num::real_t;
+    using RP = RealPair<R>;
+    using RK = RkConst<Num>;
+    constexpr bool ONE = WOFF > 0;
+    constexpr int NBO = SH::NB - 1, NBR = SH::NBR, NBC = NBO - NBR;
+    constexpr int NTL = 2 + SH::NT;               // D_re, D_im, jumps with an offset
+    constexpr int NA = 2 * NBO + 1 + SH::NT;      // neighbour slots: rows, columns, own entry, jumps
+    constexpr int NRP = NBR / 2 + NBC;            // 16-byte pairs of a band row in use (of 3)
+    static_assert(NBR % 2 == 0 && NRP <= 3, "band row");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint64_t mbar[2];
+    __shared__ int s_err;
+    __shared__ R s_uc[GRAPE_MAXR];                // the next slice's controls
+    const int d = p.d, d2 = d * d;
+    const int NU = d * (d + 1) / 2;
+    const int nbd = SH::NB * d;
+    const int wst = p.maxwin + 1;                 // window stride; slot maxwin is the zero slot
+    const int cu = p.cu;
+    const uint32_t boff1 = ONE ? (uint32_t)WOFF : (uint32_t)(wst * (int)sizeof(S));
+    S *buf0 = reinterpret_cast<S *>(smem_raw);
+    RP *rows = reinterpret_cast<RP *>(smem_raw + boff1 + wst * sizeof(S));   // [2][d][3]
+    S *b0t = reinterpret_cast<S *>(rows + 6 * d); // [2][d]
+    S *raw = b0t + 2 * d;                         // [1 + R][nb][d] when p.raw
+    S *xs = raw + (p.raw ? (1 + p.R) * nbd : 0);  // [cu] when !ONE
+    S *as = xs + (ONE ? 0 : cu);                  // [cu] when !ONE
+    R *tcs = reinterpret_cast<R *>(as + (ONE ? 0 : cu));        // [NTL][cu] when !ONE
+    int2 *rc = reinterpret_cast<int2 *>(tcs + (ONE ? 0 : NTL * cu));
+    int *tab = reinterpret_cast<int *>(rc + (ONE ? 0 : cu));
+    const int rstride = 2 * p.ncl + 1;
+    uint32_t *rowtab = reinterpret_cast<uint32_t *>(tab + p.htab_len);
+    short *nbad = reinterpret_cast<short *>(rowtab + p.rt_rows * rstride);   // [NA][cu] when !ONE
+    const S *x_in = static_cast<const S *>(p.x_in);
+    S *x_out = static_cast<S *>(p.x_out);
+    const int rank = blockIdx.x % p.ncl;
+    const int state = blockIdx.x / p.ncl;
+    const size_t soff = (size_t)state * d2;
+    const int nth = blockDim.x, tid = threadIdx.x;
+    const int lane = tid & 31;
+    const int hb = p.hb;
+    const bool clu = p.ncl > 1;
+    const uint32_t mbar_sa = smem_u32(mbar);
+    const uint32_t buf0_sa = smem_u32(buf0);
+    const S *vL = static_cast<const S *>(p.tab.vLs);
+    const S *vR = static_cast<const S *>(p.tab.vRs);
+    const S *gA0 = static_cast<const S *>(p.tab.A0s);
+    const S *gAk = static_cast<const S *>(p.tab.Aks);
+
+    if (tid == 0) {
+        s_err = 0;
+        // per phase: the announcing arrival (expect_tx) and one per warp
+        mbar_init(mbar_sa, 1u + (uint32_t)(nth >> 5));
+        mbar_init(mbar_sa + 8, 1u + (uint32_t)(nth >> 5));
+        mbar_init_fence();
+    }
+    for (int i = tid; i < p.htab_len; i += nth) tab[i] = __ldg(&p.htab[i]);
+    for (int i = tid; i < wst; i += nth) {
+        buf0[i] = Num::store(Num::zero());
+        *reinterpret_cast<S *>(smem_raw + boff1 + i * sizeof(S)) = Num::store(Num::zero());
+    }
+    if (p.raw) {
+        for (int i = tid; i < nbd; i += nth) raw[i] = gA0[i];
+        for (int i = tid; i < p.R * nbd; i += nth) raw[nbd + i] = gAk[i];
+    }
+    const long long nsub = p.sub_end - p.sub_begin;
+    long long n_first = p.reverse ? p.sub_end - 1 : p.sub_begin;
+    if (nsub <= 0) n_first = p.sub_begin;
+    int jcur = (int)(n_first / p.n_rk);
+    // substeps left in the current slice, this one included
+    const int nin = (int)(n_first % p.n_rk);
+    int left = p.reverse ? nin + 1 : p.n_rk - nin;
+    const int dir = p.reverse ? -1 : 1;
+    if (tid < p.R) s_uc[tid] = Num::real_const(__ldg(&p.u[(size_t)jcur * p.R + tid]));
+    __syncthreads();
+
+    // the band rows of buffer tbw from s_uc: index i's real bands in pairs,
+    // then (im, re) of each complex band
+    auto build = [&](int tbw) {
+        for (int idx = tid; idx < nbd; idx += nth) {
+            V v = Num::load(p.raw ? raw[idx] : gA0[idx]);
+            for (int k = 0; k < p.R; ++k)
+                v = Num::axpy(s_uc[k], Num::load(p.raw ? raw[(k + 1) * nbd + idx] : gAk[(size_t)k * nbd + idx]), v);
+            const int b = idx / d, i = idx - b * d;
+            RP *row = rows + (tbw * d + i) * 3;
+            if (b == NBO) b0t[tbw * d + i] = Num::store(v);
+            else if (b < NBR) reinterpret_cast<R *>(row)[b] = Num::re(v);
+            else row[NBR / 2 + b - NBR] = {Num::im(v), Num::re(v)};
+        }
+    };
+    build(0);
+
+    const int u0 = tab[GRAPE_HTAB_CTA(rank) + 0], u1 = tab[GRAPE_HTAB_CTA(rank) + 1];
+    const int wr0 = tab[GRAPE_HTAB_CTA(rank) + 2];
+    const int *ofs = tab + tab[GRAPE_HTAB_LISTS(p.ncl) + rank];
+    const int *kfl = tab + tab[GRAPE_HTAB_LISTS(p.ncl) + p.ncl];   // kfirst[d], klast[d]
+    const int cnt = u1 - u0;
+    const S *b0cur = b0t - (size_t)p.tab.b0 * d;                  // as diag_coef indexes it
+
+    // neighbour slots of entry (i, j): (i + o_b, j), (i, j + o_b), the entry
+    // itself, the jump terms with an offset
+    auto slots = [&](int i, int j, auto &&put) {
+        const int zs = p.maxwin;
+        const int own = ofs[i - wr0] + (j - cs_of(i, hb));
+        for (int b = 0; b < NBO; ++b) {
+            const int o = p.tab.off[b], r = i + o, c = j + o;
+            put(b, (r >= 0 && r < d) ? ofs[r - wr0] + (j - cs_of(r, hb)) : zs);
+            put(NBO + b, (c >= 0 && c < d) ? own + o : zs);
+        }
+        put(2 * NBO, own);
+        int t = 0;
+        for (int q = 0; q < SH::NT; ++q) {
+            if ((p.tab.jdiag >> q) & 1) continue;
+            const int r = i + p.tab.joL[q], c = j + p.tab.joR[q];
+            put(2 * NBO + 1 + t, (r >= 0 && r < d && c >= 0 && c < d) ? ofs[r - wr0] + (c - cs_of(r, hb)) : zs);
+            ++t;
+        }
+        for (; t < SH::NT; ++t) put(2 * NBO + 1 + t, zs);
+    };
+    const int njt = SH::NT - __popc(p.tab.jdiag);                 // jump terms with an offset
+    auto own_coef = [&](int i, int j, int tbr) {
+        return diag_coef<Num, true>(i, j, d, p.tab, b0cur + tbr * d, vL, vR, nullptr);
+    };
+    auto jump_coefs = [&](int i, int j, auto &&put) {
+        int t = 0;
+        for (int q = 0; q < SH::NT; ++q) {
+            if ((p.tab.jdiag >> q) & 1) continue;
+            put(t, jump_real<Num, false>(p.tab, q, i, j, d, vL, vR, nullptr));
+            ++t;
+        }
+        for (; t < SH::NT; ++t) put(t, Num::real_const(0.0));
+    };
+
+    // push targets per row this CTA writes: count, then (address of (r, 0) in
+    // buf0, mbarrier) per target, the peers first and the CTA itself (mbarrier
+    // 0) last
+    int rfirst = 0, rlast = -1;
+    if (cnt > 0) {
+        rfirst = upper_entry(u0, d).x;
+        rlast = min(d - 1, upper_entry(u1 - 1, d).x + hb);
+    }
+    for (int r = rfirst + tid; r <= rlast; r += nth) {
+        uint32_t *e = rowtab + (r - rfirst) * rstride;
+        const int kf = kfl[r], kl = kfl[d + r];
+        int n = 0;
+        for (int pass = 0; pass < 2; ++pass)
+            for (int k = kf; k <= kl; ++k) {
+                if ((k == rank) != (pass == 1)) continue;
+                const int wk = tab[GRAPE_HTAB_CTA(k) + 2];
+                const int *ofk = tab + tab[GRAPE_HTAB_LISTS(p.ncl) + k];
+                const uint32_t boffs = (uint32_t)((ofk[r - wk] - cs_of(r, hb)) * (int)sizeof(S));
+                e[1 + 2 * n] = (pass ? buf0_sa : map_to_rank(buf0_sa, (uint32_t)k)) + boffs;
+                e[2 + 2 * n] = pass ? 0u : map_to_rank(mbar_sa, (uint32_t)k);
+                ++n;
+            }
+        e[0] = (uint32_t)n;
+    }
+    __syncthreads();                              // band rows and push table
+
+    // ONE: the thread's entry in registers
+    const bool mine = tid < cnt;
+    int2 ij1 = make_int2(0, 0);
+    uint32_t ad[NA];                              // neighbours, byte offsets in a window
+    R tc[NTL];
+    V x1 = Num::zero(), a1 = Num::zero();         // base value, RK accumulator
+    uint32_t pa[2] = {0u, 0u}, pm[2] = {0u, 0u};  // push targets: (i, j) in a peer's buf0, its mbarrier
+    int npeer = 0;
+    if constexpr (ONE) {
+#pragma unroll
+        for (int k = 0; k < NA; ++k) ad[k] = (uint32_t)p.maxwin * (uint32_t)sizeof(S);
+#pragma unroll
+        for (int t = 0; t < NTL; ++t) tc[t] = Num::real_const(0.0);
+        if (mine) {
+            ij1 = upper_entry(u0 + tid, d);
+            // (compile-time indices: the arrays stay in registers)
+            slots(ij1.x, ij1.y, [&](int k, int slot) {
+#pragma unroll
+                for (int q = 0; q < NA; ++q)
+                    if (q == k) ad[q] = (uint32_t)slot * (uint32_t)sizeof(S);
+            });
+            jump_coefs(ij1.x, ij1.y, [&](int t, R c) {
+#pragma unroll
+                for (int q = 0; q < SH::NT; ++q)
+                    if (q == t) tc[2 + q] = c;
+            });
+            const V dij = own_coef(ij1.x, ij1.y, 0);
+            tc[0] = Num::re(dij);
+            tc[1] = Num::im(dij);
+            const uint32_t *e = rowtab + (ij1.x - rfirst) * rstride;
+            npeer = (int)e[0] - 1;
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+                if (t < npeer) {
+                    pa[t] = e[1 + 2 * t] + (uint32_t)ij1.y * (uint32_t)sizeof(S);
+                    pm[t] = e[2 + 2 * t];
+                }
+        }
+    } else {
+        for (int li = tid; li < cnt; li += nth) {
+            const int2 ij = upper_entry(u0 + li, d);
+            rc[li] = ij;
+            slots(ij.x, ij.y, [&](int k, int slot) { nbad[k * cu + li] = (short)slot; });
+            jump_coefs(ij.x, ij.y, [&](int t, R c) { tcs[(2 + t) * cu + li] = c; });
+            const V dij = own_coef(ij.x, ij.y, 0);
+            tcs[li] = Num::re(dij);
+            tcs[cu + li] = Num::im(dij);
+        }
+    }
+    const bool mirror1 = mine && ij1.y > ij1.x && ij1.y - ij1.x <= hb;
+    cluster_sync_all();   // every CTA runs, windows zeroed, mbarriers initialised, tables built
+    // bytes peers push into this CTA's window each stage
+    const uint32_t expect = (uint32_t)kfl[2 * d + rank] * (uint32_t)sizeof(S);
+    const long long limit = 1LL << 31;            // SM cycles a window wait may take
+    bool failed = false;
+
+    // entry (i, j)'s value z to every window holding (i, j) and, near the
+    // diagonal, its mirror, in window `par` (the own window included)
+    auto push_rows = [&](int2 ij, int par, V z) {
+        hpush_async(rowtab, rstride, ij.x - rfirst, ij.y, par ? boff1 : 0u, (uint32_t)par * 8u, Num::store(z));
+        if (ij.y > ij.x && ij.y - ij.x <= hb)
+            hpush_async(rowtab, rstride, ij.y - rfirst, ij.x, par ? boff1 : 0u, (uint32_t)par * 8u,
+                        conj_store<Num>(z));
+    };
+    // every thread's end of a stage whose values went to window `par`
+    auto arrive = [&](int par) {
+        if (clu) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(mbar_sa + 8u * par);
+            cluster_arrive_relaxed();
+        } else {
+            __syncthreads();
+        }
+    };
+
+    // the initial stage input (window 0)
+    if (clu && tid == 0) mbar_expect(mbar_sa, expect);
+    if constexpr (ONE) {
+        if (mine) {
+            x1 = Num::load(x_in[soff + (size_t)ij1.x * d + ij1.y]);
+            push_rows(ij1, 0, Num::scale(RK::g(p, 0), x1));
+        }
+    } else {
+        for (int li = tid; li < cnt; li += nth) {
+            const V x = Num::load(x_in[soff + (size_t)rc[li].x * d + rc[li].y]);
+            xs[li] = Num::store(x);
+            push_rows(rc[li], 0, Num::scale(RK::g(p, 0), x));
+        }
+    }
+    arrive(0);
+
+    const bool unit_g = p.unit_g != 0;            // forward RK4
+    // stage storage of the current substep (this CTA's first entry), per stage
+    // and per substep strides
+    const size_t sset = (size_t)p.n_states * NU;
+    S *st = static_cast<S *>(p.stage_store);
+    if (st) st += ((size_t)(n_first - p.sub_begin) * 4 * p.n_states + state) * NU + u0;
+    const long long sstep = dir * 4 * (long long)sset;
+    // boundary store: at every substep whose index in the sweep's time order
+    // is a multiple of bound_step
+    S *bnd = static_cast<S *>(p.bound_store);
+    long long bcount = 0, bslot = 0;              // substeps to the next one, and its slot
+    if (bnd && p.reverse) {
+        bcount = nsub % p.bound_step;
+        bslot = nsub / p.bound_step;
+    }
+    auto store_bound = [&]() {
+        S *dst = bnd + ((size_t)bslot * p.n_states) * d2 + soff;
+        if constexpr (ONE) {
+            if (mine) store_herm<Num>(dst, d, ij1.x, ij1.y, Num::store(x1));
+        } else {
+            for (int li = tid; li < cnt; li += nth) store_herm<Num>(dst, d, rc[li].x, rc[li].y, xs[li]);
+        }
+        bcount = p.bound_step;
+        bslot += dir;
+    };
+
+    int tb = 0;
+    bool dfresh = false;                          // own coefficients to rebuild for this slice
+    for (long long it = 0; it < nsub; ++it) {
+        if (bnd && bcount == 0) store_bound();
+        const bool newslice = left == 1 && it + 1 < nsub;    // the next substep is in another slice
+        double un = 0.0;
+        if (newslice && tid < p.R) un = __ldg(&p.u[(size_t)(jcur + dir) * p.R + tid]);
+        const RP *rows_t = rows + tb * d * 3;
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            // stage 4 it + s reads window s & 1, whose phase parity is s >> 1
+            const unsigned char *win = smem_raw + ((s & 1) ? boff1 : 0u);
+            const int par = (s & 1) ^ 1;          // next window
+            const uint32_t bo = par ? boff1 : 0u;
+            if (clu) {
+                if (!failed && !mbar_wait_window(mbar_sa + (s & 1) * 8, s >> 1, limit, &s_err)) {
+                    failed = true;
+                    s_err = 1;
+                    atomicExch(&p.gbar[2], 2u);
+                }
+                if (tid == 0 && !failed) mbar_expect(mbar_sa + par * 8, expect);
+                cluster_wait_only();
+            }
+            // one entry's stage: neighbours at at(k), coefficients tail(t), the
+            // base value x and accumulator a; returns the next stage value
+            auto entry = [&](int i, int j, auto &&at, auto &&tail, V &x, V &a, S *dst) -> V {
+                auto val = [&](int k) { return Num::load(*reinterpret_cast<const S *>(win + at(k))); };
+                const RP *ri = rows_t + i * 3, *rj = rows_t + j * 3;
+                A U = Num::acc_zero(), T = Num::acc_zero();          // W = U + i T
+#pragma unroll
+                for (int b = 0; b < NBR; b += 2) {
+                    const RP ci = ri[b / 2], cj = rj[b / 2];
+                    Num::mac_real(T, Num::neg_real(ci.u), val(b));
+                    Num::mac_real(T, cj.u, val(NBO + b));
+                    Num::mac_real(T, Num::neg_real(ci.t), val(b + 1));
+                    Num::mac_real(T, cj.t, val(NBO + b + 1));
+                }
+#pragma unroll
+                for (int b = NBR; b < NBO; ++b) {
+                    const RP ci = ri[NBR / 2 + b - NBR], cj = rj[NBR / 2 + b - NBR];
+                    const V v1 = val(b), v2 = val(NBO + b);
+                    Num::mac_real(U, ci.u, v1);
+                    Num::mac_real(T, Num::neg_real(ci.t), v1);
+                    Num::mac_real(U, cj.u, v2);
+                    Num::mac_real(T, cj.t, v2);
+                }
+                const V own = val(2 * NBO);
+                if (dst) *dst = Num::store(own);                     // the stage input itself, packed
+                Num::mac_real(U, tail(0), own);
+                Num::mac_real(T, tail(1), own);
+#pragma unroll
+                for (int t = 0; t < SH::NT; ++t)
+                    if (t < njt) Num::mac_real(U, tail(2 + t), val(2 * NBO + 1 + t));
+                const V W = Num::raw(Num::acc_add(U, Num::acc_times_i(T)));
+                const V acc = Num::axpy(RK::a(p, s), W, s == 0 ? x : a);
+                if (s < 3) {
+                    a = acc;
+                    return unit_g ? Num::axpy(RK::b(p, (s + 1) & 3), W, x)
+                                  : Num::lin2(RK::g(p, (s + 1) & 3), x, RK::b(p, (s + 1) & 3), W);
+                }
+                x = acc;
+                if (left == 1 && p.src && p.reverse && i == j)       // the running cost's source (App. B)
+                    x = Num::add_real(x, Num::real_once(p.src[i]));
+                return Num::scale(RK::g(p, 0), x);
+            };
+            S *std_ = st ? st + (size_t)p.store_map[s] * sset : nullptr;
+            if constexpr (ONE) {
+                if (mine) {
+                    if (s == 0 && dfresh) {
+                        const V dij = own_coef(ij1.x, ij1.y, tb);
+                        tc[0] = Num::re(dij);
+                        tc[1] = Num::im(dij);
+                    }
+                    const V z = entry(ij1.x, ij1.y, [&](int k) { return ad[k]; }, [&](int t) { return tc[t]; }, x1, a1,
+                                      std_ ? std_ + tid : nullptr);
+                    const S zs = Num::store(z);
+                    *reinterpret_cast<S *>(smem_raw + ad[2 * NBO] + bo) = zs;
+                    if (npeer > 0) st_async16(pa[0] + bo, zs, pm[0] + 8u * par);
+                    if (npeer > 1) st_async16(pa[1] + bo, zs, pm[1] + 8u * par);
+                    if (npeer > 2) {
+                        const uint32_t *e = rowtab + (ij1.x - rfirst) * rstride;
+                        for (int t = 2; t < npeer; ++t)
+                            st_async16(e[1 + 2 * t] + (uint32_t)ij1.y * (uint32_t)sizeof(S) + bo, zs,
+                                       e[2 + 2 * t] + 8u * par);
+                    }
+                    if (mirror1)
+                        hpush_async(rowtab, rstride, ij1.y - rfirst, ij1.x, bo, 8u * par, conj_store<Num>(z));
+                }
+            } else {
+#pragma unroll 1
+                for (int li = tid; li < cnt; li += nth) {
+                    const int2 ij = rc[li];
+                    const short *na = nbad + li;
+                    R *t = tcs + li;
+                    if (s == 0 && dfresh) {
+                        const V dij = own_coef(ij.x, ij.y, tb);
+                        t[0] = Num::re(dij);
+                        t[cu] = Num::im(dij);
+                    }
+                    V x = Num::load(xs[li]), a = s == 0 ? x : Num::load(as[li]);
+                    const V z = entry(ij.x, ij.y, [&](int k) { return (uint32_t)na[k * cu] * (uint32_t)sizeof(S); },
+                                      [&](int q) { return t[q * cu]; }, x, a, std_ ? std_ + li : nullptr);
+                    if (s < 3) as[li] = Num::store(a);
+                    else xs[li] = Num::store(x);
+                    push_rows(ij, par, z);
+                }
+            }
+            if (newslice) {
+                if (s == 2 && tid < p.R) s_uc[tid] = Num::real_once(un);
+                if (s == 3) build(tb ^ 1);
+            }
+            arrive(par);
+        }
+        if (st) st += sstep;
+        if (bnd) --bcount;
+        dfresh = false;
+        if (--left == 0) {
+            left = p.n_rk;
+            jcur += dir;
+            if (newslice) {
+                tb ^= 1;
+                dfresh = !p.dconst;
+            }
+        }
+    }
+    if (clu) {
+        // the last pushes: the matching cluster wait, then every byte peers
+        // pushed into this CTA has landed before it exits
+        cluster_wait_only();
+        if (!failed && !mbar_wait_window(mbar_sa, 0u, limit, &s_err)) atomicExch(&p.gbar[2], 2u);
+    }
+    if (bnd && bcount == 0) store_bound();
+    if constexpr (ONE) {
+        if (mine) store_herm<Num>(x_out + soff, d, ij1.x, ij1.y, Num::store(x1));
+    } else {
+        for (int li = tid; li < cnt; li += nth)
+            store_herm<Num>(x_out + soff, d, rc[li].x, rc[li].y, xs[li]);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1084,13 +1516,9 @@ __global__ void __launch_bounds__(GRAPE_GRID_THREADS, 1) prop_g_kernel(const Pro
     const int wr0 = tab[GRAPE_HTAB_CTA(rank) + 2], nrows = tab[GRAPE_HTAB_CTA(rank) + 3];
     const int *ofs = tab + tab[GRAPE_HTAB_LISTS(nct) + rank];
     for (int u = u0 + threadIdx.x; u < u1; u += nth) {
-        const double b2 = 2.0 * d + 1.0;
-        int i = (int)floor(0.5 * (b2 - sqrt(b2 * b2 - 8.0 * (double)u)));
-        i = max(0, min(d - 1, i));
-        while (i > 0 && (long long)i * d - (long long)i * (i - 1) / 2 > u) --i;
-        while (i + 1 < d && (long long)(i + 1) * d - (long long)(i + 1) * i / 2 <= u) ++i;
-        const int j = i + (int)(u - ((long long)i * d - (long long)i * (i - 1) / 2));
-        rc[u - u0] = make_int2(i, j);
+        const int2 e = upper_entry(u, d);
+        const int i = e.x, j = e.y;
+        rc[u - u0] = e;
         short *na = nbad + (size_t)(u - u0) * nstride;
         const int own = ofs[i - wr0] + (j - cs_of(i, hb));
         na[ns] = (short)own;
@@ -1166,7 +1594,7 @@ __global__ void __launch_bounds__(GRAPE_GRID_THREADS, 1) prop_g_kernel(const Pro
         __syncthreads();
     };
 
-    const bool unit_g = (p.g[1] == 1.0 && p.g[2] == 1.0 && p.g[3] == 1.0);
+    const bool unit_g = p.unit_g != 0;
     unsigned round = 1;                          // push rounds finished by this CTA
     bool dfresh = true;
     for (long long it = 0; it < nsub; ++it) {
@@ -1871,17 +2299,26 @@ __global__ void __launch_bounds__(256) to_double_kernel(const void *src_v, doubl
 // ------------------------------------------------------------------ launchers
 // `variant`: bit 0 the jump tables are real; bit 1 Hermitian (upper-triangle)
 // kernel; bits 2-3 the band/jump shape (0 from the tables, 1 ShapeT, 2 ShapeR;
-// only with real jump tables); bit 4 one entry per thread (with a shape).
+// only with real jump tables); bit 5 prop_s_kernel (with a shape), bit 4 its
+// build for one entry per thread, bit 6 with the windows GRAPE_WOFF_SMALL apart.
 using PropKernel = void (*)(const PropArgs);
 
 template <class Num>
 PropKernel prop_kernel_for(int variant) {
     const bool realj = (variant & 1) != 0, herm = (variant & 2) != 0, one = (variant & 16) != 0;
+    const bool small = (variant & 64) != 0;
     const int shape = (variant >> 2) & 3;
     if (!herm) return realj ? prop_kernel<Num, true> : prop_kernel<Num, false>;
-    if (realj && shape == 1) return one ? prop_h_kernel<Num, true, ShapeT, true> : prop_h_kernel<Num, true, ShapeT, false>;
-    if (realj && shape == 2) return one ? prop_h_kernel<Num, true, ShapeR, true> : prop_h_kernel<Num, true, ShapeR, false>;
-    return realj ? prop_h_kernel<Num, true, ShapeAny, false> : prop_h_kernel<Num, false, ShapeAny, false>;
+    if (variant & 32) {
+        if (shape == 1)
+            return !one ? prop_s_kernel<Num, ShapeT, 0>
+                        : small ? prop_s_kernel<Num, ShapeT, GRAPE_WOFF_SMALL> : prop_s_kernel<Num, ShapeT, GRAPE_WOFF>;
+        return !one ? prop_s_kernel<Num, ShapeR, 0>
+                    : small ? prop_s_kernel<Num, ShapeR, GRAPE_WOFF_SMALL> : prop_s_kernel<Num, ShapeR, GRAPE_WOFF>;
+    }
+    if (realj && shape == 1) return prop_h_kernel<Num, true, ShapeT>;
+    if (realj && shape == 2) return prop_h_kernel<Num, true, ShapeR>;
+    return realj ? prop_h_kernel<Num, true, ShapeAny> : prop_h_kernel<Num, false, ShapeAny>;
 }
 
 template <class Num>

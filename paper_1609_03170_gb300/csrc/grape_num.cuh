@@ -114,6 +114,7 @@ struct NumD {
     static __device__ __forceinline__ val zero() { return {0.0, 0.0}; }
     static __device__ __forceinline__ acc acc_zero() { return {0.0, 0.0}; }
     static __device__ __forceinline__ real_t real_const(double x) { return x; }
+    static __device__ __forceinline__ real_t real_once(double x) { return x; }
     // acc += a * b
     static __device__ __forceinline__ void mac(acc &c, val a, val b) {
         c.re = fma(a.re, b.re, fma(-a.im, b.im, c.re));
@@ -132,6 +133,7 @@ struct NumD {
     static __device__ __forceinline__ val done(acc c) { return {c.re, c.im}; }
     static __device__ __forceinline__ val raw(acc c) { return {c.re, c.im}; }
     static __device__ __forceinline__ acc acc_minus_i(acc c) { return {c.im, -c.re}; }
+    static __device__ __forceinline__ acc acc_times_i(acc c) { return {-c.im, c.re}; }
     static __device__ __forceinline__ acc acc_add(acc a, acc b) { return {a.re + b.re, a.im + b.im}; }
     // a - conj(b), a + b, a + c (c real)
     static __device__ __forceinline__ val sub_conj(val a, val b) { return {a.re - b.re, a.im + b.im}; }
@@ -256,6 +258,20 @@ struct NumF {
     static __device__ __forceinline__ val zero() { return {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
     static __device__ __forceinline__ acc acc_zero() { return {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
     static __device__ __forceinline__ real_t real_const(double x) { return ff_from_double(x); }
+    // the same where it stands: the compiler may neither hoist it out of its
+    // branch nor repeat it (at 2 lanes per cycle and SM, an FP64 conversion
+    // that every warp runs every substep costs more than the stage's loads)
+    static __device__ __forceinline__ real_t real_once(double x) {
+        ff r;
+        asm volatile("{\n\t.reg .f64 t;\n\t"
+                     "cvt.rn.f32.f64 %0, %2;\n\t"
+                     "cvt.f64.f32 t, %0;\n\t"
+                     "sub.rn.f64 t, %2, t;\n\t"
+                     "cvt.rn.f32.f64 %1, t;\n\t}"
+                     : "=&f"(r.h), "=f"(r.l)
+                     : "d"(x));
+        return r;
+    }
     // acc += a b: re += a.re b.re - a.im b.im, im += a.re b.im + a.im b.re
     // (per lane, in that order)
     static __device__ __forceinline__ void mac(acc &c, val a, val b) {
@@ -284,6 +300,9 @@ struct NumF {
     static __device__ __forceinline__ val raw(acc c) { return {c.h, c.l}; }
     static __device__ __forceinline__ acc acc_minus_i(acc c) {
         return {make_float2(c.h.y, -c.h.x), make_float2(c.l.y, -c.l.x)};
+    }
+    static __device__ __forceinline__ acc acc_times_i(acc c) {
+        return {make_float2(-c.h.y, c.h.x), make_float2(-c.l.y, c.l.x)};
     }
     // a + b of two accumulators: the high parts with TwoSum, every error in
     // the low part (still unnormalised)
