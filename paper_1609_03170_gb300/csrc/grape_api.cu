@@ -141,21 +141,42 @@ bool hermitian(const Bands &A, int d) {
     return max_abs(D) <= 1e-12 * std::max(1.0, max_abs(A));
 }
 
+// The operators of one set of tables: H_eff = A0 + sum_k u_k Ak, the trace's
+// control bands Tk and the jump operators sqrt(gamma) c (jctl: control that
+// scales the dissipator, -1 fixed).
+struct Ops {
+    Bands A0;
+    std::vector<Bands> Ak, Tk, J;
+    std::vector<int> jctl;
+};
+
+// Tables of one direction for every operator set (one set shared by all
+// states, or one per state; the sets have the same offsets).
 struct HostDir {
     std::vector<int> off;        // nb
     int nbr = 0;                 // leading bands that are real for every control value
-    std::vector<cplx> A0, Ak;    // [nb][d], [R][nb][d]
+    std::vector<cplx> A0, Ak;    // [sets][nb][d], [sets][R][nb][d]
     std::vector<int> oL, oR;     // nt
-    std::vector<cplx> vL, vR;    // [nt][d]
+    std::vector<cplx> vL, vR;    // [sets][nt][d]
     std::vector<int> jctl;       // nt: control scaling the term, -1 fixed
 };
 
-HostDir make_dir(const Bands &A0, const std::vector<Bands> &Ak,
-                 const std::vector<Bands> &jumps, const std::vector<int> &jump_ctl, int d) {
+// The dual's operators: A' = -H_eff^+, A'_k = -A_k^+, jumps sqrt(gamma) c^+.
+Ops dual_ops(const Ops &f, int d) {
+    Ops a;
+    a.A0 = scaled(adjoint(f.A0, d), -1.0, d);
+    for (const Bands &B : f.Ak) a.Ak.push_back(scaled(adjoint(B, d), -1.0, d));
+    for (const Bands &B : f.J) a.J.push_back(adjoint(B, d));
+    a.jctl = f.jctl;
+    return a;
+}
+
+HostDir make_dir(const std::vector<Ops> &sets, int d) {
     HostDir h;
+    const Ops &first = sets[0];
     std::map<int, int> idx;
-    for (const auto &kv : A0) idx[kv.first] = 0;
-    for (const auto &B : Ak)
+    for (const auto &kv : first.A0) idx[kv.first] = 0;
+    for (const auto &B : first.Ak)
         for (const auto &kv : B) idx[kv.first] = 0;
     // bands whose values are real for every control value (A0 and every Ak
     // real there) come first: the kernels multiply them as real numbers.
@@ -169,9 +190,11 @@ HostDir make_dir(const Bands &A0, const std::vector<Bands> &Ak,
                 if (c.imag() != 0.0) return false;
             return true;
         };
-        if (!is_real(A0, o)) return false;
-        for (const auto &B : Ak)
-            if (!is_real(B, o)) return false;
+        for (const Ops &set : sets) {
+            if (!is_real(set.A0, o)) return false;
+            for (const auto &B : set.Ak)
+                if (!is_real(B, o)) return false;
+        }
         return true;
     };
     for (int pass = 0; pass < 2; ++pass)
@@ -185,25 +208,195 @@ HostDir make_dir(const Bands &A0, const std::vector<Bands> &Ak,
         idx[0] = (int)h.off.size();
         h.off.push_back(0);
     }
-    const int nb = (int)h.off.size(), R = (int)Ak.size();
-    h.A0.assign((size_t)nb * d, cplx());
-    h.Ak.assign((size_t)R * nb * d, cplx());
-    for (const auto &kv : A0)
-        for (int i = 0; i < d; ++i) h.A0[(size_t)idx[kv.first] * d + i] = kv.second[i];
-    for (int k = 0; k < R; ++k)
-        for (const auto &kv : Ak[k])
-            for (int i = 0; i < d; ++i)
-                h.Ak[((size_t)k * nb + idx[kv.first]) * d + i] = kv.second[i];
-    for (size_t m = 0; m < jumps.size(); ++m)
-        for (const auto &a : jumps[m])
-            for (const auto &b : jumps[m]) {
-                h.oL.push_back(a.first);
-                h.oR.push_back(b.first);
-                h.vL.insert(h.vL.end(), a.second.begin(), a.second.end());
-                h.vR.insert(h.vR.end(), b.second.begin(), b.second.end());
-                h.jctl.push_back(jump_ctl[m]);
-            }
+    const size_t nb = h.off.size(), R = first.Ak.size(), nbd = nb * d;
+    h.A0.assign(sets.size() * nbd, cplx());
+    h.Ak.assign(sets.size() * R * nbd, cplx());
+    for (size_t s = 0; s < sets.size(); ++s) {
+        const Ops &set = sets[s];
+        for (const auto &kv : set.A0)
+            for (int i = 0; i < d; ++i) h.A0[s * nbd + (size_t)idx[kv.first] * d + i] = kv.second[i];
+        for (size_t k = 0; k < R; ++k)
+            for (const auto &kv : set.Ak[k])
+                for (int i = 0; i < d; ++i)
+                    h.Ak[(s * R + k) * nbd + (size_t)idx[kv.first] * d + i] = kv.second[i];
+        for (size_t m = 0; m < set.J.size(); ++m)
+            for (const auto &a : set.J[m])
+                for (const auto &b : set.J[m]) {
+                    h.vL.insert(h.vL.end(), a.second.begin(), a.second.end());
+                    h.vR.insert(h.vR.end(), b.second.begin(), b.second.end());
+                    if (s) continue;
+                    h.oL.push_back(a.first);
+                    h.oR.push_back(b.first);
+                    h.jctl.push_back(set.jctl[m]);
+                }
+    }
     return h;
+}
+
+// ------------------------------------------------------- invariant subspaces
+// A state whose density matrix is zero outside the index set I x I stays
+// zero there for the whole pulse when no operator of the Lindbladian (H_eff,
+// every control, every jump operator) leads from an index of I to one
+// outside: a resonator drive, for instance, keeps the transmon's level, so
+// |q><q| (x) |alpha><alpha| stays in the N x N block of level q.  Every term
+// the kernels would add for the other entries is an exact zero, the dual on
+// I x I reads only I x I, and the traces of Eq. (dphidu) pair Y with K on
+// I x I alone.  The problem then runs on the entries of I x I with the
+// operators restricted to I.
+
+// indices reachable from the rows and columns where x (d x d) is not zero
+std::vector<int> invariant_set(const Ops &ops, const cplx *x, int d) {
+    std::vector<char> in(d, 0);
+    std::vector<int> todo;
+    auto add = [&](int i) {
+        if (!in[i]) {
+            in[i] = 1;
+            todo.push_back(i);
+        }
+    };
+    for (int i = 0; i < d && (int)todo.size() < d; ++i)
+        for (int j = 0; j < d; ++j)
+            if (x[(size_t)i * d + j] != cplx()) {
+                add(i);
+                add(j);
+            }
+    std::vector<const Bands *> all{&ops.A0};
+    for (const Bands &B : ops.Ak) all.push_back(&B);
+    for (const Bands &B : ops.J) all.push_back(&B);
+    while (!todo.empty()) {
+        const int j = todo.back();
+        todo.pop_back();
+        for (const Bands *B : all)
+            for (const auto &kv : *B) {
+                const int i = j - kv.first;          // Op[i][j], j = i + offset
+                if (i >= 0 && i < d && kv.second[i] != cplx()) add(i);
+            }
+    }
+    std::vector<int> I;
+    for (int i = 0; i < d; ++i)
+        if (in[i]) I.push_back(i);
+    return I;
+}
+
+// the operator on the indices I (ascending), renumbered 0, 1, ...
+Bands restricted(const Bands &A, const std::vector<int> &I, int d) {
+    std::vector<int> pos(d, -1);
+    const int m = (int)I.size();
+    for (int p = 0; p < m; ++p) pos[I[p]] = p;
+    Bands R;
+    for (const auto &kv : A)
+        for (int p = 0; p < m; ++p) {
+            const int j = I[p] + kv.first;
+            if (j < 0 || j >= d || pos[j] < 0 || kv.second[I[p]] == cplx()) continue;
+            auto &v = R[pos[j] - p];
+            v.resize(m);
+            v[p] += kv.second[I[p]];
+        }
+    return R;
+}
+
+Ops restricted(const Ops &ops, const std::vector<int> &I, int d) {
+    Ops r;
+    r.A0 = restricted(ops.A0, I, d);
+    for (const Bands &B : ops.Ak) r.Ak.push_back(restricted(B, I, d));
+    for (const Bands &B : ops.Tk) r.Tk.push_back(restricted(B, I, d));
+    for (const Bands &B : ops.J) r.J.push_back(restricted(B, I, d));
+    r.jctl = ops.jctl;
+    return r;
+}
+
+// What a problem's tables and buffers are made from: the operator sets (one,
+// or one per state), the states and the Hermitian part of the targets.
+struct ProblemData {
+    int d = 0, ns = 0;
+    std::vector<Ops> sets;
+    std::vector<cplx> rho0, sigma;               // [ns][d][d]
+};
+
+size_t band_count(const Ops &o) {
+    std::map<int, int> offs;
+    for (const auto &kv : o.A0) offs[kv.first] = 1;
+    for (const auto &B : o.Ak)
+        for (const auto &kv : B) offs[kv.first] = 1;
+    return offs.size();
+}
+size_t jump_pairs(const Ops &o) {
+    size_t n = 0;
+    for (const auto &B : o.J) n += B.size() * B.size();
+    return n;
+}
+size_t trace_bands(const Ops &o) {
+    size_t n = 0;
+    for (const auto &B : o.Tk) n += B.size();
+    return n;
+}
+
+// The problem on its states' invariant subspaces, idx[s] = the indices of
+// state s.  False when it would not be smaller: the states' sets are of
+// different sizes and their union is everything, or the restricted operators
+// have more bands or band pairs than the full ones (an irregular set breaks
+// bands up, and each band costs every entry a multiply-add).
+bool restrict_problem(const ProblemData &full, ProblemData *out, std::vector<std::vector<int>> *idx) {
+    const int d = full.d;
+    const size_t d2 = (size_t)d * d;
+    const Ops &ops = full.sets[0];
+    std::vector<std::vector<int>> I(full.ns);
+    bool same_size = true;
+    for (int s = 0; s < full.ns; ++s) {
+        I[s] = invariant_set(ops, &full.rho0[s * d2], d);
+        if ((int)I[s].size() == d) return false;
+        if (I[s].empty()) I[s].push_back(0);     // rho = 0: any index set will do
+        same_size = same_size && I[s].size() == I[0].size();
+    }
+    if (!same_size) {
+        // one size for all states: every state on the union of the sets
+        std::vector<int> u;
+        for (int i = 0; i < d; ++i)
+            for (int s = 0; s < full.ns; ++s)
+                if (std::binary_search(I[s].begin(), I[s].end(), i)) {
+                    u.push_back(i);
+                    break;
+                }
+        for (auto &v : I) v = u;
+    }
+    const int m = (int)I[0].size();
+    if (m >= d) return false;
+    bool shared = true;
+    for (int s = 1; s < full.ns; ++s) shared = shared && I[s] == I[0];
+    std::vector<Ops> sets;
+    for (int s = 0; s < (shared ? 1 : full.ns); ++s) sets.push_back(restricted(ops, I[s], d));
+    // the same offsets in every set (zero bands where a state has none)
+    auto unite = [&](auto &&get) {
+        std::map<int, int> offs;
+        for (Ops &o : sets)
+            for (const auto &kv : get(o)) offs[kv.first] = 1;
+        for (Ops &o : sets)
+            for (const auto &kv : offs) get(o)[kv.first].resize(m);
+    };
+    unite([](Ops &o) -> Bands & { return o.A0; });
+    for (size_t k = 0; k < ops.Ak.size(); ++k) {
+        unite([k](Ops &o) -> Bands & { return o.Ak[k]; });
+        unite([k](Ops &o) -> Bands & { return o.Tk[k]; });
+    }
+    for (size_t q = 0; q < ops.J.size(); ++q) unite([q](Ops &o) -> Bands & { return o.J[q]; });
+    if (band_count(sets[0]) > band_count(ops) || jump_pairs(sets[0]) > jump_pairs(ops) ||
+        trace_bands(sets[0]) > trace_bands(ops))
+        return false;
+    out->d = m;
+    out->ns = full.ns;
+    out->sets = std::move(sets);
+    const size_t m2 = (size_t)m * m;
+    out->rho0.assign(m2 * full.ns, cplx());
+    out->sigma.assign(m2 * full.ns, cplx());
+    for (int s = 0; s < full.ns; ++s)
+        for (int a = 0; a < m; ++a)
+            for (int b = 0; b < m; ++b) {
+                const size_t f = s * d2 + (size_t)I[s][a] * d + I[s][b], r = s * m2 + (size_t)a * m + b;
+                out->rho0[r] = full.rho0[f];
+                out->sigma[r] = full.sigma[f];
+            }
+    *idx = std::move(I);
+    return true;
 }
 
 // Where a caller's pointer lives, for a call on device `dev`: *on_dev is set
@@ -371,6 +564,12 @@ struct grape_problem {
         d_Y = d_K = d_ckpt = nullptr;
         seg = nseg = 0;
     }
+    // the problem on its states' invariant subspaces, null when they are the
+    // whole space; the calls then run on it, and this problem keeps only the
+    // full size's geometry and what rho(T) needs
+    grape_problem *sub = nullptr;
+    std::vector<std::vector<int>> sub_idx;   // its states' indices
+    int *d_imap = nullptr;                   // [ns][d]: an index's place in its state's set, -1 outside
     std::vector<void *> allocs;
     void *alloc(size_t n) {
         void *p = nullptr;
@@ -384,6 +583,7 @@ struct grape_problem {
         return p;
     }
     ~grape_problem() {
+        delete sub;
         for (auto &e : ev)
             if (e) cudaEventDestroy(e);
         for (auto &e : evF)
@@ -404,6 +604,9 @@ struct grape_problem {
 
 namespace {
 
+// the problem a call runs on
+grape_problem *active(grape_problem *P) { return P && P->sub ? P->sub : P; }
+
 template <typename T>
 grape_status upload(grape_problem *P, const std::vector<T> &h, T **out) {
     *out = static_cast<T *>(P->alloc(h.size() * sizeof(T)));
@@ -419,7 +622,9 @@ grape_status upload(grape_problem *P, const std::vector<T> &h, T **out) {
 
 double2 encode(const grape_problem *P, cplx v);
 
-grape_status upload_dir(grape_problem *P, const HostDir &h, PropTables *t) {
+// counts, offsets and (unless counts_only) the device tables of one
+// direction, `sets` operator sets
+grape_status upload_dir(grape_problem *P, const HostDir &h, PropTables *t, int sets, bool counts_only) {
     const int d = P->d;
     if ((int)h.off.size() > GRAPE_MAXB)
         return fail(GRAPE_EINVAL, "too many distinct Hamiltonian bands (max 12)");
@@ -443,6 +648,12 @@ grape_status upload_dir(grape_problem *P, const HostDir &h, PropTables *t) {
         if (h.oL[q] == 0 && h.oR[q] == 0) t->jdiag |= 1 << q;
         t->jctl[q] = h.jctl[q];
         if (h.jctl[q] >= 0) t->jrate |= 1 << q;
+    }
+    if (counts_only) return GRAPE_OK;
+    if (sets > 1) {
+        t->a0_stride = (long long)t->nb * d;
+        t->ak_stride = (long long)P->R * t->nb * d;
+        t->v_stride = (long long)t->nt * d;
     }
     auto cvt = [](const std::vector<cplx> &v) {
         std::vector<double2> o(v.size());
@@ -498,6 +709,13 @@ cudaError_t k_to_double(const grape_problem *P, const void *src, double2 *dst, s
                         cudaStream_t s) {
     return P->prec == GRAPE_PREC_FP64 ? grape_launch_to_double_f64(src, dst, n, s)
                                       : grape_launch_to_double_df(src, dst, n, s);
+}
+
+// rho(T) of the subspace problem A as P's full matrices
+cudaError_t k_expand(const grape_problem *P, const grape_problem *A, double2 *dst, cudaStream_t s) {
+    return A->prec == GRAPE_PREC_FP64
+               ? grape_launch_expand_f64(A->d_x, dst, P->d_imap, A->d, P->d, P->ns, s)
+               : grape_launch_expand_df(A->d_x, dst, P->d_imap, A->d, P->d, P->ns, s);
 }
 
 // complex128 -> one 16-byte storage entry
@@ -900,7 +1118,8 @@ std::vector<int> neighbour_table(const std::vector<int> &tab, int d, int nct, in
 
 // Grid kernel: nct CTAs per state, one per SM (all resident), the
 // Hermitian kernel's ownership and window tables over nct CTAs.
-grape_status choose_geometry_grid(grape_problem *P) {
+// (geometry_only: no tables and buffers).
+grape_status choose_geometry_grid(grape_problem *P, bool geometry_only) {
     int max_smem = 0, sms = 0;
     GRAPE_CUDA_TRY(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, P->device));
     GRAPE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device));
@@ -957,11 +1176,13 @@ grape_status choose_geometry_grid(grape_problem *P) {
     int stride = 0;
     const std::vector<int> ntab = neighbour_table(tab, d, nct, hb, &stride);
     grape_status st;
-    if ((st = upload(P, tab, &P->d_htab)) != GRAPE_OK) return st;
-    if ((st = upload(P, ntab, &P->d_ntab)) != GRAPE_OK) return st;
-    P->d_gbuf = static_cast<double2 *>(P->alloc((size_t)2 * P->ns * P->d2 * sizeof(double2)));
-    P->d_gflag = static_cast<unsigned *>(P->alloc((size_t)nct * P->ns * sizeof(unsigned)));
-    if (!P->d_gbuf || !P->d_gflag) return fail(GRAPE_ENOMEM, "cudaMalloc failed for the grid kernel buffers");
+    if (!geometry_only) {
+        if ((st = upload(P, tab, &P->d_htab)) != GRAPE_OK) return st;
+        if ((st = upload(P, ntab, &P->d_ntab)) != GRAPE_OK) return st;
+        P->d_gbuf = static_cast<double2 *>(P->alloc((size_t)2 * P->ns * P->d2 * sizeof(double2)));
+        P->d_gflag = static_cast<unsigned *>(P->alloc((size_t)nct * P->ns * sizeof(unsigned)));
+        if (!P->d_gbuf || !P->d_gflag) return fail(GRAPE_ENOMEM, "cudaMalloc failed for the grid kernel buffers");
+    }
     if (const char *env = std::getenv("GRAPE_SPIN_LIMIT")) P->spin_limit = std::atoll(env);
     P->grid = true;
     P->variant = variant;
@@ -1593,6 +1814,222 @@ grape_status run_gradient(grape_problem *P, const double *ud, double *Fd, double
     return GRAPE_OK;
 }
 
+namespace {
+
+// Tables, geometry and buffers of a problem (geometry_only: no more than its
+// geometry and the staging buffer of rho(T)).
+grape_status build_problem(const grape_problem_desc *desc, const ProblemData &data, bool geometry_only,
+                           grape_problem **out) {
+    grape_status st;
+    const int d = data.d, ns = data.ns, nsets = (int)data.sets.size();
+    const size_t d2 = (size_t)d * d;
+    const std::vector<int> &jcf = data.sets[0].jctl;
+    std::vector<Ops> dual;
+    for (const Ops &o : data.sets) dual.push_back(dual_ops(o, d));
+    const HostDir hf = make_dir(data.sets, d);
+    const HostDir ha = make_dir(dual, d);
+    // control bands for the trace kernel
+    TraceArgs tr;
+    std::memset(&tr, 0, sizeof(tr));
+    std::vector<double2> cbv, stv_l, stv_r;
+    {
+        std::map<int, int> doidx;
+        for (int k = 0; k < desc->n_controls; ++k)
+            for (const auto &kv : data.sets[0].Tk[k]) {
+                if (tr.ncb >= GRAPE_MAXCB) return fail(GRAPE_EINVAL, "too many control bands (max 8)");
+                auto it = doidx.find(kv.first);
+                if (it == doidx.end()) {
+                    if ((int)doidx.size() >= GRAPE_MAXDO) return fail(GRAPE_EINVAL, "too many control band offsets");
+                    const int id = (int)doidx.size();
+                    doidx[kv.first] = id;
+                    tr.do_off[id] = kv.first;
+                    it = doidx.find(kv.first);
+                }
+                tr.cb_k[tr.ncb] = k;
+                tr.cb_do[tr.ncb] = it->second;
+                tr.ncb++;
+            }
+        for (const Ops &o : data.sets)
+            for (const Bands &B : o.Tk)
+                for (const auto &kv : B)
+                    for (const cplx &c : kv.second) cbv.push_back(make_double2(c.real(), c.imag()));
+        tr.ndo = (int)doidx.size();
+        tr.d = d;
+        tr.R = desc->n_controls;
+        // sandwich terms gamma c y c^+ of the rate-controlled dissipators: the
+        // forward jump terms (sqrt(gamma) c on both sides) of those dissipators
+        for (size_t q = 0; q < hf.oL.size(); ++q) {
+            if (hf.jctl[q] < 0) continue;
+            if (tr.nst >= GRAPE_MAXST)
+                return fail(GRAPE_EINVAL, "too many band pairs in rate-controlled dissipators (max 4)");
+            tr.st_k[tr.nst] = hf.jctl[q];
+            tr.st_oL[tr.nst] = hf.oL[q];
+            tr.st_oR[tr.nst] = hf.oR[q];
+            tr.nst++;
+        }
+        for (int s = 0; s < nsets; ++s)
+            for (size_t q = 0; q < hf.oL.size(); ++q) {
+                if (hf.jctl[q] < 0) continue;
+                const size_t at = (s * hf.oL.size() + q) * d;
+                for (int i = 0; i < d; ++i) {
+                    stv_l.push_back(make_double2(hf.vL[at + i].real(), hf.vL[at + i].imag()));
+                    stv_r.push_back(make_double2(hf.vR[at + i].real(), hf.vR[at + i].imag()));
+                }
+            }
+        if (nsets > 1) {
+            tr.cb_stride = (long long)tr.ncb * d;
+            tr.st_stride = (long long)tr.nst * d;
+        }
+    }
+
+    grape_problem *P = new grape_problem();
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        delete P;
+        return fail(GRAPE_ECUDA, "no CUDA device");
+    }
+    P->device = dev;
+    static_scratch_setup(dev);   // grape_gradient_static's array, committed once per device
+    P->d = d;
+    P->d2 = d2;
+    P->R = desc->n_controls;
+    P->J = desc->n_jumps;
+    P->ns = ns;
+    P->n_slices = desc->n_slices;
+    P->n_rk = desc->n_rk;
+    P->T = desc->T;
+    P->mode = desc->grad_mode;
+    P->ckpt_stride = desc->ckpt_stride;
+    P->prec = desc->precision;
+    auto bail = [&](grape_status s) { delete P; return s; };
+    {
+        // real jump tables select the kernels with one real coefficient per
+        // term; rate-controlled terms always take the complex-table kernels,
+        // which alone carry the per-slice scaling
+        bool real_jumps = true;
+        for (const HostDir *h : {&hf, &ha})
+            for (const auto *v : {&h->vL, &h->vR})
+                for (const cplx &c : *v) real_jumps = real_jumps && c.imag() == 0.0;
+        for (int c : jcf) real_jumps = real_jumps && c < 0;
+        P->variant = real_jumps ? 1 : 0;
+    }
+    // error word of the bounded waits (grid barrier arrivals, generation, flag)
+    P->d_gbar = static_cast<unsigned *>(P->alloc(4 * sizeof(unsigned)));
+    if (!P->d_gbar) return bail(fail(GRAPE_ENOMEM, "cudaMalloc failed for the error word"));
+    if (cudaMemset(P->d_gbar, 0, 4 * sizeof(unsigned)) != cudaSuccess ||
+        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {   // before non-blocking streams use it
+        cudaGetLastError();
+        return bail(fail(GRAPE_ECUDA, "cudaMemset of the error word failed"));
+    }
+    if ((st = upload_dir(P, hf, &P->tab[0], nsets, geometry_only)) != GRAPE_OK) return bail(st);
+    if ((st = upload_dir(P, ha, &P->tab[1], nsets, geometry_only)) != GRAPE_OK) return bail(st);
+    int omax = 0;
+    for (int dir = 0; dir < 2; ++dir) {
+        const HostDir &h = dir ? ha : hf;
+        for (int o : h.off) omax = std::max(omax, std::abs(o));
+        for (size_t q = 0; q < h.oL.size(); ++q)
+            omax = std::max(omax, std::max(std::abs(h.oL[q]), std::abs(h.oR[q])));
+    }
+    int hb = omax;   // lower entries the stencil reads: within max(omax, oL - oR) of the diagonal
+    for (int dir = 0; dir < 2; ++dir) {
+        const HostDir &h = dir ? ha : hf;
+        for (size_t q = 0; q < h.oL.size(); ++q) hb = std::max(hb, h.oL[q] - h.oR[q]);
+    }
+    // kernel choice: Hermitian cluster kernel, else full-matrix cluster kernel,
+    // else the grid kernel (GRAPE_KERNEL=grid|cluster|full forces one)
+    std::string kern = "auto";
+    if (const char *env = std::getenv("GRAPE_KERNEL")) kern = env;
+    bool herm = kern == "auto" || kern == "cluster";
+    if (const char *env = std::getenv("GRAPE_HERMITIAN")) herm = herm && std::atoi(env) != 0;
+    bool placed = false;
+    P->omax = omax;
+    P->hb_h = hb;
+    P->dconst = 1;
+    for (const Ops &o : data.sets)
+        for (const Bands &B : o.Ak) P->dconst = P->dconst && !B.count(0);
+    if (kern != "grid" && herm) {
+        st = choose_geometry_h(P);
+        if (st != GRAPE_OK && st != GRAPE_EINVAL) return bail(st);
+        placed = (st == GRAPE_OK);
+    }
+    if (kern != "grid" && !placed) {
+        st = choose_geometry(P);
+        if (st != GRAPE_OK && st != GRAPE_EINVAL) return bail(st);
+        placed = (st == GRAPE_OK);
+    }
+    if (!placed && (st = choose_geometry_grid(P, geometry_only)) != GRAPE_OK) return bail(st);
+    P->trace = tr;
+    trace_layout(P, &P->trace);
+    P->d_out = static_cast<double2 *>(P->alloc(d2 * P->ns * sizeof(double2)));
+    if (!P->d_out) return bail(fail(GRAPE_ENOMEM, "cudaMalloc failed"));
+    if (geometry_only) {
+        *out = P;
+        return GRAPE_OK;
+    }
+    {
+        std::vector<double2> r(data.rho0.size()), g2(data.sigma.size());
+        for (size_t i = 0; i < r.size(); ++i) r[i] = encode(P, data.rho0[i]);
+        for (size_t i = 0; i < g2.size(); ++i) g2[i] = encode(P, data.sigma[i]);
+        if ((st = upload(P, r, &P->d_rho0)) != GRAPE_OK) return bail(st);
+        if ((st = upload(P, g2, &P->d_sigma)) != GRAPE_OK) return bail(st);
+    }
+    // the kernels read the tables in their storage format (no conversion
+    // from FP64 in the double-float build)
+    auto to_store = [&](const std::vector<double2> &v) {
+        std::vector<double2> o(v.size());
+        for (size_t i = 0; i < v.size(); ++i) o[i] = encode(P, cplx(v[i].x, v[i].y));
+        return o;
+    };
+    double2 *cbs = nullptr;
+    if ((st = upload(P, to_store(cbv), &cbs)) != GRAPE_OK) return bail(st);
+    P->trace.cb_s = cbs;
+    if (tr.nst > 0) {
+        double2 *as = nullptr, *bs = nullptr;
+        if ((st = upload(P, to_store(stv_l), &as)) != GRAPE_OK) return bail(st);
+        if ((st = upload(P, to_store(stv_r), &bs)) != GRAPE_OK) return bail(st);
+        P->trace.st_vLs = as;
+        P->trace.st_vRs = bs;
+    }
+    if ((st = trace_tiles(P, &P->trace)) != GRAPE_OK) return bail(st);
+
+    P->d_x = static_cast<double2 *>(P->alloc(d2 * P->ns * sizeof(double2)));
+    P->d_mu = static_cast<double2 *>(P->alloc(d2 * P->ns * sizeof(double2)));
+    P->d_part = static_cast<double *>(
+        P->alloc((size_t)P->n_slices * P->trace.nsplit * std::max(P->R, 1) * sizeof(double)));
+    P->d_u = static_cast<double *>(P->alloc((size_t)P->n_slices * std::max(P->R, 1) * sizeof(double)));
+    P->d_F = static_cast<double *>(P->alloc(sizeof(double)));
+    P->d_G = static_cast<double *>(P->alloc((size_t)P->n_slices * std::max(P->R, 1) * sizeof(double)));
+    if (!P->d_x || !P->d_mu || !P->d_part || !P->d_u || !P->d_F || !P->d_G) return bail(fail(GRAPE_ENOMEM, "cudaMalloc failed"));
+    {
+        int prio_low = 0, prio_high = 0;
+        cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high);
+        if (cudaStreamCreateWithPriority(&P->s1, cudaStreamNonBlocking, prio_high) != cudaSuccess ||
+            cudaStreamCreateWithPriority(&P->s2, cudaStreamNonBlocking, prio_low) != cudaSuccess ||
+            cudaStreamCreateWithPriority(&P->s3, cudaStreamNonBlocking, prio_high) != cudaSuccess ||
+            cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+            cudaEventCreateWithFlags(&P->ev_fork3, cudaEventDisableTiming) != cudaSuccess ||
+            cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming) != cudaSuccess) {
+            cudaGetLastError();
+            return bail(fail(GRAPE_ECUDA, "cudaStreamCreate failed"));
+        }
+    }
+    for (auto &e : P->ev)
+        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+            cudaGetLastError();
+            return bail(fail(GRAPE_ECUDA, "cudaEventCreate failed"));
+        }
+    for (auto &e : P->evF)
+        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+            cudaGetLastError();
+            return bail(fail(GRAPE_ECUDA, "cudaEventCreate failed"));
+        }
+    *out = P;
+    return GRAPE_OK;
+}
+
+}  // namespace
+
 extern "C" {
 
 const char *grape_last_error(void) { return g_last_error.c_str(); }
@@ -1656,42 +2093,39 @@ grape_status grape_problem_create(const grape_problem_desc *desc, grape_problem_
         }
     // Forward: A = H_eff = H0 - i/2 sum gamma c^+ c (+ sum u_k A_k), terms from sqrt(gamma) c.
     // A rate control k contributes A_k = -i/2 gamma c^+ c and scales its terms by u_k.
-    Bands A0 = H0;
-    std::vector<Bands> Ak = Hc;                 // propagation's control parts
-    std::vector<Bands> Tk = Hc;                 // trace's control bands (see below)
-    std::vector<Bands> Jf, Ja;
-    std::vector<int> jcf;
+    Ops ops;
+    ops.A0 = H0;
+    ops.Ak = Hc;                                // propagation's control parts
+    ops.Tk = Hc;                                // trace's control bands (see below)
     for (int m = 0; m < desc->n_jumps; ++m) {
         const double g = desc->rates[m];
         if (g == 0.0 || C[m].empty()) continue;
         const Bands cdc = product(adjoint(C[m], d), C[m], d);
         if (jc[m] < 0) {
-            add_into(A0, cdc, cplx(0.0, -0.5 * g), d);
+            add_into(ops.A0, cdc, cplx(0.0, -0.5 * g), d);
         } else {
-            add_into(Ak[jc[m]], cdc, cplx(0.0, -0.5 * g), d);
+            add_into(ops.Ak[jc[m]], cdc, cplx(0.0, -0.5 * g), d);
             // -1/2 gamma {c^+c, y} enters Re Tr(kb dL/du y) as the commutator
             // term of the trace kernel does with the band values +i/2 gamma c^+c
-            add_into(Tk[jc[m]], cdc, cplx(0.0, 0.5 * g), d);
+            add_into(ops.Tk[jc[m]], cdc, cplx(0.0, 0.5 * g), d);
         }
-        Jf.push_back(scaled(C[m], std::sqrt(g), d));
-        Ja.push_back(scaled(adjoint(C[m], d), std::sqrt(g), d));
-        jcf.push_back(jc[m]);
+        ops.J.push_back(scaled(C[m], std::sqrt(g), d));
+        prune(ops.J.back());
+        ops.jctl.push_back(jc[m]);
     }
-    prune(A0);
-    for (auto &b : Ak) prune(b);
-    for (auto &b : Tk) prune(b);
-    // Dual: A' = -H_eff^+, A'_k = -A_k^+, terms from sqrt(gamma) c^+.
-    Bands A0d = scaled(adjoint(A0, d), -1.0, d);
-    std::vector<Bands> Hcd(Ak.size());
-    for (size_t k = 0; k < Ak.size(); ++k) Hcd[k] = scaled(adjoint(Ak[k], d), -1.0, d);
-    for (auto &c : Jf) prune(c);
-    for (auto &c : Ja) prune(c);
-    const HostDir hf = make_dir(A0, Ak, Jf, jcf, d);
-    const HostDir ha = make_dir(A0d, Hcd, Ja, jcf, d);
+    prune(ops.A0);
+    for (auto &b : ops.Ak) prune(b);
+    for (auto &b : ops.Tk) prune(b);
 
     // initial states (Hermitian) and the Hermitian part of sigma
     const size_t d2 = (size_t)d * d;
-    std::vector<cplx> rho0(d2 * desc->n_states), sig(d2 * desc->n_states);
+    ProblemData full;
+    full.d = d;
+    full.ns = desc->n_states;
+    full.sets.push_back(std::move(ops));
+    std::vector<cplx> &rho0 = full.rho0, &sig = full.sigma;
+    rho0.resize(d2 * desc->n_states);
+    sig.resize(d2 * desc->n_states);
     for (int s = 0; s < desc->n_states; ++s) {
         const double *r = desc->rho0 + 2 * d2 * s;
         double mx = 0.0, asym = 0.0;
@@ -1718,184 +2152,22 @@ grape_status grape_problem_create(const grape_problem_desc *desc, grape_problem_
             }
     }
 
-    // control bands for the trace kernel
-    TraceArgs tr;
-    std::memset(&tr, 0, sizeof(tr));
-    std::vector<double2> cbv, stv_l, stv_r;
-    {
-        std::map<int, int> doidx;
-        for (int k = 0; k < desc->n_controls; ++k)
-            for (const auto &kv : Tk[k]) {
-                if (tr.ncb >= GRAPE_MAXCB) return fail(GRAPE_EINVAL, "too many control bands (max 8)");
-                auto it = doidx.find(kv.first);
-                if (it == doidx.end()) {
-                    if ((int)doidx.size() >= GRAPE_MAXDO) return fail(GRAPE_EINVAL, "too many control band offsets");
-                    const int id = (int)doidx.size();
-                    doidx[kv.first] = id;
-                    tr.do_off[id] = kv.first;
-                    it = doidx.find(kv.first);
-                }
-                tr.cb_k[tr.ncb] = k;
-                tr.cb_do[tr.ncb] = it->second;
-                for (int i = 0; i < d; ++i) cbv.push_back(make_double2(kv.second[i].real(), kv.second[i].imag()));
-                tr.ncb++;
-            }
-        tr.ndo = (int)doidx.size();
-        tr.d = d;
-        tr.R = desc->n_controls;
-        // sandwich terms gamma c y c^+ of the rate-controlled dissipators: the
-        // forward jump terms (sqrt(gamma) c on both sides) of those dissipators
-        for (size_t q = 0; q < hf.oL.size(); ++q) {
-            if (hf.jctl[q] < 0) continue;
-            if (tr.nst >= GRAPE_MAXST)
-                return fail(GRAPE_EINVAL, "too many band pairs in rate-controlled dissipators (max 4)");
-            tr.st_k[tr.nst] = hf.jctl[q];
-            tr.st_oL[tr.nst] = hf.oL[q];
-            tr.st_oR[tr.nst] = hf.oR[q];
-            for (int i = 0; i < d; ++i) {
-                stv_l.push_back(make_double2(hf.vL[q * d + i].real(), hf.vL[q * d + i].imag()));
-                stv_r.push_back(make_double2(hf.vR[q * d + i].real(), hf.vR[q * d + i].imag()));
-            }
-            tr.nst++;
-        }
+    // states that never leave a part of the space: the problem on that part
+    // does the work, and the full-size one keeps its geometry
+    ProblemData part;
+    std::vector<std::vector<int>> idx;
+    const bool reduced = restrict_problem(full, &part, &idx);
+    grape_problem *P = nullptr;
+    if ((st = build_problem(desc, full, reduced, &P)) != GRAPE_OK) return st;
+    if (reduced) {
+        auto bail = [&](grape_status e) { delete P; return e; };
+        if ((st = build_problem(desc, part, false, &P->sub)) != GRAPE_OK) return bail(st);
+        std::vector<int> map((size_t)P->ns * d, -1);
+        for (int s = 0; s < P->ns; ++s)
+            for (size_t a = 0; a < idx[s].size(); ++a) map[(size_t)s * d + idx[s][a]] = (int)a;
+        if ((st = upload(P, map, &P->d_imap)) != GRAPE_OK) return bail(st);
+        P->sub_idx = std::move(idx);
     }
-
-    grape_problem *P = new grape_problem();
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) {
-        cudaGetLastError();
-        delete P;
-        return fail(GRAPE_ECUDA, "no CUDA device");
-    }
-    P->device = dev;
-    static_scratch_setup(dev);   // grape_gradient_static's array, committed once per device
-    P->d = d;
-    P->d2 = d2;
-    P->R = desc->n_controls;
-    P->J = desc->n_jumps;
-    P->ns = desc->n_states;
-    P->n_slices = desc->n_slices;
-    P->n_rk = desc->n_rk;
-    P->T = desc->T;
-    P->mode = desc->grad_mode;
-    P->ckpt_stride = desc->ckpt_stride;
-    P->prec = desc->precision;
-    auto bail = [&](grape_status s) { delete P; return s; };
-    {
-        // real jump tables select the kernels with one real coefficient per
-        // term; rate-controlled terms always take the complex-table kernels,
-        // which alone carry the per-slice scaling
-        bool real_jumps = true;
-        for (const HostDir *h : {&hf, &ha})
-            for (const auto *v : {&h->vL, &h->vR})
-                for (const cplx &c : *v) real_jumps = real_jumps && c.imag() == 0.0;
-        for (int c : jcf) real_jumps = real_jumps && c < 0;
-        P->variant = real_jumps ? 1 : 0;
-    }
-    // error word of the bounded waits (grid barrier arrivals, generation, flag)
-    P->d_gbar = static_cast<unsigned *>(P->alloc(4 * sizeof(unsigned)));
-    if (!P->d_gbar) return bail(fail(GRAPE_ENOMEM, "cudaMalloc failed for the error word"));
-    if (cudaMemset(P->d_gbar, 0, 4 * sizeof(unsigned)) != cudaSuccess ||
-        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {   // before non-blocking streams use it
-        cudaGetLastError();
-        return bail(fail(GRAPE_ECUDA, "cudaMemset of the error word failed"));
-    }
-    if ((st = upload_dir(P, hf, &P->tab[0])) != GRAPE_OK) return bail(st);
-    if ((st = upload_dir(P, ha, &P->tab[1])) != GRAPE_OK) return bail(st);
-    int omax = 0;
-    for (int dir = 0; dir < 2; ++dir) {
-        const HostDir &h = dir ? ha : hf;
-        for (int o : h.off) omax = std::max(omax, std::abs(o));
-        for (size_t q = 0; q < h.oL.size(); ++q)
-            omax = std::max(omax, std::max(std::abs(h.oL[q]), std::abs(h.oR[q])));
-    }
-    int hb = omax;   // lower entries the stencil reads: within max(omax, oL - oR) of the diagonal
-    for (int dir = 0; dir < 2; ++dir) {
-        const HostDir &h = dir ? ha : hf;
-        for (size_t q = 0; q < h.oL.size(); ++q) hb = std::max(hb, h.oL[q] - h.oR[q]);
-    }
-    // kernel choice: Hermitian cluster kernel, else full-matrix cluster kernel,
-    // else the grid kernel (GRAPE_KERNEL=grid|cluster|full forces one)
-    std::string kern = "auto";
-    if (const char *env = std::getenv("GRAPE_KERNEL")) kern = env;
-    bool herm = kern == "auto" || kern == "cluster";
-    if (const char *env = std::getenv("GRAPE_HERMITIAN")) herm = herm && std::atoi(env) != 0;
-    bool placed = false;
-    P->omax = omax;
-    P->hb_h = hb;
-    P->dconst = 1;
-    for (const Bands &B : Ak) P->dconst = P->dconst && !B.count(0);
-    if (kern != "grid" && herm) {
-        st = choose_geometry_h(P);
-        if (st != GRAPE_OK && st != GRAPE_EINVAL) return bail(st);
-        placed = (st == GRAPE_OK);
-    }
-    if (kern != "grid" && !placed) {
-        st = choose_geometry(P);
-        if (st != GRAPE_OK && st != GRAPE_EINVAL) return bail(st);
-        placed = (st == GRAPE_OK);
-    }
-    if (!placed && (st = choose_geometry_grid(P)) != GRAPE_OK) return bail(st);
-    {
-        std::vector<double2> r(rho0.size()), g2(sig.size());
-        for (size_t i = 0; i < r.size(); ++i) r[i] = encode(P, rho0[i]);
-        for (size_t i = 0; i < g2.size(); ++i) g2[i] = encode(P, sig[i]);
-        if ((st = upload(P, r, &P->d_rho0)) != GRAPE_OK) return bail(st);
-        if ((st = upload(P, g2, &P->d_sigma)) != GRAPE_OK) return bail(st);
-    }
-    // the kernels read the tables in their storage format (no conversion
-    // from FP64 in the double-float build)
-    auto to_store = [&](const std::vector<double2> &v) {
-        std::vector<double2> o(v.size());
-        for (size_t i = 0; i < v.size(); ++i) o[i] = encode(P, cplx(v[i].x, v[i].y));
-        return o;
-    };
-    double2 *cbs = nullptr;
-    if ((st = upload(P, to_store(cbv), &cbs)) != GRAPE_OK) return bail(st);
-    tr.cb_s = cbs;
-    if (tr.nst > 0) {
-        double2 *as = nullptr, *bs = nullptr;
-        if ((st = upload(P, to_store(stv_l), &as)) != GRAPE_OK) return bail(st);
-        if ((st = upload(P, to_store(stv_r), &bs)) != GRAPE_OK) return bail(st);
-        tr.st_vLs = as;
-        tr.st_vRs = bs;
-    }
-    P->trace = tr;
-    trace_layout(P, &P->trace);
-    if ((st = trace_tiles(P, &P->trace)) != GRAPE_OK) return bail(st);
-
-    P->d_x = static_cast<double2 *>(P->alloc(d2 * P->ns * sizeof(double2)));
-    P->d_mu = static_cast<double2 *>(P->alloc(d2 * P->ns * sizeof(double2)));
-    P->d_out = static_cast<double2 *>(P->alloc(d2 * P->ns * sizeof(double2)));
-    P->d_part = static_cast<double *>(
-        P->alloc((size_t)P->n_slices * P->trace.nsplit * std::max(P->R, 1) * sizeof(double)));
-    P->d_u = static_cast<double *>(P->alloc((size_t)P->n_slices * std::max(P->R, 1) * sizeof(double)));
-    P->d_F = static_cast<double *>(P->alloc(sizeof(double)));
-    P->d_G = static_cast<double *>(P->alloc((size_t)P->n_slices * std::max(P->R, 1) * sizeof(double)));
-    if (!P->d_x || !P->d_mu || !P->d_out || !P->d_part || !P->d_u || !P->d_F || !P->d_G) return bail(fail(GRAPE_ENOMEM, "cudaMalloc failed"));
-    {
-        int prio_low = 0, prio_high = 0;
-        cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high);
-        if (cudaStreamCreateWithPriority(&P->s1, cudaStreamNonBlocking, prio_high) != cudaSuccess ||
-            cudaStreamCreateWithPriority(&P->s2, cudaStreamNonBlocking, prio_low) != cudaSuccess ||
-            cudaStreamCreateWithPriority(&P->s3, cudaStreamNonBlocking, prio_high) != cudaSuccess ||
-            cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&P->ev_fork3, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming) != cudaSuccess) {
-            cudaGetLastError();
-            return bail(fail(GRAPE_ECUDA, "cudaStreamCreate failed"));
-        }
-    }
-    for (auto &e : P->ev)
-        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
-            cudaGetLastError();
-            return bail(fail(GRAPE_ECUDA, "cudaEventCreate failed"));
-        }
-    for (auto &e : P->evF)
-        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
-            cudaGetLastError();
-            return bail(fail(GRAPE_ECUDA, "cudaEventCreate failed"));
-        }
     *out = P;
     return GRAPE_OK;
 }
@@ -1909,7 +2181,7 @@ grape_status grape_problem_destroy(grape_problem_t P) {
 
 grape_status grape_problem_memory(grape_problem_t P, size_t *bytes) {
     if (!P || !bytes) return fail(GRAPE_EINVAL, "NULL argument");
-    *bytes = P->bytes;
+    *bytes = P->bytes + (P->sub ? P->sub->bytes : 0);
     return GRAPE_OK;
 }
 
@@ -1925,30 +2197,37 @@ grape_status grape_problem_geometry(grape_problem_t P, int32_t *cluster, int32_t
 grape_status grape_problem_set_penalty(grape_problem_t P, const double *diag, double beta) {
     if (!P) return fail(GRAPE_EINVAL, "NULL problem");
     if (!std::isfinite(beta)) return fail(GRAPE_EINVAL, "penalty weight must be finite");
+    grape_problem *A = active(P);
     if (!diag || beta == 0.0) {
-        P->penalty = false;
-        P->pen_beta = 0.0;
+        A->penalty = false;
+        A->pen_beta = 0.0;
         return GRAPE_OK;
     }
     for (int i = 0; i < P->d; ++i)
         if (!std::isfinite(diag[i])) return fail(GRAPE_EINVAL, "penalty operator entries must be finite");
     DeviceGuard g(P->device);
     const double dt = P->T / P->n_slices;
-    std::vector<double> a(diag, diag + P->d), src(P->d);
-    for (int i = 0; i < P->d; ++i) src[i] = -beta * dt * a[i];
-    if (!P->d_pdiag) {
-        P->d_pdiag = static_cast<double *>(P->alloc(P->d * sizeof(double)));
-        P->d_src = static_cast<double *>(P->alloc(P->d * sizeof(double)));
-        P->d_pen = static_cast<double *>(P->alloc((size_t)(P->n_slices + 1) * sizeof(double)));
-        if (!P->d_pdiag || !P->d_src || !P->d_pen) return fail(GRAPE_ENOMEM, "cudaMalloc failed for the penalty");
+    const size_t n = (size_t)A->ns * A->d;                // one row per state
+    std::vector<double> a(n), src(n);
+    for (int s = 0; s < A->ns; ++s)
+        for (int i = 0; i < A->d; ++i) {
+            const size_t e = (size_t)s * A->d + i;
+            a[e] = diag[P->sub ? P->sub_idx[s][i] : i];
+            src[e] = -beta * dt * a[e];
+        }
+    if (!A->d_pdiag) {
+        A->d_pdiag = static_cast<double *>(A->alloc(n * sizeof(double)));
+        A->d_src = static_cast<double *>(A->alloc(n * sizeof(double)));
+        A->d_pen = static_cast<double *>(A->alloc((size_t)(P->n_slices + 1) * sizeof(double)));
+        if (!A->d_pdiag || !A->d_src || !A->d_pen) return fail(GRAPE_ENOMEM, "cudaMalloc failed for the penalty");
     }
     // callers' kernels may still read the old values: order after the device
     GRAPE_CUDA_TRY(cudaDeviceSynchronize());
-    GRAPE_CUDA_TRY(cudaMemcpy(P->d_pdiag, a.data(), P->d * sizeof(double), cudaMemcpyHostToDevice));
-    GRAPE_CUDA_TRY(cudaMemcpy(P->d_src, src.data(), P->d * sizeof(double), cudaMemcpyHostToDevice));
+    GRAPE_CUDA_TRY(cudaMemcpy(A->d_pdiag, a.data(), n * sizeof(double), cudaMemcpyHostToDevice));
+    GRAPE_CUDA_TRY(cudaMemcpy(A->d_src, src.data(), n * sizeof(double), cudaMemcpyHostToDevice));
     GRAPE_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
-    P->pen_beta = beta;
-    P->penalty = true;
+    A->pen_beta = beta;
+    A->penalty = true;
     return GRAPE_OK;
 }
 
@@ -1960,11 +2239,20 @@ grape_status grape_problem_set_tile(grape_problem_t P, int32_t cluster, int32_t 
         return fail(GRAPE_EINVAL, "threads per CTA must be a multiple of 32 in [64, 512]");
     if (P->grid) return fail(GRAPE_EINVAL, "the grid kernel has no tile to set");
     DeviceGuard g(P->device);
-    return (P->variant & 2) ? plan_h(P, cluster, threads) : plan_full(P, cluster, threads);
+    const grape_status st = (P->variant & 2) ? plan_h(P, cluster, threads) : plan_full(P, cluster, threads);
+    // the subspace problem takes the tile too where it can (no more CTAs per
+    // state than the caller allowed); else it keeps its own
+    grape_problem *A = P->sub;
+    if (st == GRAPE_OK && A && !A->grid) {
+        const grape_status sa = (A->variant & 2) ? plan_h(A, cluster, threads) : plan_full(A, cluster, threads);
+        if (sa != GRAPE_OK && sa != GRAPE_EINVAL) return sa;
+    }
+    return st;
 }
 
 grape_status grape_problem_status(grape_problem_t P) {
     if (!P) return fail(GRAPE_EINVAL, "NULL problem");
+    P = active(P);
     DeviceGuard g(P->device);
     unsigned flag[3] = {0, 0, 0};
     GRAPE_CUDA_TRY(cudaDeviceSynchronize());
@@ -1987,12 +2275,13 @@ grape_status grape_problem_kernel(grape_problem_t P, int32_t *kind) {
 
 grape_status grape_set_profiling(grape_problem_t P, int32_t on) {
     if (!P) return fail(GRAPE_EINVAL, "NULL problem");
-    P->profiling = (on != 0);
+    active(P)->profiling = (on != 0);
     return GRAPE_OK;
 }
 
 grape_status grape_phase_times(grape_problem_t P, double ms[4], int32_t launches[4]) {
     if (!P || !ms || !launches) return fail(GRAPE_EINVAL, "NULL argument");
+    P = active(P);
     DeviceGuard g(P->device);
     for (int i = 0; i < 4; ++i) { ms[i] = 0.0; launches[i] = 0; }
     grape_status st = GRAPE_OK;
@@ -2013,12 +2302,14 @@ grape_status grape_phase_times(grape_problem_t P, double ms[4], int32_t launches
 
 int32_t grape_gradient_launches(grape_problem_t P) {
     if (!P) return -1;
+    P = active(P);
     return gradient_launch_count(P, P->seg, P->nseg, concurrent_sweeps(P, P->nseg));
 }
 
-grape_status grape_forward(grape_problem_t P, const double *u, double *F, double *rhoT,
+grape_status grape_forward(grape_problem_t problem, const double *u, double *F, double *rhoT,
                            void *stream) {
-    if (!P || !F) return fail(GRAPE_EINVAL, "NULL problem or F");
+    if (!problem || !F) return fail(GRAPE_EINVAL, "NULL problem or F");
+    grape_problem *P = active(problem);
     DeviceGuard g(P->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const double *ud;
@@ -2062,10 +2353,11 @@ grape_status grape_forward(grape_problem_t P, const double *u, double *F, double
     if (P->penalty && (st = pen_finish(P, f_dev ? F : P->d_F, s)) != GRAPE_OK) return st;
     bool sync = false;
     if (rhoT) {
-        const size_t n = P->d2 * P->ns;
-        GRAPE_CUDA_TRY(k_to_double(P, P->d_x, r_dev ? reinterpret_cast<double2 *>(rhoT) : P->d_out, n, s));
+        const size_t n = problem->d2 * P->ns;
+        double2 *out = r_dev ? reinterpret_cast<double2 *>(rhoT) : problem->d_out;
+        GRAPE_CUDA_TRY(problem->sub ? k_expand(problem, P, out, s) : k_to_double(P, P->d_x, out, n, s));
         if (!r_dev) {
-            GRAPE_CUDA_TRY(cudaMemcpyAsync(rhoT, P->d_out, n * sizeof(double2), cudaMemcpyDeviceToHost, s));
+            GRAPE_CUDA_TRY(cudaMemcpyAsync(rhoT, out, n * sizeof(double2), cudaMemcpyDeviceToHost, s));
             sync = true;
         }
     }
@@ -2174,6 +2466,7 @@ grape_status grape_gradient_filtered(grape_problem_t P, int32_t n_steps, const d
 grape_status grape_gradient(grape_problem_t P, const double *u, double *F, double *grad,
                             void *stream) {
     if (!P || !F || (!grad && P->R > 0)) return fail(GRAPE_EINVAL, "NULL problem, F or grad");
+    P = active(P);
     DeviceGuard g(P->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     grape_status st;
@@ -2264,6 +2557,37 @@ StaticScratch g_static[kMaxDevices];
 
 size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
 
+// The longest checkpoint segment whose scratch fits the static array (0:
+// none), the least bytes any length needs, and the parts' sizes at `seg`.
+struct StaticPlan {
+    long long seg = 0;
+    size_t least = SIZE_MAX, mat = 0, per_seg = 0, part = 0;
+};
+StaticPlan static_plan(const grape_problem *P) {
+    StaticPlan r;
+    const int nsplit = std::max(1, P->trace.nsplit);
+    r.mat = align256(P->d2 * P->ns * sizeof(double2));
+    auto per_seg = [&](long long sg) { return align256(stage_bytes(P, sg)); };
+    auto part_bytes = [&](long long sg) {
+        return nsplit > 1 ? align256((size_t)sg * nsplit * std::max(P->R, 1) * sizeof(double)) : 0;
+    };
+    // the longest segment that fits (fewest launches); the need is not
+    // monotonic in the length (stage storage grows, checkpoints shrink), so
+    // every length is tried
+    for (long long sg = P->n_slices; sg >= 1; --sg) {
+        const long long ns = (P->n_slices + sg - 1) / sg;
+        const size_t nb = 2 * r.mat + 2 * per_seg(sg) + part_bytes(sg) + (ns > 1 ? (size_t)(ns + 1) * r.mat : 0);
+        r.least = std::min(r.least, nb);
+        if (nb <= kStaticScratchBytes) {
+            r.seg = sg;
+            r.per_seg = per_seg(sg);
+            r.part = part_bytes(sg);
+            break;
+        }
+    }
+    return r;
+}
+
 }  // namespace
 
 // with device `dev` current
@@ -2290,6 +2614,8 @@ grape_status grape_gradient_static(grape_problem_t P, const double *u, double *F
     if ((st = require_device_ptr(u, P->device, "u")) != GRAPE_OK) return st;
     if ((st = require_device_ptr(F, P->device, "F")) != GRAPE_OK) return st;
     if (P->R > 0 && (st = require_device_ptr(grad, P->device, "grad")) != GRAPE_OK) return st;
+    grape_problem *const whole = P;
+    P = active(P);
     if (P->penalty)
         return fail(GRAPE_EINVAL, "grape_gradient_static does not evaluate the running-cost penalty");
     static_scratch_setup(P->device);   // done by grape_problem_create; a no-op here
@@ -2300,39 +2626,25 @@ grape_status grape_gradient_static(grape_problem_t P, const double *u, double *F
 
     // scratch plan: propagated state, adjoint state, stage storage of one
     // segment (forward and adjoint), the segment's partial traces and, with
-    // several segments, the checkpoints
+    // several segments, the checkpoints.  What the call accepts is decided by
+    // the problem's full size; the plan is that of the problem it runs on
     const bool exact = (P->mode == GRAPE_GRAD_EXACT);
-    const int nsplit = std::max(1, P->trace.nsplit);
-    const size_t mat = align256(P->d2 * P->ns * sizeof(double2));
-    auto per_seg = [&](long long sg) { return align256(stage_bytes(P, sg)); };
-    auto part_bytes = [&](long long sg) {
-        return nsplit > 1 ? align256((size_t)sg * nsplit * std::max(P->R, 1) * sizeof(double)) : 0;
-    };
-    auto need = [&](long long sg) {
-        const long long ns = (P->n_slices + sg - 1) / sg;
-        return 2 * mat + 2 * per_seg(sg) + part_bytes(sg) + (ns > 1 ? (size_t)(ns + 1) * mat : 0);
-    };
-    // the longest segment that fits (fewest launches); the need is not
-    // monotonic in the length (stage storage grows, checkpoints shrink), so
-    // every length is tried
-    long long seg = 0;
-    size_t least = SIZE_MAX;
-    for (long long sg = P->n_slices; sg >= 1; --sg) {
-        const size_t nb = need(sg);
-        least = std::min(least, nb);
-        if (nb <= kStaticScratchBytes) { seg = sg; break; }
-    }
-    if (seg == 0)
-        return fail(GRAPE_EINVAL, "problem needs at least " + std::to_string(least) +
+    StaticPlan plan = static_plan(whole);
+    if (plan.seg > 0 && P != whole) plan = static_plan(P);
+    if (plan.seg == 0)
+        return fail(GRAPE_EINVAL, "problem needs at least " + std::to_string(plan.least) +
                                       " bytes of scratch with every checkpoint segment length; "
                                       "the static scratch holds " + std::to_string(kStaticScratchBytes));
+    const long long seg = plan.seg;
+    const int nsplit = std::max(1, P->trace.nsplit);
+    const size_t mat = plan.mat, per = plan.per_seg, partb = plan.part;
     const int nseg = (int)((P->n_slices + seg - 1) / seg);
     double2 *x = reinterpret_cast<double2 *>(base);
     double2 *mu = reinterpret_cast<double2 *>(base + mat);
     double2 *Y = reinterpret_cast<double2 *>(base + 2 * mat);
-    double2 *K = reinterpret_cast<double2 *>(base + 2 * mat + per_seg(seg));
-    double *part = reinterpret_cast<double *>(base + 2 * mat + 2 * per_seg(seg));
-    double2 *ckpt = reinterpret_cast<double2 *>(base + 2 * mat + 2 * per_seg(seg) + part_bytes(seg));
+    double2 *K = reinterpret_cast<double2 *>(base + 2 * mat + per);
+    double *part = reinterpret_cast<double *>(base + 2 * mat + 2 * per);
+    double2 *ckpt = reinterpret_cast<double2 *>(base + 2 * mat + 2 * per + partb);
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const long long nsub = (long long)P->n_slices * P->n_rk;
@@ -2610,7 +2922,7 @@ grape_status grape_batch_create(grape_problem_t *problems, int32_t n, int32_t n_
     grape_batch *B = new grape_batch();
     auto bail = [&](grape_status s) { restore_tiles(B); delete B; return s; };
     B->device = dev;
-    B->probs.assign(problems, problems + n);
+    for (int i = 0; i < n; ++i) B->probs.push_back(active(problems[i]));   // on their subspaces
     bool tune = true;
     if (const char *env = std::getenv("GRAPE_BATCH_TUNE")) tune = std::atoi(env) != 0;
     if (tune) {
@@ -3242,7 +3554,7 @@ grape_status grape_submit(grape_server_t S, grape_problem_t P, const double *u0,
         !(prm->step0 > 0.0) || prm->tol < 0.0)
         return fail(GRAPE_EINVAL, "bad optimisation parameters");
     ServerJob *j = new ServerJob();
-    j->P = P;
+    j->P = active(P);
     j->prm = *prm;
     j->n = P->n_slices * P->R;
     j->u0.assign(u0, u0 + j->n);

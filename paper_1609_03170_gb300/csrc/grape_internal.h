@@ -40,6 +40,9 @@ struct PropTables {
     const double2 *vR;          // [nt][d]
     const void *vLs, *vRs;      // the same in the kernels' storage format (read from global
                                 // memory by the grid kernel)
+    // tables of state s start s * stride entries in (stride 0: all states
+    // share one table; states of different invariant subspaces do not)
+    long long a0_stride, ak_stride, v_stride;
 };
 
 // One RK4 sweep over substeps [sub_begin, sub_end) of one segment.  The
@@ -86,7 +89,7 @@ struct PropArgs {
                                         // wait before the pushes (hides its latency)
     int raw;                            // prop_s_kernel: A0 and every A_k kept in shared memory
     int dconst;                         // prop_s_kernel: own-entry coefficients the same in every slice
-    const double *src;                  // adjoint source on the diagonal per row (App. B), or null
+    const double *src;                  // [n_states][d] adjoint source on the diagonal (App. B), or null
     // grid kernel (stage values in global memory, windows loaded per stage;
     // ncl = CTAs per state, htab/maxwin/cu/hb as for the Hermitian kernel)
     void *gbuf;                         // [2][n_states][d*d] stage-input buffers
@@ -128,6 +131,8 @@ struct TraceArgs {
     int cb_do[GRAPE_MAXCB];     // distinct-offset index of band entry c
     int do_off[GRAPE_MAXDO];    // distinct offsets
     const void *cb_s;           // [ncb][d]  Hk_b[m], storage format of the number type
+    long long cb_stride, st_stride;   // entries between the states' band and sandwich tables
+                                      // (0: shared by all states)
     const void *K;              // adjoint-side matrices (storage format)
     const void *Y;              // forward-side matrices (storage format)
     long long npairs;           // matrices per output row
@@ -181,6 +186,8 @@ inline size_t trace_tile_smem(int nbuf, int kcap) {
                                            int d2, double *F, cudaStream_t stream);             \
     cudaError_t grape_launch_to_double_##SUFFIX(const void *src, double2 *dst, size_t n,        \
                                                 cudaStream_t stream);                           \
+    cudaError_t grape_launch_expand_##SUFFIX(const void *src, double2 *dst, const int *map, int m, \
+                                             int d, int n_states, cudaStream_t stream);          \
     cudaError_t grape_launch_grid_##SUFFIX(const PropArgs &p, int nblocks, int variant,         \
                                            size_t smem, cudaStream_t stream);                   \
     cudaError_t grape_prepare_grid_##SUFFIX(int variant, size_t smem_total, size_t smem,        \

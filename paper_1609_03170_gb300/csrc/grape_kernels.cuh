@@ -56,7 +56,7 @@ template <class Num>
 __device__ __forceinline__ typename Num::val with_source(const PropArgs &p, long long n, int i, int j,
                                                          typename Num::val v) {
     if (p.src && p.reverse && (n % p.n_rk) == 0 && i == j)
-        return Num::add_real(v, Num::real_const(p.src[i]));
+        return Num::add_real(v, Num::real_const(p.src[(blockIdx.x / p.ncl) * p.d + i]));   // the CTA's state
     return v;
 }
 
@@ -84,7 +84,7 @@ __device__ __forceinline__ void st_remote(uint32_t addr, float4 v) {
 // shared memory).  Called by every thread of the CTA (it holds a barrier).
 template <class Num>
 __device__ __forceinline__ void build_bands(typename Num::store_t *dst, const PropArgs &p,
-                                            int slice) {
+                                            int slice, int state) {
     using S = typename Num::store_t;
     using R = typename Num::real_t;
     __shared__ R ucv[GRAPE_MAXR];
@@ -92,8 +92,8 @@ __device__ __forceinline__ void build_bands(typename Num::store_t *dst, const Pr
     const double *uj = p.u + (size_t)slice * p.R;
     if (threadIdx.x < p.R) ucv[threadIdx.x] = Num::real_const(__ldg(&uj[threadIdx.x]));
     __syncthreads();
-    const S *A0 = static_cast<const S *>(p.tab.A0s);
-    const S *Ak = static_cast<const S *>(p.tab.Aks);
+    const S *A0 = static_cast<const S *>(p.tab.A0s) + (size_t)state * p.tab.a0_stride;
+    const S *Ak = static_cast<const S *>(p.tab.Aks) + (size_t)state * p.tab.ak_stride;
     for (int idx = threadIdx.x; idx < nbd; idx += blockDim.x) {
         typename Num::val v = Num::load(A0[idx]);
         for (int k = 0; k < p.R; ++k) v = Num::axpy(ucv[k], Num::load(Ak[(size_t)k * nbd + idx]), v);
@@ -218,8 +218,8 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_kernel(const PropA
     const V vzero = Num::zero();
     for (int i = threadIdx.x; i < 2 * p.win; i += nth) buf0[i] = Num::store(vzero);
     for (int i = threadIdx.x; i < p.tab.nt * d; i += nth) {
-        vL[i] = Num::store(Num::from_double2(__ldg(&p.tab.vL[i])));
-        vR[i] = Num::store(Num::from_double2(__ldg(&p.tab.vR[i])));
+        vL[i] = Num::store(Num::from_double2(__ldg(&p.tab.vL[(size_t)state * p.tab.v_stride + i])));
+        vR[i] = Num::store(Num::from_double2(__ldg(&p.tab.vR[(size_t)state * p.tab.v_stride + i])));
     }
     for (int e = e0 + threadIdx.x; e < e1; e += nth) rc[e - e0] = make_int2(e / d, e % d);
     if (threadIdx.x < 4) {
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_kernel(const PropA
     long long n_first = p.reverse ? p.sub_end - 1 : p.sub_begin;
     if (nsub <= 0) n_first = p.sub_begin;
     int jcur = (int)(n_first / p.n_rk);
-    build_bands<Num>(bands, p, jcur);
+    build_bands<Num>(bands, p, jcur, state);
     cluster_sync_all();   // every CTA of the cluster runs and has zeroed its windows
 
     for (int e = e0 + threadIdx.x; e < e1; e += nth) {
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_kernel(const PropA
                 const long long nn = p.reverse ? n - 1 : n + 1;
                 const int jn = (int)(nn / p.n_rk);
                 if (jn != jcur) {
-                    build_bands<Num>(bands + (tb ^ 1) * nbd, p, jn);
+                    build_bands<Num>(bands + (tb ^ 1) * nbd, p, jn, state);
                     jcur = jn;
                     flip = true;
                 }
@@ -696,8 +696,8 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
     const V vzero = Num::zero();
     for (int i = threadIdx.x; i < 2 * wst; i += nth) buf0[i] = Num::store(vzero);
     for (int i = threadIdx.x; i < p.tab.nt * d; i += nth) {
-        vL[i] = Num::store(Num::from_double2(__ldg(&p.tab.vL[i])));
-        vR[i] = Num::store(Num::from_double2(__ldg(&p.tab.vR[i])));
+        vL[i] = Num::store(Num::from_double2(__ldg(&p.tab.vL[(size_t)state * p.tab.v_stride + i])));
+        vR[i] = Num::store(Num::from_double2(__ldg(&p.tab.vR[(size_t)state * p.tab.v_stride + i])));
     }
     if (threadIdx.x < 4) {
         cg[threadIdx.x] = Num::real_const(p.g[threadIdx.x]);
@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
     long long n_first = p.reverse ? p.sub_end - 1 : p.sub_begin;
     if (nsub <= 0) n_first = p.sub_begin;
     int jcur = (int)(n_first / p.n_rk);
-    build_bands<Num>(bands, p, jcur);
+    build_bands<Num>(bands, p, jcur, state);
     __syncthreads();
     const int u0 = tab[GRAPE_HTAB_CTA(rank) + 0], u1 = tab[GRAPE_HTAB_CTA(rank) + 1];
     const int wr0 = tab[GRAPE_HTAB_CTA(rank) + 2], nrows = tab[GRAPE_HTAB_CTA(rank) + 3];
@@ -879,7 +879,7 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
                 const long long nn = p.reverse ? n - 1 : n + 1;
                 const int jn = (int)(nn / p.n_rk);
                 if (jn != jcur) {
-                    build_bands<Num>(bands + (tb ^ 1) * nbd, p, jn);
+                    build_bands<Num>(bands + (tb ^ 1) * nbd, p, jn, state);
                     __syncthreads();             // the new table before the next stage reads it
                     jcur = jn;
                     flip = true;
@@ -1038,10 +1038,10 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const Pro
     const bool clu = p.ncl > 1;
     const uint32_t mbar_sa = smem_u32(mbar);
     const uint32_t buf0_sa = smem_u32(buf0);
-    const S *vL = static_cast<const S *>(p.tab.vLs);
-    const S *vR = static_cast<const S *>(p.tab.vRs);
-    const S *gA0 = static_cast<const S *>(p.tab.A0s);
-    const S *gAk = static_cast<const S *>(p.tab.Aks);
+    const S *vL = static_cast<const S *>(p.tab.vLs) + (size_t)state * p.tab.v_stride;
+    const S *vR = static_cast<const S *>(p.tab.vRs) + (size_t)state * p.tab.v_stride;
+    const S *gA0 = static_cast<const S *>(p.tab.A0s) + (size_t)state * p.tab.a0_stride;
+    const S *gAk = static_cast<const S *>(p.tab.Aks) + (size_t)state * p.tab.ak_stride;
 
     if (tid == 0) {
         s_err = 0;
@@ -1332,7 +1332,7 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const Pro
                 }
                 x = acc;
                 if (left == 1 && p.src && p.reverse && i == j)       // the running cost's source (App. B)
-                    x = Num::add_real(x, Num::real_once(p.src[i]));
+                    x = Num::add_real(x, Num::real_once(p.src[state * d + i]));
                 return Num::scale(RK::g(p, 0), x);
             };
             S *std_ = st ? st + (size_t)p.store_map[s] * sset : nullptr;
@@ -1470,8 +1470,11 @@ __global__ void __launch_bounds__(GRAPE_GRID_THREADS, 1) prop_g_kernel(const Pro
     S *as = xs + p.cu;
     S *Dt = as + p.cu;
     S *bands = Dt + (p.fold ? p.cu : 0);
-    const S *vL = static_cast<const S *>(p.tab.vLs);
-    const S *vR = static_cast<const S *>(p.tab.vRs);
+    const int nct = p.ncl;                       // CTAs per state
+    const int rank = blockIdx.x % nct;
+    const int state = blockIdx.x / nct;
+    const S *vL = static_cast<const S *>(p.tab.vLs) + (size_t)state * p.tab.v_stride;
+    const S *vR = static_cast<const S *>(p.tab.vRs) + (size_t)state * p.tab.v_stride;
     int2 *rc = reinterpret_cast<int2 *>(bands + nbd);
     R *cg = reinterpret_cast<R *>(rc + p.cu);
     R *ca = cg + 4;
@@ -1483,9 +1486,6 @@ __global__ void __launch_bounds__(GRAPE_GRID_THREADS, 1) prop_g_kernel(const Pro
     short *nbad = reinterpret_cast<short *>(tab + p.htab_len);
     const int ns = SH::NB ? 2 * SH::NB + SH::NT : 2 * p.tab.nb + p.tab.nt;
     const int nstride = ns + 1;
-    const int nct = p.ncl;                       // CTAs per state
-    const int rank = blockIdx.x % nct;
-    const int state = blockIdx.x / nct;
     S *gb0 = static_cast<S *>(p.gbuf) + (size_t)state * d2;
     S *gb1 = static_cast<S *>(p.gbuf) + (size_t)(p.n_states + state) * d2;
     const S *x_in = static_cast<const S *>(p.x_in) + (size_t)state * d2;
@@ -1510,7 +1510,7 @@ __global__ void __launch_bounds__(GRAPE_GRID_THREADS, 1) prop_g_kernel(const Pro
     long long n_first = p.reverse ? p.sub_end - 1 : p.sub_begin;
     if (nsub <= 0) n_first = p.sub_begin;
     int jcur = (int)(n_first / p.n_rk);
-    build_bands<Num>(bands, p, jcur);
+    build_bands<Num>(bands, p, jcur, state);
     __syncthreads();
     const int u0 = tab[GRAPE_HTAB_CTA(rank) + 0], u1 = tab[GRAPE_HTAB_CTA(rank) + 1];
     const int wr0 = tab[GRAPE_HTAB_CTA(rank) + 2], nrows = tab[GRAPE_HTAB_CTA(rank) + 3];
@@ -1579,7 +1579,7 @@ __global__ void __launch_bounds__(GRAPE_GRID_THREADS, 1) prop_g_kernel(const Pro
         }
         __syncthreads();
         if (band_next >= 0) {                    // no thread reads the table now
-            build_bands<Num>(bands, p, band_next);
+            build_bands<Num>(bands, p, band_next, state);
             band_next = -1;
         }
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = nth >> 5;
@@ -1750,13 +1750,20 @@ __global__ void __launch_bounds__(256) trace_kernel(const TraceArgs p) {
     const size_t d2 = (size_t)d * d;
     S *svL = hv + p.ncb * d;                         // [nst][d] sandwich tables
     S *svR = svL + p.nst * d;
-    for (int i = threadIdx.x; i < p.ncb * d; i += blockDim.x)
-        hv[i] = static_cast<const S *>(p.cb_s)[i];
-    for (int i = threadIdx.x; i < p.nst * d; i += blockDim.x) {
-        svL[i] = static_cast<const S *>(p.st_vLs)[i];
-        svR[i] = static_cast<const S *>(p.st_vRs)[i];
-    }
-    __syncthreads();
+    // the tables of pair q's state (pair q is state q; reloaded per pair only
+    // when the states have tables of their own)
+    auto load_tables = [&](long long q) {
+        const S *cb = static_cast<const S *>(p.cb_s) + (size_t)q * p.cb_stride;
+        const S *vl = static_cast<const S *>(p.st_vLs) + (size_t)q * p.st_stride;
+        const S *vr = static_cast<const S *>(p.st_vRs) + (size_t)q * p.st_stride;
+        for (int i = threadIdx.x; i < p.ncb * d; i += blockDim.x) hv[i] = cb[i];
+        for (int i = threadIdx.x; i < p.nst * d; i += blockDim.x) {
+            svL[i] = vl[i];
+            svR[i] = vr[i];
+        }
+        __syncthreads();
+    };
+    load_tables(q0);
     typename Num::acc Z[GRAPE_MAXCB];                // lane-private, in the number type
 #pragma unroll
     for (int c = 0; c < GRAPE_MAXCB; ++c) Z[c] = Num::acc_zero();
@@ -1768,6 +1775,10 @@ __global__ void __launch_bounds__(256) trace_kernel(const TraceArgs p) {
 
 #pragma unroll 1
     for (long long q = q0; q < q1; ++q) {
+        if (q > q0 && (p.cb_stride | p.st_stride)) {
+            __syncthreads();                         // every warp is done with the previous state's tables
+            load_tables(q);
+        }
         const size_t moff = ((size_t)row * p.npairs + q) * d2;
         const S *K = Kb + moff;
         const S *Y = Yb + moff;
@@ -1841,9 +1852,9 @@ __global__ void __launch_bounds__(256) trace_packed_kernel(const TraceArgs p) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const S *Kb = static_cast<const S *>(p.K);
     const S *Yb = static_cast<const S *>(p.Y);
-    const S *cbs = static_cast<const S *>(p.cb_s);
-    const S *svLs = static_cast<const S *>(p.st_vLs);
-    const S *svRs = static_cast<const S *>(p.st_vRs);
+    const S *cbs = static_cast<const S *>(p.cb_s) + (size_t)state * p.cb_stride;
+    const S *svLs = static_cast<const S *>(p.st_vLs) + (size_t)state * p.st_stride;
+    const S *svRs = static_cast<const S *>(p.st_vRs) + (size_t)state * p.st_stride;
     typename Num::acc Z[GRAPE_MAXCB];
 #pragma unroll
     for (int c = 0; c < GRAPE_MAXCB; ++c) Z[c] = Num::acc_zero();
@@ -1933,7 +1944,7 @@ __global__ void __launch_bounds__(256) trace_packed_fast_kernel(const TraceArgs 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const S *Kb = static_cast<const S *>(p.K);
     const S *Yb = static_cast<const S *>(p.Y);
-    const S *cbs = static_cast<const S *>(p.cb_s);
+    const S *cbs = static_cast<const S *>(p.cb_s) + (size_t)state * p.cb_stride;
     typename Num::acc Z[GRAPE_MAXCB];
 #pragma unroll
     for (int c = 0; c < GRAPE_MAXCB; ++c) Z[c] = Num::acc_zero();
@@ -2060,7 +2071,7 @@ __global__ void __launch_bounds__(GRAPE_TRACE_THREADS, 2) trace_tile_kernel(cons
     const size_t pstride = (size_t)p.n_states * NU;
     const S *Yp = static_cast<const S *>(p.Y) + (row_base + state) * NU;
     const S *Kp = static_cast<const S *>(p.K) + (row_base + state) * NU;
-    const S *cbs = static_cast<const S *>(p.cb_s);
+    const S *cbs = static_cast<const S *>(p.cb_s) + (size_t)state * p.cb_stride;
     const long long limit = p.spin;                  // the pipeline's waits
     const long long drain = 1LL << 31;               // waits for copies already issued
 
@@ -2221,7 +2232,7 @@ static __global__ void __launch_bounds__(256) trace_finish_kernel(const TraceArg
     p.G[(size_t)row * p.R + k] = s;
 }
 
-// x[s][i][i] += src[i] (real): the adjoint's start value at the final time
+// x[s][i][i] += src[s][i] (real): the adjoint's start value at the final time
 // carries the running cost's last term (App. B)
 template <class Num>
 __global__ void __launch_bounds__(256) add_diag_kernel(void *x_v, const double *src, int d, int n_states) {
@@ -2230,10 +2241,10 @@ __global__ void __launch_bounds__(256) add_diag_kernel(void *x_v, const double *
     if (idx >= d * n_states) return;
     const int st = idx / d, i = idx - st * d;
     S *x = static_cast<S *>(x_v) + (size_t)st * d * d + (size_t)i * d + i;
-    *x = Num::store(Num::add_real(Num::load(*x), Num::real_const(src[i])));
+    *x = Num::store(Num::add_real(Num::load(*x), Num::real_const(src[idx])));
 }
 
-// out[row] = sum over states and i of diag[i] Re x_row[s][i][i], states then
+// out[row] = sum over states and i of diag[s][i] Re x_row[s][i][i], states then
 // rows in index order (FP64); x_row = x + row * row_stride entries
 // (packed: the states are upper triangles of d(d+1)/2 entries)
 template <class Num>
@@ -2249,7 +2260,7 @@ __global__ void __launch_bounds__(128) penalty_rows_kernel(const void *x_v, long
     for (int st = 0; st < n_states; ++st)
         for (int i = 0; i < d; ++i) {
             const size_t ii = packed ? (size_t)packed_index(i, i, d) : (size_t)i * d + i;
-            acc = fma(diag[i], Num::to_double2(Num::load(x[st * m + ii])).x, acc);
+            acc = fma(diag[(size_t)st * d + i], Num::to_double2(Num::load(x[st * m + ii])).x, acc);
         }
     out[row] = acc;
 }
@@ -2294,6 +2305,25 @@ __global__ void __launch_bounds__(256) to_double_kernel(const void *src_v, doubl
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
          i += (size_t)gridDim.x * blockDim.x)
         dst[i] = Num::to_double2(Num::load(src[i]));
+}
+
+// rho(T) of states kept in an invariant subspace, as full matrices: entry
+// (i, j) of state s is the subspace entry at the positions map[s][i] and
+// map[s][j], or zero when either index lies outside (-1).  Bound by the
+// 16 B written per entry of the full matrix.
+template <class Num>
+__global__ void __launch_bounds__(256) expand_kernel(const void *src_v, double2 *dst, const int *map, int m, int d,
+                                                     int n_states) {
+    using S = typename Num::store_t;
+    const S *src = static_cast<const S *>(src_v);
+    const size_t n = (size_t)n_states * d * d;
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+        const size_t row = e / d;                    // state * d + i
+        const int j = (int)(e - row * d), st = (int)(row / d);
+        const int a = map[row], b = map[(size_t)st * d + j];
+        dst[e] = (a >= 0 && b >= 0) ? Num::to_double2(Num::load(src[((size_t)st * m + a) * m + b]))
+                                    : make_double2(0.0, 0.0);
+    }
 }
 
 // ------------------------------------------------------------------ launchers
@@ -2462,6 +2492,13 @@ cudaError_t launch_to_double(const void *src, double2 *dst, size_t n, cudaStream
 }
 
 template <class Num>
+cudaError_t launch_expand(const void *src, double2 *dst, const int *map, int m, int d, int ns, cudaStream_t s) {
+    const size_t n = (size_t)ns * d * d;
+    expand_kernel<Num><<<(unsigned)std::min<size_t>((n + 255) / 256, 4096), 256, 0, s>>>(src, dst, map, m, d, ns);
+    return cudaGetLastError();
+}
+
+template <class Num>
 cudaError_t launch_add_diag(void *x, const double *src, int d, int ns, cudaStream_t s) {
     add_diag_kernel<Num><<<(d * ns + 255) / 256, 256, 0, s>>>(x, src, d, ns);
     return cudaGetLastError();
@@ -2506,6 +2543,10 @@ static cudaError_t launch_penalty_finish(const double *pen, long long count, dou
     cudaError_t grape_launch_to_double_##SUFFIX(const void *src, double2 *dst, size_t n,        \
                                                 cudaStream_t s) {                               \
         return grape_k::launch_to_double<NUM>(src, dst, n, s);                                  \
+    }                                                                                           \
+    cudaError_t grape_launch_expand_##SUFFIX(const void *src, double2 *dst, const int *map, int m, \
+                                             int d, int n_states, cudaStream_t s) {             \
+        return grape_k::launch_expand<NUM>(src, dst, map, m, d, n_states, s);                   \
     }                                                                                           \
     cudaError_t grape_launch_grid_##SUFFIX(const PropArgs &p, int nblocks, int variant,         \
                                            size_t smem, cudaStream_t s) {                       \
