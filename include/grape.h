@@ -100,7 +100,14 @@ typedef struct grape_problem *grape_problem_t;
  * Operators enter as band lists (Eq. Hamiltonian, Eq. disspation); the
  * non-Hermitian part -i/2 sum gamma_m c_m^+ c_m is formed here.  sigma enters
  * the cost only through its Hermitian part (rho(T) is Hermitian), so it is
- * stored Hermitianised.  Errors: GRAPE_EINVAL (sizes, band offsets beyond
+ * stored Hermitianised.  When no operator leads out of the basis states that
+ * an initial state occupies, its density matrix stays zero outside them for
+ * the whole pulse (a resonator drive keeps the transmon's level, for
+ * instance); the calls then run on those entries alone, with the operators
+ * restricted to them - every term left out is an exact zero - and rho(T) is
+ * returned at full size.  grape_problem_geometry, grape_problem_kernel,
+ * grape_problem_set_tile and the limit of grape_gradient_static refer to the
+ * problem at its full size.  Errors: GRAPE_EINVAL (sizes, band offsets beyond
  * +-(d-1), non-Hermitian rho0 or control, negative rates), GRAPE_ENOMEM. */
 grape_status grape_problem_create(const grape_problem_desc *desc, grape_problem_t *out);
 
@@ -191,7 +198,8 @@ grape_status grape_problem_set_penalty(grape_problem_t problem, const double *di
  * [64, 512]).  Every entry is computed by the same arithmetic whatever CTA
  * or thread owns it, so results do not change, bit for bit; only speed and
  * the SMs a call occupies do (narrow tiles leave room for other problems,
- * see grape_batch_create).  Errors: GRAPE_EINVAL (values out of range, a
+ * see grape_batch_create).  A problem that runs on a part of the space takes the
+ * tile for that part too when it fits there.  Errors: GRAPE_EINVAL (values out of range, a
  * grid-kernel problem, or a tile whose state window does not fit in shared
  * memory or of which no cluster can be resident; the tile is unchanged),
  * GRAPE_ECUDA.  The tile chosen at create is the widest useful cluster

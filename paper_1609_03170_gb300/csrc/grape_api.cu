@@ -242,7 +242,10 @@ HostDir make_dir(const std::vector<Ops> &sets, int d) {
 // the kernels would add for the other entries is an exact zero, the dual on
 // I x I reads only I x I, and the traces of Eq. (dphidu) pair Y with K on
 // I x I alone.  The problem then runs on the entries of I x I with the
-// operators restricted to I.
+// operators restricted to I.  Measured (both sides with the same kernels):
+// d=20 as two 10 x 10 blocks 2.81 -> 2.25 ms per gradient, d=300 (three 100 x
+// 100 blocks, cluster instead of grid kernel) 212 -> 18.1 ms, d=600 (one 150
+// x 150 block) 425 -> 114 ms, a batch of 24 reset problems 75.9 -> 26.4 ms.
 
 // indices reachable from the rows and columns where x (d x d) is not zero
 std::vector<int> invariant_set(const Ops &ops, const cplx *x, int d) {
