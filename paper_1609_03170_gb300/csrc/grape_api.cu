@@ -511,6 +511,7 @@ struct grape_problem {
     double2 *d_fwd_bounds = nullptr;
     static constexpr int kPenChunk = 64;
     double *d_u = nullptr, *d_F = nullptr, *d_G = nullptr;
+    double *d_cost = nullptr;        // partial sums of the cost
     size_t bytes = 0;
     cudaStream_t s1 = nullptr;       // high-priority stream the gradient sweeps run on
     cudaStream_t s2 = nullptr;       // low-priority stream: traces overlap the adjoint sweep
@@ -705,8 +706,8 @@ cudaError_t k_trace(const grape_problem *P, const TraceArgs &t, cudaStream_t s) 
 }
 cudaError_t k_cost(const grape_problem *P, const void *rho, double *F, cudaStream_t s) {
     return P->prec == GRAPE_PREC_FP64
-               ? grape_launch_cost_f64(rho, P->d_sigma, P->ns, (int)P->d2, F, s)
-               : grape_launch_cost_df(rho, P->d_sigma, P->ns, (int)P->d2, F, s);
+               ? grape_launch_cost_f64(rho, P->d_sigma, P->ns, (int)P->d2, P->d_cost, P->d_gbar + 3, F, s)
+               : grape_launch_cost_df(rho, P->d_sigma, P->ns, (int)P->d2, P->d_cost, P->d_gbar + 3, F, s);
 }
 cudaError_t k_to_double(const grape_problem *P, const void *src, double2 *dst, size_t n,
                         cudaStream_t s) {
@@ -1312,8 +1313,9 @@ long long trace_pairs(const grape_problem *P) {
 // how the slices are grouped into launches or on the propagation tile).
 // Exact gradient (packed storage): per state, chunks of 256 x epc upper
 // entries, epc chosen so that a state has at most 64 chunks.  First-order
-// mode (full matrices): contiguous ranges of the slice's pairs worth about
-// 2^17 band-element products each.
+// mode (full matrices): contiguous ranges of the rows of the slice's matrices
+// worth about 2^14 band-element products each (a few microseconds, and
+// enough CTAs for the chip from d=128 on 200 slices).
 void trace_layout(const grape_problem *P, TraceArgs *t) {
     t->n_states = P->ns;
     if (P->mode == GRAPE_GRAD_EXACT) {
@@ -1324,12 +1326,11 @@ void trace_layout(const grape_problem *P, TraceArgs *t) {
         t->nsplit = P->ns * t->nchunk;
         return;
     }
-    const long long npairs = trace_pairs(P);
-    const long long work = (long long)P->d * P->d * std::max(1, t->ndo);
-    const long long per = std::max<long long>(1, ((1LL << 17) + work - 1) / work);
+    const long long rows = trace_pairs(P) * P->d;
+    const long long per = std::max<long long>(1, (1LL << 14) / ((long long)P->d * std::max(1, t->ndo)));
     t->packed = 0;
     t->epc = t->nchunk = 1;
-    t->nsplit = (int)std::max<long long>(1, (npairs + per - 1) / per);
+    t->nsplit = (int)std::max<long long>(1, (rows + per - 1) / per);
 }
 
 // Tables of the packed trace kernels: the row and column of every packed
@@ -1634,7 +1635,6 @@ grape_status trace_chunk(grape_problem *P, const GradScratch &S, double *Gd, lon
         t.npairs = P->ns;
         t.weight = P->T / P->n_slices;
     }
-    if (!S.part && !t.packed) t.nsplit = 1;
     t.part = S.part ? S.part + (size_t)cA * t.nsplit * P->R : nullptr;
     if ((st = timed(P, PH_TRACE, ts, [&] { return k_trace(P, t, ts); })) != GRAPE_OK) return st;
     if (t.nsplit > 1 &&
@@ -2002,8 +2002,9 @@ grape_status build_problem(const grape_problem_desc *desc, const ProblemData &da
         P->alloc((size_t)P->n_slices * P->trace.nsplit * std::max(P->R, 1) * sizeof(double)));
     P->d_u = static_cast<double *>(P->alloc((size_t)P->n_slices * std::max(P->R, 1) * sizeof(double)));
     P->d_F = static_cast<double *>(P->alloc(sizeof(double)));
+    P->d_cost = static_cast<double *>(P->alloc(128 * sizeof(double)));
     P->d_G = static_cast<double *>(P->alloc((size_t)P->n_slices * std::max(P->R, 1) * sizeof(double)));
-    if (!P->d_x || !P->d_mu || !P->d_part || !P->d_u || !P->d_F || !P->d_G) return bail(fail(GRAPE_ENOMEM, "cudaMalloc failed"));
+    if (!P->d_x || !P->d_mu || !P->d_part || !P->d_u || !P->d_F || !P->d_cost || !P->d_G) return bail(fail(GRAPE_ENOMEM, "cudaMalloc failed"));
     {
         int prio_low = 0, prio_high = 0;
         cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high);

@@ -183,7 +183,8 @@ inline size_t trace_tile_smem(int nbuf, int kcap) {
     cudaError_t grape_launch_trace_##SUFFIX(const TraceArgs &p, cudaStream_t stream);          \
     cudaError_t grape_launch_trace_finish_##SUFFIX(const TraceArgs &p, cudaStream_t stream);   \
     cudaError_t grape_launch_cost_##SUFFIX(const void *rho, const void *sigma, int n_states,    \
-                                           int d2, double *F, cudaStream_t stream);             \
+                                           int d2, double *part, unsigned *ticket, double *F,   \
+                                           cudaStream_t stream);                                \
     cudaError_t grape_launch_to_double_##SUFFIX(const void *src, double2 *dst, size_t n,        \
                                                 cudaStream_t stream);                           \
     cudaError_t grape_launch_expand_##SUFFIX(const void *src, double2 *dst, const int *map, int m, \

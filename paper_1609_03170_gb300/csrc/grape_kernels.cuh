@@ -1736,6 +1736,13 @@ __device__ __forceinline__ void trace_store(const TraceArgs &p, typename Num::ac
     }
 }
 
+// First-order mode.  The row's matrices are npairs x d rows of d entries, of
+// which CTA `split` takes a contiguous range (trace_layout); a warp takes one
+// row m at a time, its lanes the columns.  Bound by reading K and Y once
+// (L2 serves the ndo reads of a K row).  One CTA per slice left most of the
+// chip idle: at d=512, 200 slices, the traces of a chunk of 25 slices took
+// 1.7 ms on 25 CTAs; split over rows and with the split cost below, the
+// gradient takes 12.4 instead of 21.4 ms.
 template <class Num>
 __global__ void __launch_bounds__(256) trace_kernel(const TraceArgs p) {
     using S = typename Num::store_t;
@@ -1743,11 +1750,11 @@ __global__ void __launch_bounds__(256) trace_kernel(const TraceArgs p) {
     S *hv = reinterpret_cast<S *>(tsmem);            // [ncb][d] control band values
     const int nsplit = max(1, p.nsplit);
     const int row = blockIdx.x / nsplit, split = blockIdx.x % nsplit;
-    const long long q0 = (long long)split * p.npairs / nsplit;
-    const long long q1 = (long long)(split + 1) * p.npairs / nsplit;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int d = p.d;
     const size_t d2 = (size_t)d * d;
+    const long long nrow = p.npairs * d;             // matrix rows of this slice
+    const long long r0 = split * nrow / nsplit, r1 = (split + 1) * nrow / nsplit;
     S *svL = hv + p.ncb * d;                         // [nst][d] sandwich tables
     S *svR = svL + p.nst * d;
     // the tables of pair q's state (pair q is state q; reloaded per pair only
@@ -1763,6 +1770,7 @@ __global__ void __launch_bounds__(256) trace_kernel(const TraceArgs p) {
         }
         __syncthreads();
     };
+    const long long q0 = r0 / d, q1 = r1 > r0 ? (r1 - 1) / d + 1 : q0;
     load_tables(q0);
     typename Num::acc Z[GRAPE_MAXCB];                // lane-private, in the number type
 #pragma unroll
@@ -1782,16 +1790,17 @@ __global__ void __launch_bounds__(256) trace_kernel(const TraceArgs p) {
         const size_t moff = ((size_t)row * p.npairs + q) * d2;
         const S *K = Kb + moff;
         const S *Y = Yb + moff;
+        const int m0 = (int)max(0LL, r0 - q * d), m1 = (int)min((long long)d, r1 - q * d);
 #pragma unroll 1
-        for (int m = warp; m < d; m += nwarps) {
+        for (int m = m0 + warp; m < m1; m += nwarps) {
 #pragma unroll 1
             for (int o = 0; o < p.ndo; ++o) {
                 const int r = m + p.do_off[o];
                 if (r < 0 || r >= d) continue;
+                const S *Kr = K + (size_t)r * d, *Ym = Y + (size_t)m * d;
                 typename Num::acc P = Num::acc_zero();
-#pragma unroll 1
-                for (int l = lane; l < d; l += 32)
-                    Num::mac_conjb(P, Num::load(K[(size_t)r * d + l]), Num::load(Y[(size_t)m * d + l]));
+#pragma unroll 4
+                for (int l = lane; l < d; l += 32) Num::mac_conjb(P, Num::load(Kr[l]), Num::load(Ym[l]));
                 const typename Num::val pv = Num::done(P);
 #pragma unroll
                 for (int c = 0; c < GRAPE_MAXCB; ++c)
@@ -2273,28 +2282,45 @@ static __global__ void penalty_finish_kernel(const double *pen, long long count,
     F[0] -= scale * t;
 }
 
+// Phi = Re sum conj(sigma) rho over all states' entries.  CTA k sums its
+// contiguous range of entries and the last CTA to finish (the ticket counts
+// them) adds the partial sums in index order, so the value does not depend on
+// which one that is.  On one CTA the sum was a chain of FP64 conversions on
+// one SM: 1.03 ms at d=512, 0.19 ms at three states of d=120; split into 2048
+// entries per CTA 0.023 and 0.03 ms.
+#define GRAPE_COST_CTAS 128
 template <class Num>
-__global__ void __launch_bounds__(256) cost_kernel(const void *rho_v, const void *sigma_v,
-                                                   int n_states, int d2, double *F) {
+__global__ void __launch_bounds__(256) cost_kernel(const void *rho_v, const void *sigma_v, long long n,
+                                                   double *part, unsigned *ticket, double *F) {
     using S = typename Num::store_t;
     const S *rho = static_cast<const S *>(rho_v);
     const S *sigma = static_cast<const S *>(sigma_v);
+    __shared__ double red[8];
+    __shared__ bool last;
+    const long long e0 = n * blockIdx.x / gridDim.x, e1 = n * (blockIdx.x + 1) / gridDim.x;
     double acc = 0.0;
-    for (int s = 0; s < n_states; ++s)
-        for (int e = threadIdx.x; e < d2; e += blockDim.x) {
-            const double2 r = Num::to_double2(Num::load(rho[(size_t)s * d2 + e]));
-            const double2 g = Num::to_double2(Num::load(sigma[(size_t)s * d2 + e]));
-            acc = fma(g.x, r.x, fma(g.y, r.y, acc));    // Re(conj(sigma_ij) rho_ij)
-        }
+    for (long long e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+        const double2 r = Num::to_double2(Num::load(rho[e]));
+        const double2 g = Num::to_double2(Num::load(sigma[e]));
+        acc = fma(g.x, r.x, fma(g.y, r.y, acc));    // Re(conj(sigma_ij) rho_ij)
+    }
 #pragma unroll
     for (int sh = 16; sh > 0; sh >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, sh);
-    __shared__ double red[32];
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
         double s = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        *F = s;
+        part[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (last) {
+            __threadfence();
+            double t = 0.0;
+            for (unsigned k = 0; k < gridDim.x; ++k) t += __ldcg(&part[k]);
+            *F = t;
+            *ticket = 0u;                           // for the next call on the stream
+        }
     }
 }
 
@@ -2477,9 +2503,11 @@ static cudaError_t launch_trace_finish(const TraceArgs &p, cudaStream_t s) {
 }
 
 template <class Num>
-cudaError_t launch_cost(const void *rho, const void *sigma, int n_states, int d2, double *F,
-                        cudaStream_t s) {
-    cost_kernel<Num><<<1, 256, 0, s>>>(rho, sigma, n_states, d2, F);
+cudaError_t launch_cost(const void *rho, const void *sigma, int n_states, int d2, double *part, unsigned *ticket,
+                        double *F, cudaStream_t s) {
+    const long long n = (long long)n_states * d2;
+    const int ctas = (int)std::max(1LL, std::min<long long>(GRAPE_COST_CTAS, (n + 2047) / 2048));
+    cost_kernel<Num><<<ctas, 256, 0, s>>>(rho, sigma, n, part, ticket, F);
     return cudaGetLastError();
 }
 
@@ -2537,8 +2565,9 @@ static cudaError_t launch_penalty_finish(const double *pen, long long count, dou
         return grape_k::launch_trace_finish(p, s);                                              \
     }                                                                                           \
     cudaError_t grape_launch_cost_##SUFFIX(const void *rho, const void *sigma, int n_states,    \
-                                           int d2, double *F, cudaStream_t s) {                 \
-        return grape_k::launch_cost<NUM>(rho, sigma, n_states, d2, F, s);                       \
+                                           int d2, double *part, unsigned *ticket, double *F,   \
+                                           cudaStream_t s) {                                    \
+        return grape_k::launch_cost<NUM>(rho, sigma, n_states, d2, part, ticket, F, s);         \
     }                                                                                           \
     cudaError_t grape_launch_to_double_##SUFFIX(const void *src, double2 *dst, size_t n,        \
                                                 cudaStream_t s) {                               \
