@@ -520,6 +520,7 @@ struct grape_problem {
     static constexpr int kMaxChunks = 16;
     cudaEvent_t ev[kMaxChunks + 2] = {};
     cudaEvent_t evF[kMaxChunks] = {};   // forward chunk c done (concurrent sweeps)
+    cudaEvent_t evT[kMaxChunks] = {};   // traces of chunk c done (its stage storage may be reused)
     bool profiling = false;
     struct Mark { int phase; cudaEvent_t a, b; };
     std::vector<Mark> marks;
@@ -591,6 +592,8 @@ struct grape_problem {
         for (auto &e : ev)
             if (e) cudaEventDestroy(e);
         for (auto &e : evF)
+            if (e) cudaEventDestroy(e);
+        for (auto &e : evT)
             if (e) cudaEventDestroy(e);
         if (ev_fork3) cudaEventDestroy(ev_fork3);
         if (s3) cudaStreamDestroy(s3);
@@ -1298,10 +1301,11 @@ struct GradScratch {
     cudaEvent_t *ev = nullptr;   // kMaxChunks + 2 events when s2 is set
     double *part = nullptr;      // partial traces; null: one CTA per slice
     // concurrent sweeps (see concurrent_sweeps): the adjoint's stream, its
-    // fork event and the forward chunks' events; null: one sweep after the other
+    // fork event, the forward chunks' and the traces' events; null: one sweep
+    // after the other
     cudaStream_t s3 = nullptr;
     cudaEvent_t fork3 = nullptr;
-    cudaEvent_t *evF = nullptr;
+    cudaEvent_t *evF = nullptr, *evT = nullptr;
 };
 
 long long trace_pairs(const grape_problem *P) {
@@ -1492,12 +1496,15 @@ int adjoint_chunks(const grape_problem *P, long long j0, long long j1, bool conc
 // forward states: only the traces pair the two sweeps.  The forward sweep
 // then runs in the adjoint's chunks, and the trace of chunk c waits for both
 // sweeps to pass it.  The same holds for the first-order mode's boundary
-// states (d=128, 200 slices: 3.26 against 6.50 ms).  With the whole problem in one segment, on a
-// cluster kernel (the grid kernel's per-problem stage buffers and flags admit
+// states (d=128, 200 slices: 3.26 against 6.50 ms).  With checkpoints, the
+// forward sweep to the last checkpoint runs first beside nothing but the last
+// segment's adjoint; then each segment's recomputation runs beside its
+// adjoint, so the gradient takes about two sweeps instead of three (d=600,
+// 1000 slices in 5 segments: 113.5 -> 69.0 ms).  On a cluster kernel (the grid kernel's per-problem stage buffers and flags admit
 // one sweep at a time); GRAPE_CONCURRENT=0 turns it off.  Same kernels, same
 // arithmetic: the same bits.
-bool concurrent_sweeps(const grape_problem *P, int nseg) {
-    if (nseg != 1 || P->grid) return false;
+bool concurrent_sweeps(const grape_problem *P) {
+    if (P->grid) return false;
     if (const char *env = std::getenv("GRAPE_CONCURRENT"))
         if (std::atoi(env) == 0) return false;
     if (const char *env = std::getenv("GRAPE_TRACE_OVERLAP"))
@@ -1507,14 +1514,15 @@ bool concurrent_sweeps(const grape_problem *P, int nseg) {
 
 int gradient_launch_count(const grape_problem *P, int seg, int nseg, bool concurrent = false) {
     if (nseg <= 0) return -1;
-    int n = 2;                                    // forward sweep, cost
-    if (concurrent) n += adjoint_chunks(P, 0, P->n_slices, true) - 1;   // the forward in chunks
+    // the cost, and the forward sweep to the checkpoints (to the end when the
+    // sweeps are not side by side)
+    int n = 1 + ((nseg > 1 || !concurrent) ? 1 : 0);
     if (P->penalty) n += 3;                       // adjoint start, final-state value, sum
     for (int gi = 0; gi < nseg; ++gi) {
         const long long j0 = (long long)gi * seg;
         const long long j1 = std::min<long long>(P->n_slices, j0 + seg);
         const int nch = adjoint_chunks(P, j0, j1, concurrent);
-        n += (nseg > 1 ? 1 : 0) + nch;
+        n += nch + (concurrent ? nch : (nseg > 1 ? 1 : 0));   // adjoint, forward of the segment
         if (P->R > 0) n += nch * (P->trace.nsplit > 1 ? 2 : 1);
         if (P->penalty) n += 1;                   // boundary values of the segment
     }
@@ -1651,17 +1659,17 @@ grape_status trace_chunk(grape_problem *P, const GradScratch &S, double *Gd, lon
 }
 
 // The gradient with the forward and the adjoint sweep at the same time (see
-// concurrent_sweeps): the forward in the adjoint's chunks on s (then the
-// cost and the running penalty's rows), the adjoint on S.s3 (start value,
-// chunks last first), the trace of chunk c on S.s2 once both sweeps have
-// passed it; s then waits for both.
+// concurrent_sweeps).  With checkpoints, the forward sweep first stores them
+// up to the last segment.  Then per segment (last first): the forward in
+// chunks on s from its checkpoint (after the last segment the cost, and the
+// running penalty's rows), the adjoint on S.s3 (chunks last first), the trace
+// of chunk c on S.s2 once both sweeps have passed it.  The next segment's
+// sweeps write a chunk's stage storage once its traces are done.
 grape_status run_gradient_concurrent(grape_problem *P, const double *ud, double *Fd, double *Gd,
                                      cudaStream_t s, const GradScratch &S) {
     grape_status st;
     const size_t mat = full_set(P);
     const size_t pst = packed_set(P);
-    const long long j0 = 0, j1 = P->n_slices;
-    const int nch = adjoint_chunks(P, j0, j1, true);
     const bool exact = (P->mode == GRAPE_GRAD_EXACT);
     // stored entries per slice: every stage input, or the slice's boundary
     const size_t per_slice = exact ? (size_t)P->n_rk * 4 * pst : mat;
@@ -1673,57 +1681,87 @@ grape_status run_gradient_concurrent(grape_problem *P, const double *ud, double 
     if (P->penalty)
         GRAPE_CUDA_TRY(P->prec == GRAPE_PREC_FP64 ? grape_launch_add_diag_f64(S.mu, P->d_src, P->d, P->ns, sa)
                                                   : grape_launch_add_diag_df(S.mu, P->d_src, P->d, P->ns, sa));
-    // forward sweep in chunks, each storing its slices' stage inputs
-    for (int ci = 0; ci < nch; ++ci) {
-        const long long cA = j0 + (j1 - j0) * ci / nch;
-        const long long cB = j0 + (j1 - j0) * (ci + 1) / nch;
+    const double2 *seg_x0 = P->d_rho0;               // a segment's first state
+    if (S.nseg > 1) {
         PropArgs f = base_args(P, 0, ud);
-        f.sub_begin = cA * P->n_rk;
-        f.sub_end = cB * P->n_rk;
-        f.x_in = ci == 0 ? P->d_rho0 : S.x;
+        f.sub_begin = 0;
+        f.sub_end = (long long)(S.nseg - 1) * S.seg * P->n_rk;
+        f.x_in = P->d_rho0;
         f.x_out = S.x;
-        if (exact) f.stage_store = S.Y + (size_t)(cA - j0) * per_slice;
-        else { f.bound_store = S.Y + (size_t)(cA - j0) * per_slice; f.bound_step = P->n_rk; }
+        f.bound_store = S.ckpt;
+        f.bound_step = (long long)S.seg * P->n_rk;
         if ((st = launch_prop(P, f, s)) != GRAPE_OK) return st;
-        GRAPE_CUDA_TRY(cudaEventRecord(S.evF[ci], s));
     }
-    if ((st = timed(P, PH_COST, s, [&] { return k_cost(P, S.x, Fd, s); })) != GRAPE_OK) return st;
-    if (P->penalty) {
-        if ((st = pen_rows(P, S.x, 0, 1, P->n_slices, s)) != GRAPE_OK) return st;
-        if ((st = pen_rows(P, S.Y, (long long)per_slice, j1 - j0, j0, s, exact ? 1 : 0)) != GRAPE_OK)
+    long long prev = -1;                             // slices of the segment before, none: -1
+    for (int gi = S.nseg - 1; gi >= 0; --gi) {
+        const long long j0 = (long long)gi * S.seg;
+        const long long j1 = std::min<long long>(P->n_slices, j0 + S.seg);
+        const int nch = adjoint_chunks(P, j0, j1, true);
+        auto first = [&](int ci) { return j0 + (j1 - j0) * ci / nch; };
+        if (S.nseg > 1) seg_x0 = S.ckpt + (size_t)gi * mat;
+        // a segment of another length has other chunks: wait for all traces
+        // before it, else for those of the same chunk
+        const bool wait_all = prev >= 0 && prev != j1 - j0 && P->R > 0;
+        const bool wait_chunk = prev == j1 - j0 && P->R > 0;
+        if (wait_all) {
+            GRAPE_CUDA_TRY(cudaEventRecord(S.ev[grape_problem::kMaxChunks], ts));
+            GRAPE_CUDA_TRY(cudaStreamWaitEvent(s, S.ev[grape_problem::kMaxChunks], 0));
+            GRAPE_CUDA_TRY(cudaStreamWaitEvent(sa, S.ev[grape_problem::kMaxChunks], 0));
+        }
+        prev = j1 - j0;
+        // forward sweep in chunks, each storing its slices' stage inputs
+        for (int ci = 0; ci < nch; ++ci) {
+            if (wait_chunk) GRAPE_CUDA_TRY(cudaStreamWaitEvent(s, S.evT[ci], 0));
+            PropArgs f = base_args(P, 0, ud);
+            f.sub_begin = first(ci) * P->n_rk;
+            f.sub_end = first(ci + 1) * P->n_rk;
+            f.x_in = ci == 0 ? seg_x0 : S.x;
+            f.x_out = S.x;
+            double2 *store = S.Y + (size_t)(first(ci) - j0) * per_slice;
+            if (exact) f.stage_store = store;
+            else { f.bound_store = store; f.bound_step = P->n_rk; }
+            if ((st = launch_prop(P, f, s)) != GRAPE_OK) return st;
+            GRAPE_CUDA_TRY(cudaEventRecord(S.evF[ci], s));
+        }
+        if (gi == S.nseg - 1) {
+            if ((st = timed(P, PH_COST, s, [&] { return k_cost(P, S.x, Fd, s); })) != GRAPE_OK) return st;
+            if (P->penalty && (st = pen_rows(P, S.x, 0, 1, P->n_slices, s)) != GRAPE_OK) return st;
+        }
+        if (P->penalty && (st = pen_rows(P, S.Y, (long long)per_slice, j1 - j0, j0, s, exact ? 1 : 0)) != GRAPE_OK)
             return st;
-    }
-    // adjoint chunks (last slices first)
-    for (int ci = nch - 1; ci >= 0; --ci) {
-        const long long cA = j0 + (j1 - j0) * ci / nch;
-        const long long cB = j0 + (j1 - j0) * (ci + 1) / nch;
-        PropArgs b = base_args(P, 1, ud);
-        b.sub_begin = cA * P->n_rk;
-        b.sub_end = cB * P->n_rk;
-        b.reverse = 1;
-        b.x_in = S.mu;
-        b.x_out = S.mu;
-        if (exact) b.stage_store = S.K + (size_t)(cA - j0) * per_slice;
-        else { b.bound_store = S.K + (size_t)(cA - j0) * per_slice; b.bound_step = P->n_rk; }
-        if ((st = launch_prop(P, b, sa)) != GRAPE_OK) return st;
-        GRAPE_CUDA_TRY(cudaEventRecord(S.ev[ci], sa));
-    }
-    // the traces in the order the chunks become ready: the forward passes
-    // chunk c after c + 1 chunks, the adjoint after nch - c, so the middle
-    // chunks are ready first and the two ends last (one in-order stream)
-    int order[grape_problem::kMaxChunks];
-    for (int c = 0; c < nch; ++c) order[c] = c;
-    std::sort(order, order + nch, [nch](int a, int b) {
-        const int ra = std::max(a + 1, nch - a), rb = std::max(b + 1, nch - b);
-        return ra != rb ? ra < rb : a < b;
-    });
-    for (int k = 0; k < nch && P->R > 0; ++k) {
-        const int ci = order[k];
-        const long long cA = j0 + (j1 - j0) * ci / nch;
-        const long long cB = j0 + (j1 - j0) * (ci + 1) / nch;
-        GRAPE_CUDA_TRY(cudaStreamWaitEvent(ts, S.ev[ci], 0));
-        GRAPE_CUDA_TRY(cudaStreamWaitEvent(ts, S.evF[ci], 0));
-        if ((st = trace_chunk(P, S, Gd, cA, cB, (size_t)(cA - j0) * per_slice, ts)) != GRAPE_OK) return st;
+        // adjoint chunks (last slices first)
+        for (int ci = nch - 1; ci >= 0; --ci) {
+            if (wait_chunk) GRAPE_CUDA_TRY(cudaStreamWaitEvent(sa, S.evT[ci], 0));
+            PropArgs b = base_args(P, 1, ud);
+            b.sub_begin = first(ci) * P->n_rk;
+            b.sub_end = first(ci + 1) * P->n_rk;
+            b.reverse = 1;
+            b.x_in = S.mu;
+            b.x_out = S.mu;
+            double2 *store = S.K + (size_t)(first(ci) - j0) * per_slice;
+            if (exact) b.stage_store = store;
+            else { b.bound_store = store; b.bound_step = P->n_rk; }
+            if ((st = launch_prop(P, b, sa)) != GRAPE_OK) return st;
+            GRAPE_CUDA_TRY(cudaEventRecord(S.ev[ci], sa));
+        }
+        // the traces in the order the chunks become ready: the forward passes
+        // chunk c after c + 1 chunks, the adjoint after nch - c, so the middle
+        // chunks are ready first and the two ends last (one in-order stream)
+        int order[grape_problem::kMaxChunks];
+        for (int c = 0; c < nch; ++c) order[c] = c;
+        std::sort(order, order + nch, [nch](int a, int b) {
+            const int ra = std::max(a + 1, nch - a), rb = std::max(b + 1, nch - b);
+            return ra != rb ? ra < rb : a < b;
+        });
+        for (int k = 0; k < nch && P->R > 0; ++k) {
+            const int ci = order[k];
+            GRAPE_CUDA_TRY(cudaStreamWaitEvent(ts, S.ev[ci], 0));
+            GRAPE_CUDA_TRY(cudaStreamWaitEvent(ts, S.evF[ci], 0));
+            if ((st = trace_chunk(P, S, Gd, first(ci), first(ci + 1), (size_t)(first(ci) - j0) * per_slice, ts)) !=
+                GRAPE_OK)
+                return st;
+            GRAPE_CUDA_TRY(cudaEventRecord(S.evT[ci], ts));
+        }
     }
     GRAPE_CUDA_TRY(cudaEventRecord(S.ev[grape_problem::kMaxChunks + 1], sa));
     GRAPE_CUDA_TRY(cudaStreamWaitEvent(s, S.ev[grape_problem::kMaxChunks + 1], 0));
@@ -1741,7 +1779,7 @@ grape_status run_gradient_concurrent(grape_problem *P, const double *ud, double 
 // trace kernels of the finished chunks.
 grape_status run_gradient(grape_problem *P, const double *ud, double *Fd, double *Gd,
                           cudaStream_t s, const GradScratch &S) {
-    if (S.s3 && S.s2 && S.evF && concurrent_sweeps(P, S.nseg))
+    if (S.s3 && S.s2 && S.evF && concurrent_sweeps(P))
         return run_gradient_concurrent(P, ud, Fd, Gd, s, S);
     grape_status st;
     const bool exact = (P->mode == GRAPE_GRAD_EXACT);
@@ -2032,11 +2070,12 @@ grape_status build_problem(const grape_problem_desc *desc, const ProblemData &da
             cudaGetLastError();
             return bail(fail(GRAPE_ECUDA, "cudaEventCreate failed"));
         }
-    for (auto &e : P->evF)
-        if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
-            cudaGetLastError();
-            return bail(fail(GRAPE_ECUDA, "cudaEventCreate failed"));
-        }
+    for (auto *evs : {&P->evF, &P->evT})
+        for (auto &e : *evs)
+            if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+                cudaGetLastError();
+                return bail(fail(GRAPE_ECUDA, "cudaEventCreate failed"));
+            }
     *out = P;
     return GRAPE_OK;
 }
@@ -2316,7 +2355,7 @@ grape_status grape_phase_times(grape_problem_t P, double ms[4], int32_t launches
 int32_t grape_gradient_launches(grape_problem_t P) {
     if (!P) return -1;
     P = active(P);
-    return gradient_launch_count(P, P->seg, P->nseg, concurrent_sweeps(P, P->nseg));
+    return gradient_launch_count(P, P->seg, P->nseg, concurrent_sweeps(P));
 }
 
 grape_status grape_forward(grape_problem_t problem, const double *u, double *F, double *rhoT,
@@ -2502,10 +2541,11 @@ grape_status grape_gradient(grape_problem_t P, const double *u, double *F, doubl
     bool overlap = true;
     if (const char *env = std::getenv("GRAPE_TRACE_OVERLAP")) overlap = std::atoi(env) != 0;
     S.s2 = overlap ? P->s2 : nullptr;
-    if (S.s2 && concurrent_sweeps(P, P->nseg)) {
+    if (S.s2 && concurrent_sweeps(P)) {
         S.s3 = P->s3;
         S.fork3 = P->ev_fork3;
         S.evF = P->evF;
+        S.evT = P->evT;
     }
     // the sweeps run on the problem's high-priority streams, ordered after and
     // before the caller's stream; the traces on its low-priority stream
@@ -2737,7 +2777,8 @@ struct grape_batch {
     std::vector<cudaStream_t> lanes;
     std::vector<cudaEvent_t> lane_done;
     // per lane, for concurrent sweeps: the adjoint's and the traces' streams
-    // and the events that order them (kMaxChunks + 2 + kMaxChunks + 1 each)
+    // and the events that order them (kMaxChunks + 2, kMaxChunks, 1 and
+    // kMaxChunks)
     std::vector<cudaStream_t> lane_adj, lane_tr;
     std::vector<std::vector<cudaEvent_t>> lane_ev;
     cudaEvent_t fork = nullptr, ev_in = nullptr, ev_out = nullptr;
@@ -3046,7 +3087,7 @@ grape_status grape_batch_create(grape_problem_t *problems, int32_t n, int32_t n_
     bool lane_conc = false;
     if (const char *env = std::getenv("GRAPE_BATCH_CONCURRENT")) lane_conc = std::atoi(env) != 0;
     if (lane_conc) {
-        const int nev = 2 * grape_problem::kMaxChunks + 3;
+        const int nev = 3 * grape_problem::kMaxChunks + 3;
         B->lane_adj.assign(B->n_lanes, nullptr);
         B->lane_tr.assign(B->n_lanes, nullptr);
         B->lane_ev.assign(B->n_lanes, std::vector<cudaEvent_t>(nev, nullptr));
@@ -3061,12 +3102,13 @@ grape_status grape_batch_create(grape_problem_t *problems, int32_t n, int32_t n_
             }
             for (int i : B->items[l]) {
                 GradScratch &S = B->scratch[i];
-                if (!concurrent_sweeps(B->probs[i], S.nseg)) continue;
+                if (!concurrent_sweeps(B->probs[i])) continue;
                 S.s2 = B->lane_tr[l];
                 S.s3 = B->lane_adj[l];
                 S.ev = B->lane_ev[l].data();                                   // kMaxChunks + 2
                 S.evF = B->lane_ev[l].data() + grape_problem::kMaxChunks + 2;  // kMaxChunks
                 S.fork3 = B->lane_ev[l][2 * grape_problem::kMaxChunks + 2];
+                S.evT = B->lane_ev[l].data() + 2 * grape_problem::kMaxChunks + 3;  // kMaxChunks
             }
         }
     }

@@ -1,7 +1,9 @@
 """How a gradient's launches are scheduled changes no bit: the sweeps side by
-side or one after the other (GRAPE_CONCURRENT=0) in the first-order mode,
-with and without the penalty.  The exact mode's side is covered by
-test_gpu_concurrent.py; the kernels and the order of every sum are the same
+side or one after the other (GRAPE_CONCURRENT=0) in the first-order mode, and
+with checkpoints (each segment's recomputation beside its adjoint; lengths
+that divide the pulse, leave a short last segment, and one slice per segment),
+with and without the penalty.  The exact mode without checkpoints is covered
+by test_gpu_concurrent.py; the kernels and the order of every sum are the same
 in both schedules, so the results are compared for equality.
 """
 import os
@@ -60,6 +62,26 @@ def test_first_order_sweeps_side_by_side(gp, make, penalty, prec):
     if penalty:
         P.set_photon_penalty(w.phys.Q, w.phys.N, 0.3)
     out = gradients(P, w.u)
+    assert np.all(np.isfinite(out[0][1]))
+    for F, G in out[1:]:
+        assert F == out[0][0] and np.array_equal(G, out[0][1])
+
+
+@pytest.mark.parametrize("first_order", [False, True])
+@pytest.mark.parametrize("penalty", [False, True])
+@pytest.mark.parametrize("stride", [1, 6, 7, 20])
+def test_checkpointed_segments_side_by_side(gp, first_order, penalty, stride):
+    w = workloads.transmon_resonator_d120(n_slices=24)
+    out = []
+    for ck in (0, stride):
+        P = gp.GrapeProblem.from_workload(w, grad_mode=int(first_order), ckpt_stride=ck)
+        if penalty:
+            P.set_photon_penalty(w.phys.Q, w.phys.N, 0.3)
+        out += gradients(P, w.u)
+        P.set_profiling(True)
+        P.gradient(w.u)
+        counted = sum(n for _, n in P.phase_times().values())
+        assert counted <= P.gradient_launches() and (penalty or counted == P.gradient_launches())
     assert np.all(np.isfinite(out[0][1]))
     for F, G in out[1:]:
         assert F == out[0][0] and np.array_equal(G, out[0][1])
