@@ -908,10 +908,16 @@ std::vector<int> hermitian_table(int d, int ncl, int omax, int hb, int *maxwin, 
 }
 
 // The compile-time band/jump layout (the kernels' Shape) that both
-// directions' tables follow: 1 transmon x resonator (bands 0, +-1 real,
-// +-Q; three jump terms), 2 resonator drives only (bands 0, +-Q; one jump
-// term), 0 none (the kernels read the counts at run time).  Real jump tables
-// only; GRAPE_SHAPE=0 turns it off.  The arithmetic is the same either way.
+// directions' tables follow: 1 five bands of which two are real (a transmon
+// drive or a Jaynes-Cummings coupling beside the resonator drive) and up to
+// three jump terms, 2 three bands (resonator drives only) and one jump term,
+// 3 the same with two (prop_s_kernel only; a build for up to two costs the
+// one-term problems 2 to 4 %), 0 none (the kernels read the counts at run
+// time).  Further real bands are
+// multiplied as complex ones with a zero imaginary part, which changes no
+// bit.  Real jump tables only; GRAPE_SHAPE=0 turns it off.  The arithmetic
+// is the same either way (Jaynes-Cummings d=128, which has one jump term:
+// 3.27 ms on the run-time layout, 2.35 ms on this).
 int shape_id(const grape_problem *P) {
     if (!(P->variant & 1)) return 0;
     if (const char *env = std::getenv("GRAPE_SHAPE"))
@@ -919,14 +925,18 @@ int shape_id(const grape_problem *P) {
     auto is = [&](int nb, int nbr, int nt) {
         for (int dir = 0; dir < 2; ++dir) {
             const PropTables &t = P->tab[dir];
-            if (t.nb != nb || t.nbr != nbr || t.nt != nt || t.b0 != nb - 1) return false;
+            if (t.nb != nb || t.nbr < nbr || t.nt > nt || t.b0 != nb - 1) return false;
         }
         return true;
     };
     if (is(5, 2, 3)) return 1;
     if (is(3, 0, 1)) return 2;
+    if (is(3, 0, 2)) return 3;
     return 0;
 }
+
+// jump terms the kernels of a shape hold room for
+int shape_jumps(int shape, int nt) { return shape == 1 ? 3 : shape ? std::max(shape - 1, nt) : nt; }
 
 // Hermitian cluster kernel with `ncl` CTAs of `threads` threads per state:
 // sets the geometry, or GRAPE_EINVAL when the tile does not fit.  Tables
@@ -943,11 +953,11 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
     // entries; bands, jump tables; (row, column), RK coefficients, the
     // window table, the row push table (address and mbarrier per target)
     // and the neighbour addresses
+    const int sh = shape_id(P), nts = shape_jumps(sh, nt);
     const size_t base = 16 + (2 * (size_t)cu + 2 * (size_t)nb * d + 2 * (size_t)nt * d) * sizeof(double2) +
                         (size_t)cu * sizeof(int2) + 12 * sizeof(double) + tab.size() * sizeof(int) +
                         (size_t)rt_rows * (2 * ncl + 1) * sizeof(uint32_t) +
-                        (size_t)cu * (2 * nb + nt + 1) * sizeof(short);
-    const int sh = shape_id(P);
+                        (size_t)cu * (2 * nb + nts + 1) * sizeof(short);
     // Options of prop_h_kernel, each kept only when the tile still fits
     // (the same values, so the same bits, either way): the own-entry
     // coefficients cached per slice (16 B per owned entry) instead of
@@ -971,8 +981,8 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
         const size_t pbase = (one ? (small ? GRAPE_WOFF_SMALL : GRAPE_WOFF) : wbytes) + wbytes +
                              (size_t)8 * d * sizeof(double2) + tab.size() * sizeof(int) +
                              (size_t)rt_rows * (2 * ncl + 1) * sizeof(uint32_t) +
-                             (one ? 0 : (size_t)cu * (2 * sizeof(double2) + (2 + nt) * sizeof(double) + sizeof(int2) +
-                                                      (2 * (nb - 1) + 1 + nt) * sizeof(short)));
+                             (one ? 0 : (size_t)cu * (2 * sizeof(double2) + (2 + nts) * sizeof(double) + sizeof(int2) +
+                                                      (2 * (nb - 1) + 1 + nts) * sizeof(short)));
         variant = (P->variant & 1) | 2 | (sh << 2) | (one ? 16 : 0) | 32 | (small ? 64 : 0);
         const cudaError_t e = P->prec == GRAPE_PREC_FP64
                                   ? grape_prepare_prop_f64(variant, (size_t)max_smem, 16)
@@ -1151,7 +1161,7 @@ grape_status choose_geometry_grid(grape_problem *P, bool geometry_only) {
     // tables stay in global memory)
     const size_t base = ((size_t)(maxwin + 1) + 2 * (size_t)cu + (size_t)nb * d) * sizeof(double2) +
                         (size_t)cu * sizeof(int2) + 12 * sizeof(double) + tab.size() * sizeof(int) +
-                        (size_t)cu * (2 * nb + nt + 1) * sizeof(short);
+                        (size_t)cu * (2 * nb + shape_jumps(shape_id(P), nt) + 1) * sizeof(short);
     bool want_fold = true, want_jc = variant != 0;
     if (const char *env = std::getenv("GRAPE_FOLD")) want_fold = std::atoi(env) != 0;
     if (const char *env = std::getenv("GRAPE_JCACHE")) want_jc = want_jc && std::atoi(env) != 0;

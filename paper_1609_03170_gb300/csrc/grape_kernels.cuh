@@ -374,7 +374,8 @@ __device__ __forceinline__ typename Num::val diag_coef(int i, int j, int d, cons
 }
 
 // Band and jump layout known at compile time (NB bands including the
-// offset-0 band, which is last; the first NBR are real; NT jump terms), so
+// offset-0 band, which is last; the first NBR are real; at most NT jump
+// terms, t.nt of them in use), so
 // the per-entry loops unroll and the neighbour indices can live in
 // registers; ShapeAny reads the counts from the tables at run time.  The
 // host picks a shape only when both directions' tables match it.
@@ -383,8 +384,10 @@ struct Shape {
     static constexpr int NB = NB_, NBR = NBR_, NT = NT_;
 };
 using ShapeAny = Shape<0, 0, 0>;
-using ShapeT = Shape<5, 2, 3>;   // transmon x resonator: bands 0, +-1 (real drive), +-Q; jumps a, b, b^dag b
+using ShapeT = Shape<5, 2, 3>;   // transmon x resonator: bands 0, +-1 (real drive) or +-(Q-1) (Jaynes-Cummings
+                                 // coupling), +-Q; up to three jump terms
 using ShapeR = Shape<3, 0, 1>;   // resonator drives only: bands 0, +-Q; jump a
+using ShapeD = Shape<3, 0, 2>;   // the same with a second jump term (dephasing)
 template <class SH> __device__ __forceinline__ int sh_nb(const PropTables &t) { return SH::NB ? SH::NB : t.nb; }
 template <class SH> __device__ __forceinline__ int sh_nt(const PropTables &t) { return SH::NB ? SH::NT : t.nt; }
 
@@ -445,7 +448,8 @@ __device__ __forceinline__ typename Num::val lindblad_h_at(const typename Num::s
     auto each_jump = [&](auto &&term) {
         if constexpr (SH::NB > 0) {
 #pragma unroll
-            for (int q = 0; q < SH::NT; ++q) term(q);
+            for (int q = 0; q < SH::NT; ++q)
+                if (q < t.nt) term(q);
         } else {
 #pragma unroll 1
             for (int q = 0; q < nt; ++q) term(q);
@@ -1105,7 +1109,7 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const Pro
         }
         put(2 * NBO, own);
         int t = 0;
-        for (int q = 0; q < SH::NT; ++q) {
+        for (int q = 0; q < p.tab.nt; ++q) {
             if ((p.tab.jdiag >> q) & 1) continue;
             const int r = i + p.tab.joL[q], c = j + p.tab.joR[q];
             put(2 * NBO + 1 + t, (r >= 0 && r < d && c >= 0 && c < d) ? ofs[r - wr0] + (c - cs_of(r, hb)) : zs);
@@ -1113,13 +1117,13 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const Pro
         }
         for (; t < SH::NT; ++t) put(2 * NBO + 1 + t, zs);
     };
-    const int njt = SH::NT - __popc(p.tab.jdiag);                 // jump terms with an offset
+    const int njt = p.tab.nt - __popc(p.tab.jdiag);               // jump terms with an offset
     auto own_coef = [&](int i, int j, int tbr) {
         return diag_coef<Num, true>(i, j, d, p.tab, b0cur + tbr * d, vL, vR, nullptr);
     };
     auto jump_coefs = [&](int i, int j, auto &&put) {
         int t = 0;
-        for (int q = 0; q < SH::NT; ++q) {
+        for (int q = 0; q < p.tab.nt; ++q) {
             if ((p.tab.jdiag >> q) & 1) continue;
             put(t, jump_real<Num, false>(p.tab, q, i, j, d, vL, vR, nullptr));
             ++t;
@@ -2354,8 +2358,9 @@ __global__ void __launch_bounds__(256) expand_kernel(const void *src_v, double2 
 
 // ------------------------------------------------------------------ launchers
 // `variant`: bit 0 the jump tables are real; bit 1 Hermitian (upper-triangle)
-// kernel; bits 2-3 the band/jump shape (0 from the tables, 1 ShapeT, 2 ShapeR;
-// only with real jump tables); bit 5 prop_s_kernel (with a shape), bit 4 its
+// kernel; bits 2-3 the band/jump shape (0 from the tables, 1 ShapeT, 2 ShapeR,
+// 3 ShapeD, which the other kernels read from the tables; only with real jump
+// tables); bit 5 prop_s_kernel (with a shape), bit 4 its
 // build for one entry per thread, bit 6 with the windows GRAPE_WOFF_SMALL apart.
 using PropKernel = void (*)(const PropArgs);
 
@@ -2369,8 +2374,11 @@ PropKernel prop_kernel_for(int variant) {
         if (shape == 1)
             return !one ? prop_s_kernel<Num, ShapeT, 0>
                         : small ? prop_s_kernel<Num, ShapeT, GRAPE_WOFF_SMALL> : prop_s_kernel<Num, ShapeT, GRAPE_WOFF>;
-        return !one ? prop_s_kernel<Num, ShapeR, 0>
-                    : small ? prop_s_kernel<Num, ShapeR, GRAPE_WOFF_SMALL> : prop_s_kernel<Num, ShapeR, GRAPE_WOFF>;
+        if (shape == 2)
+            return !one ? prop_s_kernel<Num, ShapeR, 0>
+                        : small ? prop_s_kernel<Num, ShapeR, GRAPE_WOFF_SMALL> : prop_s_kernel<Num, ShapeR, GRAPE_WOFF>;
+        return !one ? prop_s_kernel<Num, ShapeD, 0>
+                    : small ? prop_s_kernel<Num, ShapeD, GRAPE_WOFF_SMALL> : prop_s_kernel<Num, ShapeD, GRAPE_WOFF>;
     }
     if (realj && shape == 1) return prop_h_kernel<Num, true, ShapeT>;
     if (realj && shape == 2) return prop_h_kernel<Num, true, ShapeR>;
