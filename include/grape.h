@@ -202,10 +202,9 @@ grape_status grape_problem_set_penalty(grape_problem_t problem, const double *di
  * tile for that part too when it fits there.  Errors: GRAPE_EINVAL (values out of range, a
  * grid-kernel problem, or a tile whose state window does not fit in shared
  * memory or of which no cluster can be resident; the tile is unchanged),
- * GRAPE_ECUDA.  The tile chosen at create is the widest useful cluster
- * (shortest stage latency) with 512 threads per CTA or, when one CTA holds
- * a whole state on the Hermitian kernel, the state's upper entries
- * rounded up to whole warps (at least 64 threads). */
+ * GRAPE_ECUDA.  The tile chosen at create is the one of shortest stage
+ * latency: about 128 to 160 entries per CTA up to 16 CTAs, threads for the
+ * owned entries rounded up to whole warps (at least 64). */
 grape_status grape_problem_set_tile(grape_problem_t problem, int32_t cluster, int32_t threads);
 
 /* Which propagation kernel the problem runs on: 0 = Hermitian cluster kernel

@@ -1065,9 +1065,29 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
     return GRAPE_OK;
 }
 
-grape_status choose_geometry_h(grape_problem *P) {
+// The tile chosen at create.  A stage's time is its exchange (about 0.3 us
+// however few the entries) plus its entries' arithmetic, so one problem is
+// fastest spread thin: about 128 entries per CTA, 160 with five bands (the
+// pushes then cost as much as the arithmetic saved).  Measured, ms per
+// gradient of 100 slices and two states, against 512 entries per CTA: three
+// bands d=32 1.48 (1.90), d=60 1.56 (2.31), d=80 1.76 (2.38); five bands
+// d=30 1.78 (2.70), d=60 2.31 (2.93), d=90 2.42 (3.02); FP64, bound by its
+// pipe, d=60 4.16 (10.1); d=10 on two CTAs 1.51 (1.29 on one).  Not wider than
+// lets both sweeps' clusters of every state be resident (eight of 16 CTAs).
+// Threads: whole warps for the owned entries, at least 64 (a warp without
+// entries still takes part in every barrier: d=60 1.56 against 1.64 ms).
+// A problem that is only there for its full size (geometry_only) reports 512
+// entries per CTA and 512 threads, whole warps when one CTA holds the state.
+grape_status choose_geometry_h(grape_problem *P, bool geometry_only) {
     const long long NU = (long long)P->d * (P->d + 1) / 2;
-    const int start = env_cluster(std::min(16, pow2ceil((NU + 511) / 512)));
+    int start = std::min(16, pow2ceil((NU + 511) / 512));
+    if (!geometry_only) {
+        const int per = (P->prec == GRAPE_PREC_FP64 || std::max(P->tab[0].nb, P->tab[1].nb) <= 3) ? 128 : 160;
+        int wide = std::min(16, pow2ceil((NU + per - 1) / per));
+        while (wide > start && 2 * P->ns * wide > 128) wide /= 2;
+        start = wide;
+    }
+    start = env_cluster(start);
     const int variant = (P->variant & 1) | 2;
     cudaError_t e = P->prec == GRAPE_PREC_FP64 ? grape_prepare_prop_f64(variant, (size_t)max_smem_optin(P), 16)
                                                : grape_prepare_prop_df(variant, (size_t)max_smem_optin(P), 16);
@@ -1079,12 +1099,9 @@ grape_status choose_geometry_h(grape_problem *P) {
     const int nw = candidate_widths(start, widths);
     for (int wi = 0; wi < nw; ++wi) {
         const grape_status st = plan_h(P, widths[wi], GRAPE_PROP_THREADS);
-        if (st == GRAPE_OK && P->ncl == 1) {
-            // one CTA per state: whole warps for the owned entries only, so
-            // the per-stage CTA barrier waits on fewer warps (d=20: 4.15
-            // against 4.38 ms per gradient with 512 threads, same bits)
-            const int t = std::max(64, (P->cu + 31) / 32 * 32);
-            if (t < GRAPE_PROP_THREADS && plan_h(P, 1, t) != GRAPE_OK) return plan_h(P, 1, GRAPE_PROP_THREADS);
+        if (st == GRAPE_OK && (P->ncl == 1 || !geometry_only)) {
+            const int w = P->ncl, t = std::max(64, (P->cu + 31) / 32 * 32);
+            if (t < GRAPE_PROP_THREADS && plan_h(P, w, t) != GRAPE_OK) return plan_h(P, w, GRAPE_PROP_THREADS);
         }
         if (st == GRAPE_OK || st != GRAPE_EINVAL) return st;
     }
@@ -2009,7 +2026,7 @@ grape_status build_problem(const grape_problem_desc *desc, const ProblemData &da
     for (const Ops &o : data.sets)
         for (const Bands &B : o.Ak) P->dconst = P->dconst && !B.count(0);
     if (kern != "grid" && herm) {
-        st = choose_geometry_h(P);
+        st = choose_geometry_h(P, geometry_only);
         if (st != GRAPE_OK && st != GRAPE_EINVAL) return bail(st);
         placed = (st == GRAPE_OK);
     }
