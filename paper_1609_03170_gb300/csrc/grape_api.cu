@@ -1476,8 +1476,8 @@ grape_status trace_tiles(grape_problem *P, TraceArgs *t) {
     // one CTA per SM (a 108 KB budget, 4 buffers at d=120, measured 7 % slower)
     int nbuf = 0;
     for (int n = 4; n >= 2 && !nbuf; --n)
-        if (trace_tile_smem(n, kcap) <= 104 * 1024) nbuf = n;
-    if (!nbuf && trace_tile_smem(2, kcap) + 4096 <= (size_t)max_smem_optin(P)) nbuf = 2;
+        if (trace_tile_smem(n, kcap, t->ncb) <= 104 * 1024) nbuf = n;
+    if (!nbuf && trace_tile_smem(2, kcap, t->ncb) + 4096 <= (size_t)max_smem_optin(P)) nbuf = 2;
     if (!nbuf) return GRAPE_OK;
     int4 *dblk = nullptr, *drun = nullptr;
     uint4 *dnb = nullptr;
@@ -1931,6 +1931,33 @@ grape_status build_problem(const grape_problem_desc *desc, const ProblemData &da
                 for (const auto &kv : B)
                     for (const cplx &c : kv.second) cbv.push_back(make_double2(c.real(), c.imag()));
         tr.ndo = (int)doidx.size();
+        // the part of an offset's products that its band values ask for: Im
+        // (H S) needs im S where H is real and re S where it is imaginary.
+        // Offsets that need both come first, at least two of them
+        {
+            std::vector<char> re(tr.ndo, 0), im(tr.ndo, 0);      // some value has a real / imaginary part
+            for (const Ops &o : data.sets)
+                for (const Bands &B : o.Tk)
+                    for (const auto &kv : B)
+                        for (const cplx &c : kv.second) {
+                            re[doidx[kv.first]] |= c.real() != 0.0;
+                            im[doidx[kv.first]] |= c.imag() != 0.0;
+                        }
+            std::vector<int> order(tr.ndo);
+            for (int i = 0; i < tr.ndo; ++i) order[i] = i;
+            std::stable_sort(order.begin(), order.end(),
+                             [&](int a, int b) { return (re[a] && im[a]) > (re[b] && im[b]); });
+            tr.n2 = 0;
+            for (int i = 0; i < tr.ndo; ++i) tr.n2 += re[i] && im[i];
+            tr.n2 = std::min(tr.ndo, std::max(2, tr.n2));
+            std::vector<int> place(tr.ndo), off(tr.do_off, tr.do_off + tr.ndo);
+            for (int i = 0; i < tr.ndo; ++i) {
+                place[order[i]] = i;
+                tr.do_off[i] = off[order[i]];
+                if (i >= tr.n2 && im[order[i]]) tr.single_re |= 1 << i;
+            }
+            for (int c = 0; c < tr.ncb; ++c) tr.cb_do[c] = place[tr.cb_do[c]];
+        }
         tr.d = d;
         tr.R = desc->n_controls;
         // sandwich terms gamma c y c^+ of the rate-controlled dissipators: the

@@ -129,7 +129,9 @@ struct TraceArgs {
     int ncb, ndo;
     int cb_k[GRAPE_MAXCB];      // control of band entry c
     int cb_do[GRAPE_MAXCB];     // distinct-offset index of band entry c
-    int do_off[GRAPE_MAXDO];    // distinct offsets
+    int do_off[GRAPE_MAXDO];    // distinct offsets, the n2 whose products need both parts first
+    int n2;                     // (the rest need the real part when bit oi of single_re is set,
+    int single_re;              // else the imaginary part)
     const void *cb_s;           // [ncb][d]  Hk_b[m], storage format of the number type
     long long cb_stride, st_stride;   // entries between the states' band and sandwich tables
                                       // (0: shared by all states)
@@ -156,7 +158,7 @@ struct TraceArgs {
     // staged trace (packed storage, nst == 0, ndo <= 4): per 256-entry block
     // b of the packed triangle, the runs of K its entries' neighbours fall in
     // are copied to shared memory with Y's block, per pair, into nbuf buffers
-    // of 256 + kcap entries
+    // of 256 + kcap + 1 entries
     int tile, kcap, nbuf;
     const int4 *tblk;               // [blocks]: first run, run count, K entries copied
     const int4 *trun;               // runs: packed start, length, offset in the buffer's K part
@@ -168,9 +170,9 @@ struct TraceArgs {
 };
 
 // dynamic shared memory of the staged trace kernel: 8 mbarriers, the
-// per-band sums [8][256] (16 B each), nbuf buffers of 256 + kcap entries
-inline size_t trace_tile_smem(int nbuf, int kcap) {
-    return 64 + (size_t)GRAPE_MAXCB * 256 * 16 + (size_t)nbuf * (256 + kcap) * 16;
+// per-band sums [ncb][256] (16 B each), nbuf buffers of 256 + kcap + 1 entries
+inline size_t trace_tile_smem(int nbuf, int kcap, int ncb) {
+    return 64 + (size_t)ncb * 256 * 16 + (size_t)nbuf * (256 + kcap + 1) * 16;
 }
 
 // Launchers, one set per number type: _f64 native FP64, _df double-float.

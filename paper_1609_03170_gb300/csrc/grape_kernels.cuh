@@ -1939,11 +1939,20 @@ __global__ void __launch_bounds__(256) trace_packed_kernel(const TraceArgs p) {
     trace_store<Num, true>(p, Z, Zs, row, split);
 }
 
+// S = sum conj(Y) K from its lane sums R = sum (K.re Y.re, K.im Y.im) and
+// I = sum (K.re Y.im, K.im Y.re), K's mirror read when cj; T = sum Y conj(K)
+// is its conjugate.
+template <class Num>
+__device__ __forceinline__ typename Num::val lane_sums(typename Num::acc R, typename Num::acc I, bool cj, bool conj) {
+    typename Num::real_t im = Num::lanes_add(I, !cj);       // K.re Y.im -+ K.im Y.re = im Y conj(K)
+    if (!conj) im = Num::neg_real(im);
+    return Num::make(Num::lanes_add(R, cj), im);
+}
+
 // The same sums for problems without rate-controlled dissipators and with
 // at most NDO distinct control offsets: the pairs are the outer loop (each
 // Y entry is loaded once per pair) and every offset's sums stay in
-// registers.  Each sum adds the same terms in the same order as
-// trace_packed_kernel, so both give the same bits.
+// registers, the products' lanes apart until the end.
 template <class Num, int NDO>
 __global__ void __launch_bounds__(256) trace_packed_fast_kernel(const TraceArgs p) {
     using S = typename Num::store_t;
@@ -1972,7 +1981,7 @@ __global__ void __launch_bounds__(256) trace_packed_fast_kernel(const TraceArgs 
         const int i = (int)(ij & 0xffffu), j = (int)(ij >> 16);
         int x1[NDO], x2[NDO];
         bool v1[NDO], v2[NDO], cj1[NDO], cj2[NDO];
-        typename Num::acc Sa[NDO], Ta[NDO];
+        typename Num::acc R1[NDO], I1[NDO], R2[NDO], I2[NDO];
 #pragma unroll
         for (int oi = 0; oi < NDO; ++oi) {
             const int o = oi < p.ndo ? p.do_off[oi] : 0;
@@ -1983,25 +1992,33 @@ __global__ void __launch_bounds__(256) trace_packed_fast_kernel(const TraceArgs 
             cj2[oi] = v2[oi] && c2 < i;
             x1[oi] = !v1[oi] ? u : (cj1[oi] ? packed_index(j, r1, d) : packed_index(r1, j, d));
             x2[oi] = !v2[oi] ? u : (cj2[oi] ? packed_index(c2, i, d) : packed_index(i, c2, d));
-            Sa[oi] = Num::acc_zero();
-            Ta[oi] = Num::acc_zero();
+            R1[oi] = I1[oi] = R2[oi] = I2[oi] = Num::acc_zero();
         }
         const S *Yp = Yb + (row_base + state) * NU;
         const S *Kp = Kb + (row_base + state) * NU;
-#pragma unroll 4
+#pragma unroll 2
         for (long long qs = 0; qs < pps; ++qs) {
             const size_t moff = (size_t)qs * pstride;
-            const V y = Num::load(Yp[moff + u]);
+            const V y = Num::load(Yp[moff + u]), ysw = Num::swap(y);
 #pragma unroll
             for (int oi = 0; oi < NDO; ++oi) {
-                if (v1[oi]) Num::mac_conjb(Sa[oi], conj_if<Num>(Num::load(Kp[moff + x1[oi]]), cj1[oi]), y);
-                if (v2[oi]) Num::mac_conjb(Ta[oi], y, conj_if<Num>(Num::load(Kp[moff + x2[oi]]), cj2[oi]));
+                if (v1[oi]) {
+                    const V k = Num::load(Kp[moff + x1[oi]]);
+                    Num::mac_lanes(R1[oi], k, y);
+                    Num::mac_lanes(I1[oi], k, ysw);
+                }
+                if (v2[oi]) {
+                    const V k = Num::load(Kp[moff + x2[oi]]);
+                    Num::mac_lanes(R2[oi], k, y);
+                    Num::mac_lanes(I2[oi], k, ysw);
+                }
             }
         }
 #pragma unroll
         for (int oi = 0; oi < NDO; ++oi) {
             if (oi >= p.ndo) break;
-            const V Sv = Num::done(Sa[oi]), Tv = Num::done(Ta[oi]);
+            const V Sv = lane_sums<Num>(R1[oi], I1[oi], cj1[oi], false);
+            const V Tv = lane_sums<Num>(R2[oi], I2[oi], cj2[oi], true);
 #pragma unroll
             for (int c = 0; c < GRAPE_MAXCB; ++c) {
                 if (c < p.ncb && p.cb_do[c] == oi) {
@@ -2026,13 +2043,22 @@ __global__ void __launch_bounds__(256) trace_packed_fast_kernel(const TraceArgs 
 // buffer's "empty" mbarrier shows that the eight consumer warps are done with
 // its previous use.  Warps 0..7 are the consumers, thread t owning entry
 // b * 256 + t: they read its neighbour positions in the buffer from the host
-// table tnb (15-bit index, bit 15: read the conjugate of the mirror, 0xffff:
-// outside the matrix) and release the buffer warp by warp, so no CTA-wide
-// barrier stands between pairs.  Every term and the order of every sum is
-// that of the fast kernel: the same bits.  Waits are bounded: one that gives
-// up sets the error word to 3 and a shared stop flag, the CTA stops, waits
-// (bounded) for the copies it issued and writes no result (the host reports
-// GRAPE_ETIMEOUT).
+// table tnb (15-bit index, bit 15: the mirror is stored, 0xffff: outside the
+// matrix, read as the buffer's last entry, which stays zero) and release the
+// buffer warp by warp, so no CTA-wide barrier stands between pairs.  The order
+// of every sum is that of the fast kernel: the same bits.  Waits are bounded:
+// one that gives up sets the error word to 3 and a shared stop flag, the CTA
+// stops, waits (bounded) for the copies it issued and writes no result (the
+// host reports GRAPE_ETIMEOUT).
+//
+// Bound by the FP32 pipe.  Of each sum only the part that the control bands
+// ask for is formed: an offset whose band values are real for every control
+// needs the imaginary parts of its products only, one with imaginary values
+// the real parts; the host puts the offsets that need both first (N2 of
+// them), then N1 that need one (p.single_re: the real part).  At d=120 that
+// is 144 paired instructions per entry and pair instead of 192, and keeping
+// the products' lanes apart leaves no other arithmetic in the loop (d=120
+// gradient, whose traces the sweeps outrun: 60.6 -> 56.9 ms).
 #define GRAPE_TRACE_CONSUMERS 8
 #define GRAPE_TRACE_THREADS (32 * (GRAPE_TRACE_CONSUMERS + 1))
 
@@ -2055,8 +2081,9 @@ __device__ __forceinline__ bool mbar_wait_or_stop(uint32_t mbar, uint32_t parity
     }
 }
 
-template <class Num, int NDO>
+template <class Num, int N2, int N1>
 __global__ void __launch_bounds__(GRAPE_TRACE_THREADS, 2) trace_tile_kernel(const TraceArgs p) {
+    constexpr int NDO = N2 + N1;
     using S = typename Num::store_t;
     using V = typename Num::val;
     using A = typename Num::acc;
@@ -2070,12 +2097,12 @@ __global__ void __launch_bounds__(GRAPE_TRACE_THREADS, 2) trace_tile_kernel(cons
     const int pps = (int)(p.npairs / p.n_states);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nbuf = p.nbuf;
-    const int stride = 256 + p.kcap;                       // entries per buffer: Y block, then K runs
+    const int stride = 256 + p.kcap + 1;                   // entries per buffer: Y block, K runs, a zero
     const uint32_t full0 = (uint32_t)__cvta_generic_to_shared(tsm);     // [nbuf] "full" mbarriers
     const uint32_t empty0 = full0 + 32u;                                // [nbuf] "empty" mbarriers
-    A *Zsm = reinterpret_cast<A *>(tsm + 64);                           // [GRAPE_MAXCB][256]
-    S *bufs = reinterpret_cast<S *>(tsm + 64 + GRAPE_MAXCB * 256 * sizeof(A));
-    const uint32_t ba0 = full0 + 64u + (uint32_t)(GRAPE_MAXCB * 256 * sizeof(A));
+    A *Zsm = reinterpret_cast<A *>(tsm + 64);                           // [ncb][256]
+    S *bufs = reinterpret_cast<S *>(tsm + 64 + p.ncb * 256 * sizeof(A));
+    const uint32_t ba0 = full0 + 64u + (uint32_t)(p.ncb * 256 * sizeof(A));
     const int nblk_all = (NU + 255) / 256;
     const int b0 = chunk * p.epc;
     const int nblk = max(0, min(p.epc, nblk_all - b0));
@@ -2097,7 +2124,8 @@ __global__ void __launch_bounds__(GRAPE_TRACE_THREADS, 2) trace_tile_kernel(cons
         s_stop = 0;
     }
     if (tid < 256)
-        for (int c = 0; c < GRAPE_MAXCB; ++c) Zsm[c * 256 + tid] = Num::acc_zero();
+        for (int c = 0; c < p.ncb; ++c) Zsm[c * 256 + tid] = Num::acc_zero();
+    if (tid < nbuf) bufs[(tid + 1) * stride - 1] = Num::store(Num::zero());
     __syncthreads();
 
     int issued = 0;                                  // producer: steps whose copies it issued
@@ -2156,20 +2184,21 @@ __global__ void __launch_bounds__(GRAPE_TRACE_THREADS, 2) trace_tile_kernel(cons
             const unsigned w16[8] = {nb.x & 0xffffu, nb.x >> 16, nb.y & 0xffffu, nb.y >> 16,
                                      nb.z & 0xffffu, nb.z >> 16, nb.w & 0xffffu, nb.w >> 16};
             int x1[NDO], x2[NDO];
-            bool v1[NDO], v2[NDO], cj1[NDO], cj2[NDO];
-            A Sa[NDO], Ta[NDO];
+            bool cj1[NDO], cj2[NDO];
+            // lane sums of the products with Y as it is (the first N2
+            // offsets) and with its parts swapped (N1: as single_re says)
+            A R1[N2], R2[N2], I1[NDO], I2[NDO];
 #pragma unroll
             for (int oi = 0; oi < NDO; ++oi) {
                 const unsigned a = w16[2 * oi], c = w16[2 * oi + 1];
-                v1[oi] = valid && a != 0xffffu;
-                v2[oi] = valid && c != 0xffffu;
                 cj1[oi] = (a & 0x8000u) != 0u;
                 cj2[oi] = (c & 0x8000u) != 0u;
-                x1[oi] = 256 + (v1[oi] ? (int)(a & 0x7fffu) : 0);
-                x2[oi] = 256 + (v2[oi] ? (int)(c & 0x7fffu) : 0);
-                Sa[oi] = Num::acc_zero();
-                Ta[oi] = Num::acc_zero();
+                x1[oi] = a != 0xffffu ? 256 + (int)(a & 0x7fffu) : stride - 1;
+                x2[oi] = c != 0xffffu ? 256 + (int)(c & 0x7fffu) : stride - 1;
+                I1[oi] = I2[oi] = Num::acc_zero();
             }
+#pragma unroll
+            for (int oi = 0; oi < N2; ++oi) R1[oi] = R2[oi] = Num::acc_zero();
 #pragma unroll 1
             for (int q = 0; q < pps; ++q) {
                 const bool ok = mbar_wait_or_stop(full0 + 8u * buf, (uint32_t)(use & 1), limit, &s_stop);
@@ -2182,11 +2211,21 @@ __global__ void __launch_bounds__(GRAPE_TRACE_THREADS, 2) trace_tile_kernel(cons
                     break;
                 }
                 if (valid) {
-                    const V y = Num::load(Ys[tid]);
+                    const V y = Num::load(Ys[tid]), ysw = Num::swap(y);
 #pragma unroll
                     for (int oi = 0; oi < NDO; ++oi) {
-                        if (v1[oi]) Num::mac_conjb(Sa[oi], conj_if<Num>(Num::load(Ys[x1[oi]]), cj1[oi]), y);
-                        if (v2[oi]) Num::mac_conjb(Ta[oi], y, conj_if<Num>(Num::load(Ys[x2[oi]]), cj2[oi]));
+                        const V k1 = Num::load(Ys[x1[oi]]), k2 = Num::load(Ys[x2[oi]]);
+                        if (oi < N2) {
+                            Num::mac_lanes(R1[oi], k1, y);
+                            Num::mac_lanes(R2[oi], k2, y);
+                            Num::mac_lanes(I1[oi], k1, ysw);
+                            Num::mac_lanes(I2[oi], k2, ysw);
+                        } else {
+                            const bool re = (p.single_re >> oi) & 1;
+                            const V op = re ? y : ysw;
+                            Num::mac_lanes(I1[oi], k1, op);
+                            Num::mac_lanes(I2[oi], k2, op);
+                        }
                     }
                 }
                 __syncwarp();
@@ -2204,7 +2243,12 @@ __global__ void __launch_bounds__(GRAPE_TRACE_THREADS, 2) trace_tile_kernel(cons
 #pragma unroll
                 for (int oi = 0; oi < NDO; ++oi) {
                     if (oi >= p.ndo) break;
-                    const V Sv = Num::done(Sa[oi]), Tv = Num::done(Ta[oi]);
+                    const bool re = oi >= N2 && ((p.single_re >> oi) & 1);
+                    const A z0 = Num::acc_zero();
+                    const A Ra = oi < N2 ? R1[oi < N2 ? oi : 0] : re ? I1[oi] : z0;
+                    const A Rb = oi < N2 ? R2[oi < N2 ? oi : 0] : re ? I2[oi] : z0;
+                    const V Sv = lane_sums<Num>(Ra, re ? z0 : I1[oi], cj1[oi], false);
+                    const V Tv = lane_sums<Num>(Rb, re ? z0 : I2[oi], cj2[oi], true);
 #pragma unroll
                     for (int c = 0; c < GRAPE_MAXCB; ++c) {
                         if (c < p.ncb && p.cb_do[c] == oi) {
@@ -2230,7 +2274,7 @@ __global__ void __launch_bounds__(GRAPE_TRACE_THREADS, 2) trace_tile_kernel(cons
     }
     A Z[GRAPE_MAXCB];
 #pragma unroll
-    for (int c = 0; c < GRAPE_MAXCB; ++c) Z[c] = tid < 256 ? Zsm[c * 256 + tid] : Num::acc_zero();
+    for (int c = 0; c < GRAPE_MAXCB; ++c) Z[c] = tid < 256 && c < p.ncb ? Zsm[c * 256 + tid] : Num::acc_zero();
     A Z_unused[GRAPE_MAXST];                        // no sandwich terms
     trace_store<Num, false>(p, Z, Z_unused, row, split, GRAPE_TRACE_CONSUMERS);
 }
@@ -2483,8 +2527,10 @@ cudaError_t launch_trace(const TraceArgs &p, cudaStream_t s) {
     if (p.packed) {
         const int grid = p.n_rows * max(1, p.nsplit);
         if (p.tile && p.nst == 0 && p.ndo <= 4) {
-            const size_t smem = trace_tile_smem(p.nbuf, p.kcap);
-            void (*k)(const TraceArgs) = p.ndo <= 2 ? trace_tile_kernel<Num, 2> : trace_tile_kernel<Num, 4>;
+            const size_t smem = trace_tile_smem(p.nbuf, p.kcap, p.ncb);
+            void (*k)(const TraceArgs) = p.ndo <= 2   ? trace_tile_kernel<Num, 2, 0>
+                                         : p.n2 <= 2 ? trace_tile_kernel<Num, 2, 2>
+                                                     : trace_tile_kernel<Num, 4, 0>;
             const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
             k<<<grid, GRAPE_TRACE_THREADS, smem, s>>>(p);

@@ -130,6 +130,14 @@ struct NumD {
         c.re = fma(a.re, b.re, fma(a.im, b.im, c.re));
         c.im = fma(a.im, b.re, fma(-a.re, b.im, c.im));
     }
+    // lane-wise sums of a conj(b) or b conj(a) (see NumF)
+    static __device__ __forceinline__ val swap(val a) { return {a.im, a.re}; }
+    static __device__ __forceinline__ void mac_lanes(acc &c, val a, val b) {
+        c.re = fma(a.re, b.re, c.re);
+        c.im = fma(a.im, b.im, c.im);
+    }
+    static __device__ __forceinline__ real_t lanes_add(acc c, bool neg) { return neg ? c.re - c.im : c.re + c.im; }
+    static __device__ __forceinline__ val make(real_t re, real_t im) { return {re, im}; }
     static __device__ __forceinline__ val done(acc c) { return {c.re, c.im}; }
     static __device__ __forceinline__ val raw(acc c) { return {c.re, c.im}; }
     static __device__ __forceinline__ acc acc_minus_i(acc c) { return {c.im, -c.re}; }
@@ -289,6 +297,25 @@ struct NumF {
     static __device__ __forceinline__ void mac_conjb(acc &c, val a, val b) {
         p_lacc_fma(c.h, c.l, a.h, a.l, p_bx(b.h), p_bx(b.l));
         p_lacc_fma(c.h, c.l, make_float2(a.h.y, -a.h.x), make_float2(a.l.y, -a.l.x), p_by(b.h), p_by(b.l));
+    }
+    // The real products of a complex one kept in separate lanes until the
+    // end: with c += (a.re b.re, a.im b.im) over many pairs, re(a conj b) is
+    // the sum of c's lanes, and with b's parts swapped im(a conj b) the
+    // difference - no operand is rotated, broadcast or negated in the loop.
+    static __device__ __forceinline__ val swap(val a) {
+        return {make_float2(a.h.y, a.h.x), make_float2(a.l.y, a.l.x)};
+    }
+    static __device__ __forceinline__ void mac_lanes(acc &c, val a, val b) {
+        p_lacc_fma(c.h, c.l, a.h, a.l, b.h, b.l);
+    }
+    // c's first lane plus (neg: minus) the second
+    static __device__ __forceinline__ real_t lanes_add(acc c, bool neg) {
+        const float yh = neg ? -c.h.y : c.h.y, yl = neg ? -c.l.y : c.l.y;
+        const ff t = two_sum(c.h.x, yh);
+        return two_sum(t.h, __fadd_rn(t.l, __fadd_rn(c.l.x, yl)));
+    }
+    static __device__ __forceinline__ val make(real_t re, real_t im) {
+        return {make_float2(re.h, im.h), make_float2(re.l, im.l)};
     }
     static __device__ __forceinline__ val done(acc c) {
         val v;
