@@ -977,13 +977,16 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
     bool found = false, fold = false, defer = false, jcache = false, raw = false;
     if (sh && want_fold && want_jc && !want_defer) {
         const size_t wbytes = (size_t)(maxwin + 1) * sizeof(double2);
-        const bool one = cu <= threads && wbytes <= GRAPE_WOFF, small = one && wbytes <= GRAPE_WOFF_SMALL;
+        // one entry per thread, or two; any number with the data in shared memory
+        const bool two = cu > threads && cu <= 2 * threads && threads <= GRAPE_TWO_THREADS && wbytes <= GRAPE_WOFF;
+        const bool one = two || (cu <= threads && wbytes <= GRAPE_WOFF);
+        const bool small = one && !two && wbytes <= GRAPE_WOFF_SMALL;
         const size_t pbase = (one ? (small ? GRAPE_WOFF_SMALL : GRAPE_WOFF) : wbytes) + wbytes +
                              (size_t)8 * d * sizeof(double2) + tab.size() * sizeof(int) +
                              (size_t)rt_rows * (2 * ncl + 1) * sizeof(uint32_t) +
                              (one ? 0 : (size_t)cu * (2 * sizeof(double2) + (2 + nts) * sizeof(double) + sizeof(int2) +
                                                       (2 * (nb - 1) + 1 + nts) * sizeof(short)));
-        variant = (P->variant & 1) | 2 | (sh << 2) | (one ? 16 : 0) | 32 | (small ? 64 : 0);
+        variant = (P->variant & 1) | 2 | (sh << 2) | (one ? 16 : 0) | 32 | (small ? 64 : 0) | (two ? 128 : 0);
         const cudaError_t e = P->prec == GRAPE_PREC_FP64
                                   ? grape_prepare_prop_f64(variant, (size_t)max_smem, 16)
                                   : grape_prepare_prop_df(variant, (size_t)max_smem, 16);
@@ -1075,7 +1078,8 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
 // pipe, d=60 4.16 (10.1); d=10 on two CTAs 1.51 (1.29 on one).  Not wider than
 // lets both sweeps' clusters of every state be resident (eight of 16 CTAs).
 // Threads: whole warps for the owned entries, at least 64 (a warp without
-// entries still takes part in every barrier: d=60 1.56 against 1.64 ms).
+// entries still takes part in every barrier: d=60 1.56 against 1.64 ms); for
+// 513 to 768 entries half as many threads with two entries each.
 // A problem that is only there for its full size (geometry_only) reports 512
 // entries per CTA and 512 threads, whole warps when one CTA holds the state.
 grape_status choose_geometry_h(grape_problem *P, bool geometry_only) {
@@ -1100,7 +1104,10 @@ grape_status choose_geometry_h(grape_problem *P, bool geometry_only) {
     for (int wi = 0; wi < nw; ++wi) {
         const grape_status st = plan_h(P, widths[wi], GRAPE_PROP_THREADS);
         if (st == GRAPE_OK && (P->ncl == 1 || !geometry_only)) {
-            const int w = P->ncl, t = std::max(64, (P->cu + 31) / 32 * 32);
+            const int w = P->ncl;
+            int t = P->cu;                       // threads that own entries
+            if (!geometry_only && t > GRAPE_PROP_THREADS && t <= 2 * GRAPE_TWO_THREADS) t = (t + 1) / 2;
+            t = std::max(64, (t + 31) / 32 * 32);
             if (t < GRAPE_PROP_THREADS && plan_h(P, w, t) != GRAPE_OK) return plan_h(P, w, GRAPE_PROP_THREADS);
         }
         if (st == GRAPE_OK || st != GRAPE_EINVAL) return st;

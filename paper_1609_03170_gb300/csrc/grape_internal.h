@@ -14,6 +14,7 @@
 #define GRAPE_PROP_THREADS 512   // threads per CTA of the propagation kernel
 #define GRAPE_WOFF_SMALL 8192    // bytes between prop_s_kernel's two windows, one entry per thread
 #define GRAPE_WOFF 32768
+#define GRAPE_TWO_THREADS 384    // most threads per CTA of prop_s_kernel with two entries per thread
 
 // One direction of the Lindblad action in the common form
 //   W = -i (A X - X A^+) + sum_t vL_t[i] conj(vR_t[j]) X[i + oL_t][j + oR_t]

@@ -950,8 +950,16 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
 // next slice are built at the last stage of a slice and published by the same
 // arrival, so the rebuild needs no barrier; A0 and every A_k stay in shared
 // memory (p.raw) and the slice's controls are fetched at its first stage.
-// WOFF > 0: at most one entry per thread (cu <= threads) and windows within
-// WOFF bytes; WOFF = 0: any tile, with the entries' data in shared memory.
+// WOFF > 0: at most EPT entries per thread (cu <= EPT threads), all in
+// registers, and windows within WOFF bytes; WOFF = 0: any tile, with the
+// entries' data in shared memory.  Two entries per thread (at most
+// GRAPE_TWO_THREADS threads, for their registers) are for tiles of more than
+// 512 entries, the most one CTA can hold with one per thread, against
+// WOFF = 0: the checkpointed gradient of one 150 x 150 state (708 entries,
+// three bands) 69.5 -> 56.2 ms, Jaynes-Cummings d=128 (516, five bands) 2.34
+// -> 2.07 ms.  Where one per thread fits it is faster (454 entries: 1.61
+// against 1.88 us per stage): more warps hide more than two independent sums
+// in one thread do.
 //
 // Shared memory: buf0, buf1 [maxwin + 1] (buf1 at WOFF when that is set); the
 // band rows [2][d][48 B]; the offset-0 band [2][d]; raw [1 + R][nb][d] when
@@ -995,8 +1003,9 @@ struct alignas(16) RealPair {
     R u, t;
 };
 
-template <class Num, class SH, int WOFF>
-__global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const PropArgs p) {
+template <class Num, class SH, int WOFF, int EPT>
+__global__ void __launch_bounds__(EPT == 2 ? GRAPE_TWO_THREADS : GRAPE_PROP_THREADS, 1)
+    prop_s_kernel(const PropArgs p) {
     using S = typename Num::store_t;
     using V = typename Num::val;
     using A = typename Num::acc;
@@ -1157,42 +1166,53 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const Pro
     }
     __syncthreads();                              // band rows and push table
 
-    // ONE: the thread's entry in registers
-    const bool mine = tid < cnt;
-    int2 ij1 = make_int2(0, 0);
-    uint32_t ad[NA];                              // neighbours, byte offsets in a window
-    R tc[NTL];
-    V x1 = Num::zero(), a1 = Num::zero();         // base value, RK accumulator
-    uint32_t pa[2] = {0u, 0u}, pm[2] = {0u, 0u};  // push targets: (i, j) in a peer's buf0, its mbarrier
-    int npeer = 0;
+    // ONE: the thread's entries tid, tid + nth (EPT of them) in registers; an
+    // entry it does not have reads the zero slot and stores nothing
+    bool mine[EPT];                               // has it
+    int2 ij1[EPT];
+    uint32_t ad[EPT][NA];                         // neighbours, byte offsets in a window
+    R tc[EPT][NTL];
+    V x1[EPT], a1[EPT];                           // base value, RK accumulator
+    uint32_t pa[EPT][2], pm[EPT][2];              // push targets: (i, j) in a peer's buf0, its mbarrier
+    int npeer[EPT];
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) {
+        mine[e] = tid + e * nth < cnt;
+        ij1[e] = make_int2(0, 0);
+        x1[e] = a1[e] = Num::zero();
+        pa[e][0] = pa[e][1] = pm[e][0] = pm[e][1] = 0u;
+        npeer[e] = 0;
+    }
     if constexpr (ONE) {
 #pragma unroll
-        for (int k = 0; k < NA; ++k) ad[k] = (uint32_t)p.maxwin * (uint32_t)sizeof(S);
+        for (int e = 0; e < EPT; ++e) {
 #pragma unroll
-        for (int t = 0; t < NTL; ++t) tc[t] = Num::real_const(0.0);
-        if (mine) {
-            ij1 = upper_entry(u0 + tid, d);
+            for (int k = 0; k < NA; ++k) ad[e][k] = (uint32_t)p.maxwin * (uint32_t)sizeof(S);
+#pragma unroll
+            for (int t = 0; t < NTL; ++t) tc[e][t] = Num::real_const(0.0);
+            if (!mine[e]) continue;
+            ij1[e] = upper_entry(u0 + tid + e * nth, d);
             // (compile-time indices: the arrays stay in registers)
-            slots(ij1.x, ij1.y, [&](int k, int slot) {
+            slots(ij1[e].x, ij1[e].y, [&](int k, int slot) {
 #pragma unroll
                 for (int q = 0; q < NA; ++q)
-                    if (q == k) ad[q] = (uint32_t)slot * (uint32_t)sizeof(S);
+                    if (q == k) ad[e][q] = (uint32_t)slot * (uint32_t)sizeof(S);
             });
-            jump_coefs(ij1.x, ij1.y, [&](int t, R c) {
+            jump_coefs(ij1[e].x, ij1[e].y, [&](int t, R c) {
 #pragma unroll
                 for (int q = 0; q < SH::NT; ++q)
-                    if (q == t) tc[2 + q] = c;
+                    if (q == t) tc[e][2 + q] = c;
             });
-            const V dij = own_coef(ij1.x, ij1.y, 0);
-            tc[0] = Num::re(dij);
-            tc[1] = Num::im(dij);
-            const uint32_t *e = rowtab + (ij1.x - rfirst) * rstride;
-            npeer = (int)e[0] - 1;
+            const V dij = own_coef(ij1[e].x, ij1[e].y, 0);
+            tc[e][0] = Num::re(dij);
+            tc[e][1] = Num::im(dij);
+            const uint32_t *r = rowtab + (ij1[e].x - rfirst) * rstride;
+            npeer[e] = (int)r[0] - 1;
 #pragma unroll
             for (int t = 0; t < 2; ++t)
-                if (t < npeer) {
-                    pa[t] = e[1 + 2 * t] + (uint32_t)ij1.y * (uint32_t)sizeof(S);
-                    pm[t] = e[2 + 2 * t];
+                if (t < npeer[e]) {
+                    pa[e][t] = r[1 + 2 * t] + (uint32_t)ij1[e].y * (uint32_t)sizeof(S);
+                    pm[e][t] = r[2 + 2 * t];
                 }
         }
     } else {
@@ -1206,7 +1226,9 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const Pro
             tcs[cu + li] = Num::im(dij);
         }
     }
-    const bool mirror1 = mine && ij1.y > ij1.x && ij1.y - ij1.x <= hb;
+    bool mirror1[EPT];                            // the entry's mirror lies in a window too
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) mirror1[e] = mine[e] && ij1[e].y > ij1[e].x && ij1[e].y - ij1[e].x <= hb;
     cluster_sync_all();   // every CTA runs, windows zeroed, mbarriers initialised, tables built
     // bytes peers push into this CTA's window each stage
     const uint32_t expect = (uint32_t)kfl[2 * d + rank] * (uint32_t)sizeof(S);
@@ -1235,10 +1257,12 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const Pro
     // the initial stage input (window 0)
     if (clu && tid == 0) mbar_expect(mbar_sa, expect);
     if constexpr (ONE) {
-        if (mine) {
-            x1 = Num::load(x_in[soff + (size_t)ij1.x * d + ij1.y]);
-            push_rows(ij1, 0, Num::scale(RK::g(p, 0), x1));
-        }
+#pragma unroll
+        for (int e = 0; e < EPT; ++e)
+            if (mine[e]) {
+                x1[e] = Num::load(x_in[soff + (size_t)ij1[e].x * d + ij1[e].y]);
+                push_rows(ij1[e], 0, Num::scale(RK::g(p, 0), x1[e]));
+            }
     } else {
         for (int li = tid; li < cnt; li += nth) {
             const V x = Num::load(x_in[soff + (size_t)rc[li].x * d + rc[li].y]);
@@ -1266,7 +1290,9 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const Pro
     auto store_bound = [&]() {
         S *dst = bnd + ((size_t)bslot * p.n_states) * d2 + soff;
         if constexpr (ONE) {
-            if (mine) store_herm<Num>(dst, d, ij1.x, ij1.y, Num::store(x1));
+#pragma unroll
+            for (int e = 0; e < EPT; ++e)
+                if (mine[e]) store_herm<Num>(dst, d, ij1[e].x, ij1[e].y, Num::store(x1[e]));
         } else {
             for (int li = tid; li < cnt; li += nth) store_herm<Num>(dst, d, rc[li].x, rc[li].y, xs[li]);
         }
@@ -1341,26 +1367,43 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const Pro
             };
             S *std_ = st ? st + (size_t)p.store_map[s] * sset : nullptr;
             if constexpr (ONE) {
-                if (mine) {
+                if (mine[0]) {
                     if (s == 0 && dfresh) {
-                        const V dij = own_coef(ij1.x, ij1.y, tb);
-                        tc[0] = Num::re(dij);
-                        tc[1] = Num::im(dij);
+#pragma unroll
+                        for (int e = 0; e < EPT; ++e)
+                            if (mine[e]) {
+                                const V dij = own_coef(ij1[e].x, ij1[e].y, tb);
+                                tc[e][0] = Num::re(dij);
+                                tc[e][1] = Num::im(dij);
+                            }
                     }
-                    const V z = entry(ij1.x, ij1.y, [&](int k) { return ad[k]; }, [&](int t) { return tc[t]; }, x1, a1,
-                                      std_ ? std_ + tid : nullptr);
-                    const S zs = Num::store(z);
-                    *reinterpret_cast<S *>(smem_raw + ad[2 * NBO] + bo) = zs;
-                    if (npeer > 0) st_async16(pa[0] + bo, zs, pm[0] + 8u * par);
-                    if (npeer > 1) st_async16(pa[1] + bo, zs, pm[1] + 8u * par);
-                    if (npeer > 2) {
-                        const uint32_t *e = rowtab + (ij1.x - rfirst) * rstride;
-                        for (int t = 2; t < npeer; ++t)
-                            st_async16(e[1 + 2 * t] + (uint32_t)ij1.y * (uint32_t)sizeof(S) + bo, zs,
-                                       e[2 + 2 * t] + 8u * par);
+                    // the entries' values first, then all stores: nothing
+                    // orders one entry's arithmetic against the other's
+                    V z[EPT];
+#pragma unroll
+                    for (int e = 0; e < EPT; ++e) {
+                        S *dst = std_ ? std_ + tid + e * nth : nullptr;
+                        if (e > 0 && !mine[e]) dst = nullptr;
+                        z[e] = entry(ij1[e].x, ij1[e].y, [&](int k) { return ad[e][k]; }, [&](int t) { return tc[e][t]; },
+                                     x1[e], a1[e], dst);
                     }
-                    if (mirror1)
-                        hpush_async(rowtab, rstride, ij1.y - rfirst, ij1.x, bo, 8u * par, conj_store<Num>(z));
+#pragma unroll
+                    for (int e = 0; e < EPT; ++e) {
+                        if (e > 0 && !mine[e]) break;
+                        const S zs = Num::store(z[e]);
+                        *reinterpret_cast<S *>(smem_raw + ad[e][2 * NBO] + bo) = zs;
+                        if (npeer[e] > 0) st_async16(pa[e][0] + bo, zs, pm[e][0] + 8u * par);
+                        if (npeer[e] > 1) st_async16(pa[e][1] + bo, zs, pm[e][1] + 8u * par);
+                        if (npeer[e] > 2) {
+                            const uint32_t *r = rowtab + (ij1[e].x - rfirst) * rstride;
+                            for (int t = 2; t < npeer[e]; ++t)
+                                st_async16(r[1 + 2 * t] + (uint32_t)ij1[e].y * (uint32_t)sizeof(S) + bo, zs,
+                                           r[2 + 2 * t] + 8u * par);
+                        }
+                        if (mirror1[e])
+                            hpush_async(rowtab, rstride, ij1[e].y - rfirst, ij1[e].x, bo, 8u * par,
+                                        conj_store<Num>(z[e]));
+                    }
                 }
             } else {
 #pragma unroll 1
@@ -1407,7 +1450,9 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_s_kernel(const Pro
     }
     if (bnd && bcount == 0) store_bound();
     if constexpr (ONE) {
-        if (mine) store_herm<Num>(x_out + soff, d, ij1.x, ij1.y, Num::store(x1));
+#pragma unroll
+        for (int e = 0; e < EPT; ++e)
+            if (mine[e]) store_herm<Num>(x_out + soff, d, ij1[e].x, ij1[e].y, Num::store(x1[e]));
     } else {
         for (int li = tid; li < cnt; li += nth)
             store_herm<Num>(x_out + soff, d, rc[li].x, rc[li].y, xs[li]);
@@ -2405,24 +2450,26 @@ __global__ void __launch_bounds__(256) expand_kernel(const void *src_v, double2 
 // kernel; bits 2-3 the band/jump shape (0 from the tables, 1 ShapeT, 2 ShapeR,
 // 3 ShapeD, which the other kernels read from the tables; only with real jump
 // tables); bit 5 prop_s_kernel (with a shape), bit 4 its
-// build for one entry per thread, bit 6 with the windows GRAPE_WOFF_SMALL apart.
+// build for one entry per thread, bit 6 with the windows GRAPE_WOFF_SMALL
+// apart, bit 7 for two entries per thread.
 using PropKernel = void (*)(const PropArgs);
+
+template <class Num, class SH>
+PropKernel prop_s_for(int variant) {
+    if (variant & 128) return prop_s_kernel<Num, SH, GRAPE_WOFF, 2>;
+    if (!(variant & 16)) return prop_s_kernel<Num, SH, 0, 1>;
+    return (variant & 64) ? prop_s_kernel<Num, SH, GRAPE_WOFF_SMALL, 1> : prop_s_kernel<Num, SH, GRAPE_WOFF, 1>;
+}
 
 template <class Num>
 PropKernel prop_kernel_for(int variant) {
-    const bool realj = (variant & 1) != 0, herm = (variant & 2) != 0, one = (variant & 16) != 0;
-    const bool small = (variant & 64) != 0;
+    const bool realj = (variant & 1) != 0, herm = (variant & 2) != 0;
     const int shape = (variant >> 2) & 3;
     if (!herm) return realj ? prop_kernel<Num, true> : prop_kernel<Num, false>;
     if (variant & 32) {
-        if (shape == 1)
-            return !one ? prop_s_kernel<Num, ShapeT, 0>
-                        : small ? prop_s_kernel<Num, ShapeT, GRAPE_WOFF_SMALL> : prop_s_kernel<Num, ShapeT, GRAPE_WOFF>;
-        if (shape == 2)
-            return !one ? prop_s_kernel<Num, ShapeR, 0>
-                        : small ? prop_s_kernel<Num, ShapeR, GRAPE_WOFF_SMALL> : prop_s_kernel<Num, ShapeR, GRAPE_WOFF>;
-        return !one ? prop_s_kernel<Num, ShapeD, 0>
-                    : small ? prop_s_kernel<Num, ShapeD, GRAPE_WOFF_SMALL> : prop_s_kernel<Num, ShapeD, GRAPE_WOFF>;
+        if (shape == 1) return prop_s_for<Num, ShapeT>(variant);
+        if (shape == 2) return prop_s_for<Num, ShapeR>(variant);
+        return prop_s_for<Num, ShapeD>(variant);
     }
     if (realj && shape == 1) return prop_h_kernel<Num, true, ShapeT>;
     if (realj && shape == 2) return prop_h_kernel<Num, true, ShapeR>;

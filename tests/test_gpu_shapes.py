@@ -86,3 +86,21 @@ def test_sixteen_cta_clusters(gp, model):
     F1, G1 = P1.gradient(w.u)
     F0, G0 = P0.gradient(w.u)
     assert np.all(np.isfinite(G1)) and F1 == F0 and np.array_equal(G1, G0)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("model,N,tile", [("driven", 33, (8, 352)),          # 619 entries: two per thread
+                                          ("dephasing", 46, (16, 320)),      # 600 on 320: the second pass ragged
+                                          ("driven_relaxation", 23, (4, 320)),   # 604, windows 32 KB apart
+                                          ("dephasing", 30, (16, 256))])     # 256 on 256: exactly one each
+def test_two_entries_per_thread(gp, model, N, tile, prec):
+    w = make(model, N, 3)
+    P1, P0 = problems(gp, w, precision=prec)
+    F0, G0 = P0.gradient(w.u)
+    for t in (tile, None):                              # and the tile chosen at create
+        P = P1 if t else gp.GrapeProblem.from_workload(w, precision=prec)
+        if t:
+            P.set_tile(*t)
+        F1, G1 = P.gradient(w.u)
+        assert np.all(np.isfinite(G1)) and F1 == F0 and np.array_equal(G1, G0)
+        assert np.array_equal(P.forward(w.u)[1], P0.forward(w.u)[1])
