@@ -105,7 +105,9 @@ typedef struct grape_problem *grape_problem_t;
  * the whole pulse (a resonator drive keeps the transmon's level, for
  * instance); the calls then run on those entries alone, with the operators
  * restricted to them - every term left out is an exact zero - and rho(T) is
- * returned at full size.  grape_problem_geometry, grape_problem_kernel,
+ * returned at full size.  Where no operator connects two sectors of the basis
+ * and no target reaches between them, calls that return Phi and the gradient
+ * only run on a state's blocks within the sectors.  grape_problem_geometry, grape_problem_kernel,
  * grape_problem_set_tile and the limit of grape_gradient_static refer to the
  * problem at its full size.  Errors: GRAPE_EINVAL (sizes, band offsets beyond
  * +-(d-1), non-Hermitian rho0 or control, negative rates), GRAPE_ENOMEM. */

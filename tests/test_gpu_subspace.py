@@ -179,3 +179,95 @@ def test_checkpoints_batch_static_and_tiles_give_the_same_bits(gp, form):
     torch.cuda.synchronize()
     for i in range(2):
         assert Fb[i].item() == F and np.array_equal(Gb[i].cpu().numpy(), G)
+
+
+def superposed(Q, N, controls=("res_x", "res_y"), n_slices=7, **kw):
+    """Two states over all levels, no operator between the levels."""
+    phys = workloads.Physics(Q=Q, N=N, chi=tuple(0.7 * q for q in range(Q)), kerr=-0.02, kappa=1.0,
+                             controls=controls, **kw)
+    w = workloads.make("superposed", phys, T=0.4, n_slices=n_slices, n_rk=3, states=[(0, 0.8), (1, 0.5j)], u_bound=1.0)
+    rng = np.random.default_rng(Q * 100 + N)
+    for s in range(2):
+        amp = rng.normal(size=Q) + 1j * rng.normal(size=Q)
+        if s == 1:
+            amp[0] = 0.0                               # the second state leaves level 0 empty
+        psi = np.kron(workloads.coherent_ket(N, 0.6 + 0.3j * s), amp / np.linalg.norm(amp))
+        w.rho0[s] = np.outer(psi, psi.conj())
+    return w
+
+
+@pytest.mark.parametrize("Q,N", [(2, 1), (2, 7), (3, 9), (4, 5)])
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("first_order", [False, True])
+@pytest.mark.parametrize("kernel", ["hermitian", "full", "grid"])
+def test_sectors_of_a_superposition(gp, Q, N, prec, first_order, kernel):
+    """Phi and the gradient from the levels' blocks, rho(T) with its coherences."""
+    w = superposed(Q, N)
+    F_ref, G_ref, r_ref = reference(w, first_order)
+    kv = {"hermitian": {}, "full": {"GRAPE_HERMITIAN": 0}, "grid": {"GRAPE_KERNEL": "grid"}}[kernel]
+    with env(**kv):
+        P = gp.GrapeProblem.from_workload(w, grad_mode=int(first_order), precision=prec)
+    F2, G = P.gradient(w.u)
+    F, r = P.forward(w.u)
+    F3, none = P.forward(w.u, want_rho=False)
+    assert none is None and F3 == F2
+    assert rel(r, r_ref) < TOL
+    assert abs(F - F_ref) < TOL * abs(F_ref) and abs(F2 - F_ref) < TOL * abs(F_ref)
+    assert np.max(np.abs(G - G_ref)) < TOL * max(np.max(np.abs(G_ref)), 1e-3)
+
+
+@pytest.mark.parametrize("first_order", [False, True])
+@pytest.mark.parametrize("form", ["penalty", "dephasing", "rate", "between"])
+def test_sectors_with_options(gp, form, first_order):
+    kw = {}
+    controls = ("res_x", "res_y")
+    if form == "dephasing":
+        kw["gamma_phi"] = 0.4
+    if form == "rate":
+        controls = ("res_x", "rate_a")
+    w = superposed(3, 7, controls=controls, **kw)
+    if form == "rate":
+        w.u[:, 1] = np.abs(w.u[:, 1])
+    if form == "between":                              # a target between levels: nothing may be split
+        s = w.sigma.copy()
+        s[0, 1], s[1, 0] = 0.4 - 0.1j, 0.4 + 0.1j
+        w.sigma = s
+    diag = np.repeat(np.arange(7.0), 3) + 0.3 * np.tile(np.arange(3), 7)
+    A = np.diag(diag).astype(complex) if form == "penalty" else None
+    F_ref, G_ref, _ = reference(w, first_order, A, 0.4)
+    P = gp.GrapeProblem.from_workload(w, grad_mode=int(first_order))
+    if form == "penalty":
+        P.set_penalty(diag, 0.4)
+    F, G = P.gradient(w.u)
+    assert abs(F - F_ref) < TOL * abs(F_ref) and rel(G, G_ref) < TOL
+    for want in (True, False):
+        assert abs(P.forward(w.u, want_rho=want)[0] - F_ref) < TOL * abs(F_ref)
+    if form == "penalty":
+        P.set_penalty(None, 0.0)
+        F0, G0, _ = reference(w, first_order)
+        F, G = P.gradient(w.u)
+        assert abs(F - F0) < TOL * abs(F0) and rel(G, G0) < TOL
+        assert abs(P.forward(w.u)[0] - F0) < TOL * abs(F0)
+
+
+def test_sectors_in_checkpoints_batch_and_static_give_the_same_bits(gp):
+    torch = pytest.importorskip("torch")
+    w = superposed(3, 9, n_slices=13)
+    P, Pc = gp.GrapeProblem.from_workload(w), gp.GrapeProblem.from_workload(w, ckpt_stride=4)
+    F, G = P.gradient(w.u)
+    Fc, Gc = Pc.gradient(w.u)
+    assert Fc == F and np.array_equal(Gc, G)
+    for tile in ((2, 64), (16, 512)):
+        P.set_tile(*tile)
+        r0 = P.forward(w.u)[1]
+        Ft, Gt = P.gradient(w.u)
+        assert Ft == F and np.array_equal(Gt, G) and np.array_equal(P.forward(w.u)[1], r0)
+    u = torch.from_numpy(w.u).cuda()
+    Fs, Gs = torch.empty(1, dtype=torch.float64, device="cuda"), torch.empty_like(u)
+    gp._lib.grape_gradient_static(P.handle, u.data_ptr(), Fs.data_ptr(), Gs.data_ptr(), 0)
+    B = gp.GrapeBatch([P, Pc], n_lanes=2)
+    Fb, Gb = B.gradient([u, u])
+    torch.cuda.synchronize()
+    assert Fs.item() == F and np.array_equal(Gs.cpu().numpy(), G)
+    for i in range(2):
+        assert Fb[i].item() == F and np.array_equal(Gb[i].cpu().numpy(), G)
