@@ -1586,15 +1586,32 @@ long long seg_for_budget(const grape_problem *P, size_t budget) {
     return seg;
 }
 
-// The adjoint sweep of a segment runs in chunks of slices; the trace kernel
-// of each finished chunk runs on the problem's second stream while the next
-// chunk propagates, on the SMs the propagation leaves idle.
-int adjoint_chunks(const grape_problem *P, long long j0, long long j1, bool concurrent = false) {
-    // concurrent sweeps: finer chunks shorten the traces left after both sweeps
-    // (first order: one chunk, its traces are a few per cent of a sweep, and a
-    // boundary that two chunks share would be written while a trace reads it)
-    if (concurrent && P->mode != GRAPE_GRAD_EXACT) return 1;
-    int n = concurrent ? 16 : 8;
+// How a gradient's launches are spread: everything on one stream, the traces
+// on a second one beside the adjoint, or the two sweeps side by side and the
+// traces beside both.
+enum class Overlap { none, traces, sweeps };
+
+// Launches a segment's adjoint (and, side by side, forward) sweep is split
+// into; the traces of a finished chunk run on the SMs that the propagation
+// leaves idle.  On one stream there is nothing to overlap: one launch (a
+// chunk more costs 10 us of launch and set-up).  Side by side, the traces of
+// the two end chunks are waited for after the sweeps, 2 trace / n for n
+// chunks, and each chunk costs a launch: n = sqrt(2 trace / launch), with
+// measured constants per entry, offset and slice.  In FP64 a launch also
+// waits for trace CTAs of some hundred microseconds that took its SMs (d=60:
+// 9.3 ms with 4 chunks, 10.5 with 16).
+int adjoint_chunks(const grape_problem *P, long long j0, long long j1, Overlap how) {
+    // (first order side by side: one chunk, its traces are a few per cent of
+    // a sweep, and a boundary that two chunks share would be written while a
+    // trace reads it)
+    if (how == Overlap::sweeps && P->mode != GRAPE_GRAD_EXACT) return 1;
+    int n = how == Overlap::none ? 1 : 8;
+    if (how == Overlap::sweeps) {
+        const bool f64 = P->prec == GRAPE_PREC_FP64;
+        const double trace_us = (f64 ? 6.7e-4 : 8e-5) * (double)(j1 - j0) * P->n_rk / 4.0 * (double)packed_set(P) *
+                                std::max(1, P->trace.ndo);
+        n = std::max(2, (int)std::lround(std::sqrt(2.0 * trace_us / (f64 ? 370.0 : 10.0))));
+    }
     if (const char *env = std::getenv("GRAPE_ADJ_CHUNKS")) n = std::atoi(env);
     n = std::max(1, std::min(n, grape_problem::kMaxChunks));
     return (int)std::min<long long>(n, j1 - j0);
@@ -1624,8 +1641,9 @@ bool concurrent_sweeps(const grape_problem *P) {
     return true;
 }
 
-int gradient_launch_count(const grape_problem *P, int seg, int nseg, bool concurrent = false) {
+int gradient_launch_count(const grape_problem *P, int seg, int nseg, Overlap how) {
     if (nseg <= 0) return -1;
+    const bool concurrent = how == Overlap::sweeps;
     // the cost, and the forward sweep to the checkpoints (to the end when the
     // sweeps are not side by side)
     int n = 1 + ((nseg > 1 || !concurrent) ? 1 : 0);
@@ -1633,7 +1651,7 @@ int gradient_launch_count(const grape_problem *P, int seg, int nseg, bool concur
     for (int gi = 0; gi < nseg; ++gi) {
         const long long j0 = (long long)gi * seg;
         const long long j1 = std::min<long long>(P->n_slices, j0 + seg);
-        const int nch = adjoint_chunks(P, j0, j1, concurrent);
+        const int nch = adjoint_chunks(P, j0, j1, how);
         n += nch + (concurrent ? nch : (nseg > 1 ? 1 : 0));   // adjoint, forward of the segment
         if (P->R > 0) n += nch * (P->trace.nsplit > 1 ? 2 : 1);
         if (P->penalty) n += 1;                   // boundary values of the segment
@@ -1808,7 +1826,7 @@ grape_status run_gradient_concurrent(grape_problem *P, const double *ud, double 
     for (int gi = S.nseg - 1; gi >= 0; --gi) {
         const long long j0 = (long long)gi * S.seg;
         const long long j1 = std::min<long long>(P->n_slices, j0 + S.seg);
-        const int nch = adjoint_chunks(P, j0, j1, true);
+        const int nch = adjoint_chunks(P, j0, j1, Overlap::sweeps);
         auto first = [&](int ci) { return j0 + (j1 - j0) * ci / nch; };
         if (S.nseg > 1) seg_x0 = S.ckpt + (size_t)gi * mat;
         // a segment of another length has other chunks: wait for all traces
@@ -1945,7 +1963,7 @@ grape_status run_gradient(grape_problem *P, const double *ud, double *Fd, double
             return st;
         // adjoint sweep in chunks (last slices first); the trace of each
         // finished chunk runs on s2, overlapping the next chunk
-        const int nch = adjoint_chunks(P, j0, j1);
+        const int nch = adjoint_chunks(P, j0, j1, S.s2 ? Overlap::traces : Overlap::none);
         for (int ci = nch - 1; ci >= 0; --ci) {
             const long long cA = j0 + (j1 - j0) * ci / nch;
             const long long cB = j0 + (j1 - j0) * (ci + 1) / nch;
@@ -2538,7 +2556,10 @@ grape_status grape_phase_times(grape_problem_t P, double ms[4], int32_t launches
 int32_t grape_gradient_launches(grape_problem_t P) {
     if (!P) return -1;
     P = grad_problem(P);
-    return gradient_launch_count(P, P->seg, P->nseg, concurrent_sweeps(P));
+    bool traces = true;
+    if (const char *env = std::getenv("GRAPE_TRACE_OVERLAP")) traces = std::atoi(env) != 0;
+    return gradient_launch_count(P, P->seg, P->nseg,
+                                 concurrent_sweeps(P) ? Overlap::sweeps : traces ? Overlap::traces : Overlap::none);
 }
 
 grape_status grape_forward(grape_problem_t problem, const double *u, double *F, double *rhoT,
@@ -3323,7 +3344,7 @@ grape_status grape_batch_info(grape_batch_t B, int32_t *n_lanes, size_t *scratch
         int n = 0;
         for (size_t i = 0; i < B->probs.size(); ++i)
             n += gradient_launch_count(B->probs[i], B->scratch[i].seg, B->scratch[i].nseg,
-                                       B->scratch[i].s3 != nullptr);
+                                       B->scratch[i].s3 ? Overlap::sweeps : Overlap::none);
         *launches = n;
     }
     return GRAPE_OK;
