@@ -3034,8 +3034,10 @@ int resident_clusters(const grape_problem *P) {
 // each bucket the largest problem stands in for the rest: for every tile
 // (cluster width x threads per CTA) that fits it, a forward propagation of
 // a few slices runs as C concurrent copies, C = the copies whose clusters
-// can be resident at once (at most kMaxCopies), and the tile with the most
-// slices per second over all copies wins.  It is then set on every problem
+// can be resident at once (at most kMaxCopies, and no more than the batch
+// has problems: a small batch is better off on wide tiles than waiting for
+// its longest problem on a narrow one, 24 problems 26.4 -> 12.6 ms), and the tile with
+// the most slices per second over all copies wins.  It is then set on every problem
 // of the bucket it fits (results do not depend on the tile).
 constexpr int kMaxCopies = 64;
 constexpr int kProbeSlices = 32;
@@ -3119,7 +3121,7 @@ grape_status tune_batch(grape_batch *B) {
                 const grape_status ps = grape_problem_set_tile(R, w, t);
                 if (ps == GRAPE_EINVAL) continue;
                 if (ps != GRAPE_OK) { st = ps; break; }
-                const int C = std::max(1, std::min(kMaxCopies, resident_clusters(R) / R->ns));
+                const int C = std::max(1, std::min({kMaxCopies, n, resident_clusters(R) / R->ns}));
                 float ms = 0.0f, ms2 = 0.0f;
                 if ((st = probe(R, C, &ms)) != GRAPE_OK || (st = probe(R, C, &ms2)) != GRAPE_OK) break;
                 const double rate = C / (double)std::max(1e-3f, std::min(ms, ms2));
@@ -3285,10 +3287,11 @@ grape_status grape_batch_create(grape_problem_t *problems, int32_t n, int32_t n_
         }
     }
     // concurrent sweeps inside each lane (the problems' forward and adjoint
-    // sweeps side by side, as in grape_gradient): GRAPE_BATCH_CONCURRENT=1
-    // (measured: the same throughput as one sweep after the other, the batch
-    // being bound by SM time, with 22 % more launches; off by default)
-    bool lane_conc = false;
+    // sweeps side by side, as in grape_gradient): a lane's longest problem
+    // bounds a small batch, and the SMs its narrow tiles leave idle take the
+    // second sweep (24 reset problems 12.6 -> 9.6 ms, 256 at a tenth of their
+    // slices 105 -> 101 ms); GRAPE_BATCH_CONCURRENT=0 turns it off
+    bool lane_conc = true;
     if (const char *env = std::getenv("GRAPE_BATCH_CONCURRENT")) lane_conc = std::atoi(env) != 0;
     if (lane_conc) {
         const int nev = 3 * grape_problem::kMaxChunks + 3;
