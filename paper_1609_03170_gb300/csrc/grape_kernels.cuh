@@ -504,6 +504,14 @@ __device__ __forceinline__ void store_herm(typename Num::store_t *dst, int d, in
     if (j != i) dst[(size_t)j * d + i] = conj_store<Num>(Num::load(v));
 }
 
+// store of upper entry (i, j) and, within hb of the diagonal, its mirror
+template <class Num>
+__device__ __forceinline__ void store_near(typename Num::store_t *dst, int d, int hb, int i, int j,
+                                           typename Num::val v) {
+    dst[(size_t)i * d + j] = Num::store(v);
+    if (j != i && j - i <= hb) dst[(size_t)j * d + i] = conj_store<Num>(v);
+}
+
 // push value v of entry (r, c) to every window holding row r: rowtab holds,
 // per row, the target count and each target's distributed-shared-memory
 // address of (r, 0) in buf0 (buffer offset boff selects buf1)
@@ -1468,7 +1476,10 @@ __global__ void __launch_bounds__(EPT == 2 ? GRAPE_TWO_THREADS : GRAPE_PROP_THRE
 // tables and the same per-entry arithmetic, so the same bits), but a window
 // lives in the CTA's shared memory only while one stage is computed: the
 // stage values themselves live as full matrices in two global buffers
-// (L2-resident), each upper entry written with its conjugate mirror.  Per
+// (L2-resident), each upper entry written, and near the diagonal, where the
+// windows read it, its conjugate mirror.  (Mirrors everywhere were half of
+// the writes, one 16-byte piece of a sector each: d=512 12.37 -> 11.79 ms per
+// first-order gradient.)  Per
 // stage a CTA
 //  - waits until every neighbour CTA - one that writes a row of its window
 //    or holds a row it writes - has finished the previous stage (a flag per
@@ -1596,7 +1607,7 @@ __global__ void __launch_bounds__(GRAPE_GRID_THREADS, 1) prop_g_kernel(const Pro
         const int2 ij = rc[u - u0];
         const V x = Num::load(x_in[(size_t)ij.x * d + ij.y]);
         xs[u - u0] = Num::store(x);
-        store_herm<Num>(gb0, d, ij.x, ij.y, Num::store(Num::scale(cg[0], x)));
+        store_near<Num>(gb0, d, hb, ij.x, ij.y, Num::scale(cg[0], x));
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1691,7 +1702,7 @@ __global__ void __launch_bounds__(GRAPE_GRID_THREADS, 1) prop_g_kernel(const Pro
                     xs[li] = Num::store(nx);
                     z = Num::scale(cg[0], nx);
                 }
-                store_herm<Num>(nxt, d, ij.x, ij.y, Num::store(z));
+                store_near<Num>(nxt, d, hb, ij.x, ij.y, z);
             }
             if (s == 3 && it + 1 < nsub) {
                 const long long nn = p.reverse ? n - 1 : n + 1;
