@@ -1025,7 +1025,7 @@ __global__ void __launch_bounds__(EPT == 2 ? GRAPE_TWO_THREADS : GRAPE_PROP_THRE
     constexpr int NTL = 2 + SH::NT;               // D_re, D_im, jumps with an offset
     constexpr int NA = 2 * NBO + 1 + SH::NT;      // neighbour slots: rows, columns, own entry, jumps
     constexpr int NRP = NBR / 2 + NBC;            // 16-byte pairs of a band row in use (of 3)
-    static_assert(NBR % 2 == 0 && NRP <= 3, "band row");
+    static_assert(NBR % 2 == 0 && NBC > 0 && NRP <= 3, "band row");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint64_t mbar[2];
     __shared__ int s_err;
@@ -1336,11 +1336,12 @@ __global__ void __launch_bounds__(EPT == 2 ? GRAPE_TWO_THREADS : GRAPE_PROP_THRE
             auto entry = [&](int i, int j, auto &&at, auto &&tail, V &x, V &a, S *dst) -> V {
                 auto val = [&](int k) { return Num::load(*reinterpret_cast<const S *>(win + at(k))); };
                 const RP *ri = rows_t + i * 3, *rj = rows_t + j * 3;
-                A U = Num::acc_zero(), T = Num::acc_zero();          // W = U + i T
+                A U, T;                                              // W = U + i T
 #pragma unroll
                 for (int b = 0; b < NBR; b += 2) {
                     const RP ci = ri[b / 2], cj = rj[b / 2];
-                    Num::mac_real(T, Num::neg_real(ci.u), val(b));
+                    if (b == 0) T = Num::mul_real(Num::neg_real(ci.u), val(b));
+                    else Num::mac_real(T, Num::neg_real(ci.u), val(b));
                     Num::mac_real(T, cj.u, val(NBO + b));
                     Num::mac_real(T, Num::neg_real(ci.t), val(b + 1));
                     Num::mac_real(T, cj.t, val(NBO + b + 1));
@@ -1349,8 +1350,10 @@ __global__ void __launch_bounds__(EPT == 2 ? GRAPE_TWO_THREADS : GRAPE_PROP_THRE
                 for (int b = NBR; b < NBO; ++b) {
                     const RP ci = ri[NBR / 2 + b - NBR], cj = rj[NBR / 2 + b - NBR];
                     const V v1 = val(b), v2 = val(NBO + b);
-                    Num::mac_real(U, ci.u, v1);
-                    Num::mac_real(T, Num::neg_real(ci.t), v1);
+                    if (b == NBR) U = Num::mul_real(ci.u, v1);
+                    else Num::mac_real(U, ci.u, v1);
+                    if (b == 0) T = Num::mul_real(Num::neg_real(ci.t), v1);
+                    else Num::mac_real(T, Num::neg_real(ci.t), v1);
                     Num::mac_real(U, cj.u, v2);
                     Num::mac_real(T, cj.t, v2);
                 }
@@ -1371,7 +1374,7 @@ __global__ void __launch_bounds__(EPT == 2 ? GRAPE_TWO_THREADS : GRAPE_PROP_THRE
                 x = acc;
                 if (left == 1 && p.src && p.reverse && i == j)       // the running cost's source (App. B)
                     x = Num::add_real(x, Num::real_once(p.src[state * d + i]));
-                return Num::scale(RK::g(p, 0), x);
+                return unit_g ? x : Num::scale(RK::g(p, 0), x);
             };
             S *std_ = st ? st + (size_t)p.store_map[s] * sset : nullptr;
             if constexpr (ONE) {

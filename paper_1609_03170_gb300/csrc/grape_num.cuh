@@ -162,6 +162,8 @@ struct NumD {
         w.re = fma(c, b.re, w.re);
         w.im = fma(c, b.im, w.im);
     }
+    // acc = c * b, c real: mac_real on an empty sum (the same bits)
+    static __device__ __forceinline__ acc mul_real(real_t c, val b) { return {c * b.re, c * b.im}; }
     // x + s*w
     static __device__ __forceinline__ val axpy(real_t s, val w, val x) {
         return {fma(s, w.re, x.re), fma(s, w.im, x.im)};
@@ -370,6 +372,15 @@ struct NumF {
     // acc += c b, c real
     static __device__ __forceinline__ void mac_real(acc &w, real_t c, val b) {
         p_lacc_fma(w.h, w.l, p_b(c.h), p_b(c.l), b.h, b.l);
+    }
+    // acc = c b, c real: mac_real on an empty sum (the same bits without the
+    // sum's eight operations)
+    static __device__ __forceinline__ acc mul_real(real_t c, val b) {
+        const float2 ch = p_b(c.h), cl = p_b(c.l);
+        const float2 p = p_mul(ch, b.h);
+        float2 e = p_fma(ch, b.h, p_neg(p));
+        e = p_fma(ch, b.l, e);
+        return {p, p_fma(cl, b.h, e)};
     }
     static __device__ __forceinline__ val axpy(real_t s, val w, val x) {
         val v;
