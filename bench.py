@@ -189,7 +189,7 @@ def kernel_source_sha(csrc=None):
 def profiled_traffic(kernel_src_sha):
     """DRAM bytes per launch of the forward propagation kernel from the
     committed ncu summary, if it was taken on the current kernel source."""
-    path = os.path.join(ROOT, "profiles", "prop_h_kernel_transmon_resonator_d120.md")
+    path = os.path.join(ROOT, "profiles", "prop_s_kernel_transmon_resonator_d120.md")
     if not os.path.exists(path):
         return None
     text = open(path).read()

@@ -948,9 +948,10 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
 //    addresses, own-entry and jump coefficients, RK state and push targets are
 //    registers for the whole launch.
 // Measured (GB300, 2070 MHz, against prop_h_kernel with one entry per thread
-// in registers): d=120 on 16 CTAs 2.44 -> 1.69 us per stage, 376 instructions;
-// the d=120 gradient 81.1 -> 60.4 ms; d=20 on one CTA 1.28 -> 0.85 us.  Two
-// lanes per entry, which halves each thread's dependent chain, measured
+// in registers): d=120 on 16 CTAs 2.44 -> 1.65 us per stage, about 390
+// instructions; the d=120 gradient 81.1 -> 60.4 ms by this kernel (56.2 ms
+// with the later trace kernel); d=20 on one CTA 1.28 -> 0.85 us.  Two lanes
+// per entry, which halves each thread's dependent chain, measured
 // 2.35 us at d=120: it doubles the instructions that are not arithmetic.
 //
 // Ownership, windows, pushes and the two mbarriers are prop_h_kernel's; each
