@@ -785,10 +785,18 @@ cudaError_t k_prop(const grape_problem *P, const PropArgs &a, cudaStream_t s) {
 cudaError_t k_trace(const grape_problem *P, const TraceArgs &t, cudaStream_t s) {
     return P->prec == GRAPE_PREC_FP64 ? grape_launch_trace_f64(t, s) : grape_launch_trace_df(t, s);
 }
-cudaError_t k_cost(const grape_problem *P, const void *rho, double *F, cudaStream_t s) {
+// part, ticket: the kernel's partial sums and the count of finished CTAs (0
+// before the launch, and again after it); no two launches that may overlap
+// share them
+cudaError_t k_cost(const grape_problem *P, const void *rho, double *part, unsigned *ticket, double *F,
+                   cudaStream_t s) {
     return P->prec == GRAPE_PREC_FP64
-               ? grape_launch_cost_f64(rho, P->d_sigma, P->ns, (int)P->d2, P->d_cost, P->d_gbar + 3, F, s)
-               : grape_launch_cost_df(rho, P->d_sigma, P->ns, (int)P->d2, P->d_cost, P->d_gbar + 3, F, s);
+               ? grape_launch_cost_f64(rho, P->d_sigma, P->ns, (int)P->d2, part, ticket, F, s)
+               : grape_launch_cost_df(rho, P->d_sigma, P->ns, (int)P->d2, part, ticket, F, s);
+}
+// with the problem's own pair (the calls that use the problem's other buffers)
+cudaError_t k_cost(const grape_problem *P, const void *rho, double *F, cudaStream_t s) {
+    return k_cost(P, rho, P->d_cost, P->d_gbar + 3, F, s);
 }
 cudaError_t k_to_double(const grape_problem *P, const void *src, double2 *dst, size_t n,
                         cudaStream_t s) {
@@ -2919,7 +2927,10 @@ grape_status grape_gradient_static(grape_problem_t P, const double *u, double *F
         f.bound_step = seg * P->n_rk;
     }
     GRAPE_CUDA_TRY(k_prop(P, f, s));
-    GRAPE_CUDA_TRY(k_cost(P, x, F, s));
+    // the cost's ticket and partial sums (8 B for 2048 entries) lie where the
+    // adjoint's stages come later: a slice of those is 32 B per entry or more
+    GRAPE_CUDA_TRY(cudaMemsetAsync(K, 0, sizeof(double2), s));
+    GRAPE_CUDA_TRY(k_cost(P, x, reinterpret_cast<double *>(K + 1), reinterpret_cast<unsigned *>(K), F, s));
     GRAPE_CUDA_TRY(cudaMemcpyAsync(mu, P->d_sigma, m * sizeof(double2), cudaMemcpyDeviceToDevice, s));
     for (int gi = nseg - 1; gi >= 0; --gi) {
         const long long j0 = (long long)gi * seg;
