@@ -2383,24 +2383,42 @@ grape_status grape_problem_create(const grape_problem_desc *desc, grape_problem_
     std::vector<int> from;
     std::vector<std::vector<int>> bidx;
     const bool splits = split_problem(reduced ? part : full, &blocks, &from, &bidx);
-    const BuildMode whole = splits ? BuildMode::forward : BuildMode::all;
+    // the problem on `parts` of the space: 0 none, 1 its states' subspaces (if
+    // there are any), 2 the sectors' blocks as well
+    auto assemble = [&](int parts, grape_problem **made) -> grape_status {
+        const bool sub = reduced && parts >= 1, blks = splits && parts >= 2;
+        const BuildMode whole = blks ? BuildMode::forward : BuildMode::all;
+        grape_problem *P = nullptr;
+        if ((st = build_problem(desc, full, sub ? BuildMode::geometry : whole, &P)) != GRAPE_OK) return st;
+        auto bail = [&](grape_status e) { delete P; return e; };
+        if (sub) {
+            if ((st = build_problem(desc, part, whole, &P->sub)) != GRAPE_OK) return bail(st);
+            std::vector<int> map((size_t)P->ns * d, -1);
+            for (int s = 0; s < P->ns; ++s)
+                for (size_t a = 0; a < idx[s].size(); ++a) map[(size_t)s * d + idx[s][a]] = (int)a;
+            if ((st = upload(P, map, &P->d_imap)) != GRAPE_OK) return bail(st);
+            P->sub_idx = idx;
+        }
+        if (blks) {
+            grape_problem *A = active(P);
+            if ((st = build_problem(desc, blocks, BuildMode::all, &A->split)) != GRAPE_OK) return bail(st);
+            A->split_from = from;
+            A->split_idx = bidx;
+        }
+        *made = P;
+        return GRAPE_OK;
+    };
+    // Parts that no table, kernel or memory holds (take_parts compares the
+    // numbers of bands and products in all, the tables have limits per kind)
+    // leave the problem on a larger part, at last on the whole space: what the
+    // full size is accepted for never depends on the parts.
     grape_problem *P = nullptr;
-    if ((st = build_problem(desc, full, reduced ? BuildMode::geometry : whole, &P)) != GRAPE_OK) return st;
-    auto bail = [&](grape_status e) { delete P; return e; };
-    if (reduced) {
-        if ((st = build_problem(desc, part, whole, &P->sub)) != GRAPE_OK) return bail(st);
-        std::vector<int> map((size_t)P->ns * d, -1);
-        for (int s = 0; s < P->ns; ++s)
-            for (size_t a = 0; a < idx[s].size(); ++a) map[(size_t)s * d + idx[s][a]] = (int)a;
-        if ((st = upload(P, map, &P->d_imap)) != GRAPE_OK) return bail(st);
-        P->sub_idx = std::move(idx);
+    for (int parts = splits ? 2 : reduced ? 1 : 0; parts >= 0; --parts) {
+        if (parts == 1 && !reduced) continue;
+        st = assemble(parts, &P);
+        if (st != GRAPE_EINVAL && st != GRAPE_ENOMEM) break;
     }
-    if (splits) {
-        grape_problem *A = active(P);
-        if ((st = build_problem(desc, blocks, BuildMode::all, &A->split)) != GRAPE_OK) return bail(st);
-        A->split_from = std::move(from);
-        A->split_idx = std::move(bidx);
-    }
+    if (st != GRAPE_OK) return st;
     *out = P;
     return GRAPE_OK;
 }
