@@ -973,7 +973,9 @@ std::vector<int> hermitian_table(int d, int ncl, int omax, int hb, int *maxwin, 
     // window slots peers write each stage: slot (r, c) of CTA k's window holds
     // the upper entry (r, c), c >= r, or the mirror of (c, r); its writer is
     // the owner of that upper entry, so a row's slots from the diagonal on
-    // are consecutive entries of which k owns a range
+    // are consecutive entries of which k owns a range.  (The table's end: a CTA
+    // reads its count once, from global memory, so that these ncl integers take
+    // no shared memory from the largest tiles.)
     for (int k = 0; k < ncl; ++k) {
         const long long u0 = head[4 * k], u1 = head[4 * k + 1];
         long long n = 0;
@@ -1034,6 +1036,7 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
     int maxwin = 0, cu = 0, rt_rows = 0;
     const std::vector<int> tab = hermitian_table(d, ncl, P->omax, hb, &maxwin, &cu, &rt_rows);
     if (maxwin >= 32767) return fail(GRAPE_EINVAL, "state window too large for 16-bit addresses");
+    const size_t tab_len = tab.size() - ncl;     // ints kept in shared memory
     // shared memory without windows, own-entry and jump-coefficient tables
     // two mbarriers; base values, accumulators and next values of the owned
     // entries; bands, jump tables; (row, column), RK coefficients, the
@@ -1041,7 +1044,7 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
     // and the neighbour addresses
     const int sh = shape_id(P), nts = shape_jumps(sh, nt);
     const size_t base = 16 + (2 * (size_t)cu + 2 * (size_t)nb * d + 2 * (size_t)nt * d) * sizeof(double2) +
-                        (size_t)cu * sizeof(int2) + 12 * sizeof(double) + tab.size() * sizeof(int) +
+                        (size_t)cu * sizeof(int2) + 12 * sizeof(double) + tab_len * sizeof(int) +
                         (size_t)rt_rows * (2 * ncl + 1) * sizeof(uint32_t) +
                         (size_t)cu * (2 * nb + nts + 1) * sizeof(short);
     // Options of prop_h_kernel, each kept only when the tile still fits
@@ -1068,7 +1071,7 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
         const bool one = two || (cu <= threads && wbytes <= GRAPE_WOFF);
         const bool small = one && !two && wbytes <= GRAPE_WOFF_SMALL;
         const size_t pbase = (one ? (small ? GRAPE_WOFF_SMALL : GRAPE_WOFF) : wbytes) + wbytes +
-                             (size_t)8 * d * sizeof(double2) + tab.size() * sizeof(int) +
+                             (size_t)8 * d * sizeof(double2) + tab_len * sizeof(int) +
                              (size_t)rt_rows * (2 * ncl + 1) * sizeof(uint32_t) +
                              (one ? 0 : (size_t)cu * (2 * sizeof(double2) + (2 + nts) * sizeof(double) + sizeof(int2) +
                                                       (2 * (nb - 1) + 1 + nts) * sizeof(short)));
@@ -1138,7 +1141,7 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
     P->cu = cu;
     P->maxwin = maxwin;
     P->hb = hb;
-    P->htab_len = (int)tab.size();
+    P->htab_len = (int)tab_len;
     P->rt_rows = rt_rows;
     P->smem = use;
     P->fold = fold ? 1 : 0;
@@ -1260,6 +1263,7 @@ grape_status choose_geometry_grid(grape_problem *P, bool geometry_only) {
     int maxwin = 0, cu = 0, rt_rows = 0;
     const std::vector<int> tab = hermitian_table(d, nct, P->omax, hb, &maxwin, &cu, &rt_rows);
     if (maxwin >= 32767) return fail(GRAPE_EINVAL, "state window too large for the grid propagation kernel");
+    const size_t tab_len = tab.size() - nct;     // ints kept in shared memory
     const int variant = (P->variant & 1) | (shape_id(P) << 2);
     int njt = 0;
     for (int dir = 0; dir < 2; ++dir) {
@@ -1270,7 +1274,7 @@ grape_status choose_geometry_grid(grape_problem *P, bool geometry_only) {
     // one window, base values and accumulators, one band table (the jump
     // tables stay in global memory)
     const size_t base = ((size_t)(maxwin + 1) + 2 * (size_t)cu + (size_t)nb * d) * sizeof(double2) +
-                        (size_t)cu * sizeof(int2) + 12 * sizeof(double) + tab.size() * sizeof(int) +
+                        (size_t)cu * sizeof(int2) + 12 * sizeof(double) + tab_len * sizeof(int) +
                         (size_t)cu * (2 * nb + shape_jumps(shape_id(P), nt) + 1) * sizeof(short);
     bool want_fold = true, want_jc = variant != 0;
     if (const char *env = std::getenv("GRAPE_FOLD")) want_fold = std::atoi(env) != 0;
@@ -1318,7 +1322,7 @@ grape_status choose_geometry_grid(grape_problem *P, bool geometry_only) {
     P->cu = cu;
     P->maxwin = maxwin;
     P->hb = hb;
-    P->htab_len = (int)tab.size();
+    P->htab_len = (int)tab_len;
     P->rt_rows = rt_rows;
     P->fold = fold ? 1 : 0;
     P->jcache = jcache ? 1 : 0;

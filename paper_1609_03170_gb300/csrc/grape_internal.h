@@ -78,7 +78,7 @@ struct PropArgs {
     // Hermitian kernel (upper triangle only): the cluster's ownership and
     // window tables, see GRAPE_HTAB_* below
     const int *htab;
-    int htab_len;                       // ints in htab
+    int htab_len;                       // ints of htab that the kernels copy to shared memory
     int hb;                             // stored half-band below the diagonal
     int cu;                             // upper-triangle entries per CTA
     int maxwin;                         // largest window (entries) of the cluster
@@ -111,6 +111,7 @@ struct PropArgs {
 //   [row-offset lists]     CTA k: nrows_k + 1 cumulative window offsets
 //   [kfirst[d], klast[d]]  first and last CTA whose window holds row r
 //   [ncl]                  window slots of CTA k that its peers write each stage
+//                          (read once from global memory: beyond htab_len)
 #define GRAPE_HTAB_CTA(k) (4 * (k))
 #define GRAPE_HTAB_LISTS(ncl) (4 * (ncl))
 

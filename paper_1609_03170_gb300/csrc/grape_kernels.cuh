@@ -784,9 +784,9 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
         }
         e[0] = (uint32_t)n;
     }
-    cluster_sync_all();   // every CTA runs, windows zeroed, mbarriers initialised, tables built
     // bytes peers push into this CTA's window each stage
-    const uint32_t expect = (uint32_t)kfl[2 * d + rank] * (uint32_t)sizeof(S);
+    const uint32_t expect = (uint32_t)__ldg(&p.htab[p.htab_len + rank]) * (uint32_t)sizeof(S);
+    cluster_sync_all();   // every CTA runs, windows zeroed, mbarriers initialised, tables built
     const long long limit = 1LL << 31;          // SM cycles a window wait may take
     const uint32_t boff1 = (uint32_t)(wst * (int)sizeof(S));
 
@@ -1238,9 +1238,9 @@ __global__ void __launch_bounds__(EPT == 2 ? GRAPE_TWO_THREADS : GRAPE_PROP_THRE
     bool mirror1[EPT];                            // the entry's mirror lies in a window too
 #pragma unroll
     for (int e = 0; e < EPT; ++e) mirror1[e] = mine[e] && ij1[e].y > ij1[e].x && ij1[e].y - ij1[e].x <= hb;
-    cluster_sync_all();   // every CTA runs, windows zeroed, mbarriers initialised, tables built
     // bytes peers push into this CTA's window each stage
-    const uint32_t expect = (uint32_t)kfl[2 * d + rank] * (uint32_t)sizeof(S);
+    const uint32_t expect = (uint32_t)__ldg(&p.htab[p.htab_len + rank]) * (uint32_t)sizeof(S);
+    cluster_sync_all();   // every CTA runs, windows zeroed, mbarriers initialised, tables built
     const long long limit = 1LL << 31;            // SM cycles a window wait may take
     bool failed = false;
 
