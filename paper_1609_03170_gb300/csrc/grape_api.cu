@@ -1023,8 +1023,10 @@ int shape_id(const grape_problem *P) {
     return 0;
 }
 
-// jump terms the kernels of a shape hold room for
+// jump terms prop_s_kernel holds room for, and the builds of prop_h_kernel and
+// prop_g_kernel for shapes 1 and 2 (which read shape 3 from the tables)
 int shape_jumps(int shape, int nt) { return shape == 1 ? 3 : shape ? std::max(shape - 1, nt) : nt; }
+int h_jumps(int shape, int nt) { return shape == 3 ? nt : shape_jumps(shape, nt); }
 
 // Hermitian cluster kernel with `ncl` CTAs of `threads` threads per state:
 // sets the geometry, or GRAPE_EINVAL when the tile does not fit.  Tables
@@ -1046,7 +1048,7 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
     const size_t base = 16 + (2 * (size_t)cu + 2 * (size_t)nb * d + 2 * (size_t)nt * d) * sizeof(double2) +
                         (size_t)cu * sizeof(int2) + 12 * sizeof(double) + tab_len * sizeof(int) +
                         (size_t)rt_rows * (2 * ncl + 1) * sizeof(uint32_t) +
-                        (size_t)cu * (2 * nb + nts + 1) * sizeof(short);
+                        (size_t)cu * (2 * nb + nt + 1) * sizeof(short);
     // Options of prop_h_kernel, each kept only when the tile still fits
     // (the same values, so the same bits, either way): the own-entry
     // coefficients cached per slice (16 B per owned entry) instead of
@@ -1091,16 +1093,6 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
             found = true;
         }
     }
-    if (!found) variant = (P->variant & 1) | 2 | (sh << 2);
-    if (!found) {
-        const cudaError_t e = P->prec == GRAPE_PREC_FP64
-                                  ? grape_prepare_prop_f64(variant, (size_t)max_smem_optin(P), 16)
-                                  : grape_prepare_prop_df(variant, (size_t)max_smem_optin(P), 16);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return fail(GRAPE_ECUDA, std::string("hermitian kernel attributes: ") + cudaGetErrorString(e));
-        }
-    }
     int njt = 0;
     for (int q = 0; q < P->tab[0].nt; ++q) njt += ((P->tab[0].jdiag >> q) & 1) ? 0 : 1;
     int njt_d = 0;
@@ -1109,20 +1101,37 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
     struct Opt { bool fold, defer, jc; };
     const Opt opts[] = {{true, true, true}, {true, true, false}, {true, false, true}, {true, false, false},
                         {false, true, false}, {false, false, false}};
-    for (const Opt &o : opts) {
-        if (found) break;
-        if ((o.fold && !want_fold) || (o.defer && !want_defer) || (o.jc && !want_jc)) continue;
-        const size_t sm = base + 2 * (size_t)(maxwin + 1) * sizeof(double2) +
-                          (o.fold ? (size_t)cu * sizeof(double2) : 0) +
-                          (o.defer ? (size_t)cu * sizeof(double2) : 0) +
-                          (o.jc ? (size_t)njt * cu * sizeof(double) : 0);
-        if (sm + 1024 > (size_t)max_smem || !cluster_fits(P, variant, threads, sm, ncl)) continue;
-        use = sm;
-        fold = o.fold;
-        defer = o.defer;
-        jcache = o.jc;
-        found = true;
-    }
+    // With each set of options the compile-time layout, and where its room for
+    // more jump terms than there are does not fit, the run-time one (the same
+    // bits): Jaynes-Cummings, one term in a layout for three, runs on clusters
+    // up to d=216 and not only d=212.
+    const int hshape = sh == 3 ? 0 : sh;         // prop_h_kernel has no build for shape 3
+    const int layouts = h_jumps(hshape, nt) > nt ? 2 : 1;
+    for (const Opt &o : opts)
+        for (int l = 0; l < layouts && !found; ++l) {
+            const int hs = l ? 0 : hshape;
+            if ((o.fold && !want_fold) || (o.defer && !want_defer) || (o.jc && !want_jc)) continue;
+            const size_t sm = base + (size_t)cu * (h_jumps(hs, nt) - nt) * sizeof(short) +
+                              2 * (size_t)(maxwin + 1) * sizeof(double2) +
+                              (o.fold ? (size_t)cu * sizeof(double2) : 0) +
+                              (o.defer ? (size_t)cu * sizeof(double2) : 0) +
+                              (o.jc ? (size_t)njt * cu * sizeof(double) : 0);
+            if (sm + 1024 > (size_t)max_smem) continue;
+            const int v = (P->variant & 1) | 2 | (hs << 2);
+            const cudaError_t e = P->prec == GRAPE_PREC_FP64 ? grape_prepare_prop_f64(v, (size_t)max_smem, 16)
+                                                             : grape_prepare_prop_df(v, (size_t)max_smem, 16);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                return fail(GRAPE_ECUDA, std::string("hermitian kernel attributes: ") + cudaGetErrorString(e));
+            }
+            if (!cluster_fits(P, v, threads, sm, ncl)) continue;
+            variant = v;
+            use = sm;
+            fold = o.fold;
+            defer = o.defer;
+            jcache = o.jc;
+            found = true;
+        }
     if (!found) {
         const size_t least = base + 2 * (size_t)(maxwin + 1) * sizeof(double2);
         if (least + 1024 > (size_t)max_smem) return fail(GRAPE_EINVAL, "state window does not fit in shared memory");
@@ -1264,7 +1273,8 @@ grape_status choose_geometry_grid(grape_problem *P, bool geometry_only) {
     const std::vector<int> tab = hermitian_table(d, nct, P->omax, hb, &maxwin, &cu, &rt_rows);
     if (maxwin >= 32767) return fail(GRAPE_EINVAL, "state window too large for the grid propagation kernel");
     const size_t tab_len = tab.size() - nct;     // ints kept in shared memory
-    const int variant = (P->variant & 1) | (shape_id(P) << 2);
+    const int shape = shape_id(P);
+    int variant = 0;
     int njt = 0;
     for (int dir = 0; dir < 2; ++dir) {
         int n = 0;
@@ -1275,34 +1285,41 @@ grape_status choose_geometry_grid(grape_problem *P, bool geometry_only) {
     // tables stay in global memory)
     const size_t base = ((size_t)(maxwin + 1) + 2 * (size_t)cu + (size_t)nb * d) * sizeof(double2) +
                         (size_t)cu * sizeof(int2) + 12 * sizeof(double) + tab_len * sizeof(int) +
-                        (size_t)cu * (2 * nb + shape_jumps(shape_id(P), nt) + 1) * sizeof(short);
-    bool want_fold = true, want_jc = variant != 0;
+                        (size_t)cu * (2 * nb + nt + 1) * sizeof(short);
+    bool want_fold = true, want_jc = (P->variant & 1) != 0;
     if (const char *env = std::getenv("GRAPE_FOLD")) want_fold = std::atoi(env) != 0;
     if (const char *env = std::getenv("GRAPE_JCACHE")) want_jc = want_jc && std::atoi(env) != 0;
     struct Opt { bool fold, jc; };
     const Opt opts[] = {{true, true}, {true, false}, {false, true}, {false, false}};
     size_t smem = 0;
     bool found = false, fold = false, jcache = false;
-    for (const Opt &o : opts) {
-        if ((o.fold && !want_fold) || (o.jc && !want_jc)) continue;
-        const size_t sm = base + (o.fold ? (size_t)cu * sizeof(double2) : 0) +
-                          (o.jc ? (size_t)njt * cu * sizeof(double) : 0);
-        if (sm + 1024 > (size_t)max_smem) continue;
-        int max_blocks = 0;
-        const cudaError_t e = P->prec == GRAPE_PREC_FP64
-                                  ? grape_prepare_grid_f64(variant, (size_t)max_smem, sm, &max_blocks)
-                                  : grape_prepare_grid_df(variant, (size_t)max_smem, sm, &max_blocks);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            continue;
+    // as on clusters: the compile-time layout, else the run-time one
+    // (Jaynes-Cummings up to d=638 and not only d=626)
+    const int layouts = h_jumps(shape, nt) > nt ? 2 : 1;
+    for (const Opt &o : opts)
+        for (int l = 0; l < layouts && !found; ++l) {
+            const int sh = l ? 0 : shape;
+            if ((o.fold && !want_fold) || (o.jc && !want_jc)) continue;
+            const size_t sm = base + (size_t)cu * (h_jumps(sh, nt) - nt) * sizeof(short) +
+                              (o.fold ? (size_t)cu * sizeof(double2) : 0) +
+                              (o.jc ? (size_t)njt * cu * sizeof(double) : 0);
+            if (sm + 1024 > (size_t)max_smem) continue;
+            int max_blocks = 0;
+            const int v = (P->variant & 1) | (sh << 2);
+            const cudaError_t e = P->prec == GRAPE_PREC_FP64
+                                      ? grape_prepare_grid_f64(v, (size_t)max_smem, sm, &max_blocks)
+                                      : grape_prepare_grid_df(v, (size_t)max_smem, sm, &max_blocks);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                continue;
+            }
+            if (max_blocks < nct * P->ns) continue;   // every CTA must be resident
+            variant = v;
+            smem = sm;
+            fold = o.fold;
+            jcache = o.jc;
+            found = true;
         }
-        if (max_blocks < nct * P->ns) continue;   // every CTA must be resident
-        smem = sm;
-        fold = o.fold;
-        jcache = o.jc;
-        found = true;
-        break;
-    }
     if (!found) return fail(GRAPE_EINVAL, "problem too large for the grid propagation kernel");
     int stride = 0;
     const std::vector<int> ntab = neighbour_table(tab, d, nct, hb, &stride);

@@ -49,3 +49,10 @@ RES, ALL = ("res_x", "res_y"), ("res_x", "res_y", "qub_x", "qub_y")
                                           (3, 201, ALL)])    # five complex bands
 def test_grid_kernel_takes_its_largest_problems(gp, Q, N, controls):
     check(gp, one_slice(Q, N, controls), "grid")
+
+
+@pytest.mark.parametrize("N,ns,kernel", [(319, 1, "grid"), (254, 2, "grid"), (108, 1, "hermitian-cluster")])
+def test_fewer_jump_terms_than_the_layout_has_room_for(gp, N, ns, kernel):
+    """Jaynes-Cummings has one jump term in a band layout built for three: where
+    the room for three does not fit, the run-time layout keeps one."""
+    check(gp, one_slice(2, N, RES, ns=ns, g=10.0, qubit_energy=(0.0, 1.0)), kernel)
