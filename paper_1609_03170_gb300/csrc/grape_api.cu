@@ -2872,8 +2872,14 @@ StaticPlan static_plan(const grape_problem *P) {
     const int nsplit = std::max(1, P->trace.nsplit);
     r.mat = align256(P->d2 * P->ns * sizeof(double2));
     auto per_seg = [&](long long sg) { return align256(stage_bytes(P, sg)); };
-    auto part_bytes = [&](long long sg) {
-        return nsplit > 1 ? align256((size_t)sg * nsplit * std::max(P->R, 1) * sizeof(double)) : 0;
+    // the partial traces; in first order, where a slice's trace is split over
+    // rows, they take the place of the propagated state, which is not read any
+    // more when a segment's traces run (a problem that needs every byte of the
+    // array for its states is not refused for their sake)
+    auto part_bytes = [&](long long sg) -> size_t {
+        if (nsplit <= 1) return 0;
+        const size_t n = align256((size_t)sg * nsplit * std::max(P->R, 1) * sizeof(double));
+        return P->mode == GRAPE_GRAD_FIRST_ORDER && n <= r.mat ? 0 : n;
     };
     // the longest segment that fits (fewest launches); the need is not
     // monotonic in the length (stage storage grows, checkpoints shrink), so
@@ -2947,7 +2953,7 @@ grape_status grape_gradient_static(grape_problem_t P, const double *u, double *F
     double2 *mu = reinterpret_cast<double2 *>(base + mat);
     double2 *Y = reinterpret_cast<double2 *>(base + 2 * mat);
     double2 *K = reinterpret_cast<double2 *>(base + 2 * mat + per);
-    double *part = reinterpret_cast<double *>(base + 2 * mat + 2 * per);
+    double *part = partb > 0 ? reinterpret_cast<double *>(base + 2 * mat + 2 * per) : reinterpret_cast<double *>(x);
     double2 *ckpt = reinterpret_cast<double2 *>(base + 2 * mat + 2 * per + partb);
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -56,3 +56,20 @@ def test_fewer_jump_terms_than_the_layout_has_room_for(gp, N, ns, kernel):
     """Jaynes-Cummings has one jump term in a band layout built for three: where
     the room for three does not fit, the run-time layout keeps one."""
     check(gp, one_slice(2, N, RES, ns=ns, g=10.0, qubit_energy=(0.0, 1.0)), kernel)
+
+
+@pytest.mark.parametrize("n_slices", [14, 15])
+def test_first_order_static_call_at_the_last_byte_of_its_scratch(gp, n_slices):
+    """At d=512 the states of 14 or 15 slices in segments of 3, with their
+    checkpoints, are exactly the 64 MiB of the no-allocation call; the partial
+    traces lie in a state that is no longer needed."""
+    torch = pytest.importorskip("torch")
+    w = workloads.jaynes_cummings(512, n_slices=n_slices)
+    P = gp.GrapeProblem.from_workload(w, grad_mode=gp._lib.GRAPE_GRAD_FIRST_ORDER)
+    F, G = P.gradient(w.u)
+    u = torch.from_numpy(w.u).cuda()
+    Fs, Gs = torch.empty(1, dtype=torch.float64, device="cuda"), torch.empty_like(u)
+    gp._lib.grape_gradient_static(P.handle, u.data_ptr(), Fs.data_ptr(), Gs.data_ptr(), 0)
+    torch.cuda.synchronize()
+    P.status()
+    assert Fs.item() == F and np.array_equal(Gs.cpu().numpy(), G)
