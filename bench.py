@@ -325,14 +325,14 @@ def run_batch256(args):
         torch.cuda.synchronize()
         seq_sample_ms += ev0.elapsed_time(ev1)
         Pi.close()
-    own = [p.geometry()[:2] for p in probs]
     t0 = time.perf_counter()
     B = GrapeBatch(probs, n_lanes=args.lanes)    # tunes the tile per d bucket
     tune_s = time.perf_counter() - t0
     tiles = {}
-    for w, p, o in zip(ws, probs, own):
-        b = f"d{32 * ((w.d - 1) // 32) + 1}-{32 * ((w.d - 1) // 32 + 1)}"
-        tiles.setdefault(b, set()).add(p.geometry()[:2])
+    for p in probs:                              # what runs: each reset problem's N x N blocks
+        d, _, _, c, t = p.running()
+        b = f"d{32 * ((d - 1) // 32) + 1}-{32 * ((d - 1) // 32 + 1)}"
+        tiles.setdefault(b, set()).add((c, t))
     tiles = {b: sorted(f"{c}x{t}" for c, t in v) for b, v in sorted(tiles.items())}
     F = torch.empty(256, dtype=torch.float64, device="cuda")
     Gs = [torch.empty((w.n_slices, w.n_controls), dtype=torch.float64, device="cuda") for w in ws]
@@ -389,7 +389,7 @@ def run_d600(args):
     P.status()
     print(json.dumps(_base_line(args, "transmon_resonator_d600", 1.0 / s, UNIT, 1000 * s, {
         "config": {"workload": "transmon_resonator_d600", "d": 600, "n_slices": n, "n_rk": 4,
-                   "n_states": 1, "ckpt_stride": 200, "kernel": P.kernel(),
+                   "n_states": 1, "ckpt_stride": 200, "kernel": P.running()[2], "block": P.running()[0],
                    "device_bytes": P.memory_bytes()},
         "phases_ms_per_step": {k: v[0] / args.steps for k, v in ph.items()},
         "gpu_launches": P.gradient_launches() * args.steps})), flush=True)
@@ -431,7 +431,7 @@ def run_d20(args):
     cpu = reps / (time.perf_counter() - t0)
     print(json.dumps(_base_line(args, "qubit_resonator_d20", 1000.0 / ms, UNIT, ms, {
         "config": {"workload": "qubit_resonator_d20", "d": 20, "n_slices": 200, "n_rk": 4,
-                   "n_states": 2, "cluster": P.geometry()[0], "l2": "inputs fit in L2 (small case)"},
+                   "n_states": 2, "cluster": P.running()[3], "l2": "inputs fit in L2 (small case)"},
         "cpu_baseline": {"value": cpu, "unit": UNIT, "cores": w.n_states, "kind": "oracle",
                          "sample": "the whole d=20 problem, 5 gradient evaluations"},
         "gpu_launches": P.gradient_launches() * args.steps})), flush=True)
@@ -567,7 +567,7 @@ def run_sweep(args):
             _lib.grape_gradient(P.handle, u.data_ptr(), F.data_ptr(), G.data_ptr(), stream.cuda_stream)
         ev1.record(stream)
         torch.cuda.synchronize()
-        gpu[d] = {"ms": ev0.elapsed_time(ev1) / reps, "kernel": P.kernel(), "cluster": P.geometry()[0]}
+        gpu[d] = {"ms": ev0.elapsed_time(ev1) / reps, "kernel": P.running()[2], "cluster": P.running()[3]}
         P.close()
     sparse.build()
     cpu = {}
@@ -890,7 +890,7 @@ def main():
         "config": {"workload": "transmon_resonator_d120", "d": w.d, "n_slices": w.n_slices,
                    "n_rk": w.n_rk, "n_states": w.n_states, "n_controls": w.n_controls,
                    "n_jumps": len(bm.jumps), "grad_mode": "exact",
-                   "cluster": P.geometry()[0], "parallelism": f"replicas{world}",
+                   "cluster": P.running()[3], "parallelism": f"replicas{world}",
                    "l2": "inputs larger than L2: %.1f GB of stage storage written and read per step"
                          % (step_bytes / 1e9)},
         "roofline": {"bound": "alu", "kernel": f"prop_kernel ({dom})", "achieved": achieved,

@@ -107,9 +107,12 @@ typedef struct grape_problem *grape_problem_t;
  * restricted to them - every term left out is an exact zero - and rho(T) is
  * returned at full size.  Where no operator connects two sectors of the basis
  * and no target reaches between them, calls that return Phi and the gradient
- * only run on a state's blocks within the sectors.  grape_problem_geometry, grape_problem_kernel,
- * grape_problem_set_tile and the limit of grape_gradient_static refer to the
- * problem at its full size.  Errors: GRAPE_EINVAL (sizes, band offsets beyond
+ * only run on a state's blocks within the sectors (so Phi of a superposition
+ * over sectors has the same bits from those calls, and may differ by rounding
+ * from the one of a grape_forward with rhoT).  grape_problem_geometry,
+ * grape_problem_kernel, grape_problem_set_tile and the limit of
+ * grape_gradient_static refer to the problem at its full size;
+ * grape_problem_running tells what is launched.  Errors: GRAPE_EINVAL (sizes, band offsets beyond
  * +-(d-1), non-Hermitian rho0 or control, negative rates), GRAPE_ENOMEM. */
 grape_status grape_problem_create(const grape_problem_desc *desc, grape_problem_t *out);
 
@@ -174,8 +177,11 @@ grape_status grape_gradient_filtered(grape_problem_t problem, int32_t n_steps, c
 /* Device memory the problem holds, in bytes (tables plus stage storage). */
 grape_status grape_problem_memory(grape_problem_t problem, size_t *bytes);
 
-/* Launch geometry chosen for the propagation kernels (cluster size, threads
- * per block, elements per thread).  For tests and benchmarks. */
+/* Launch geometry of the propagation kernels for the problem's full matrices
+ * (cluster size, threads per block, elements per thread); a problem on a part
+ * of the space launches another (grape_problem_running), and this is then the
+ * tile that its full size would take: 512 entries per CTA, or the last one that
+ * grape_problem_set_tile was given.  For tests and benchmarks. */
 grape_status grape_problem_geometry(grape_problem_t problem, int32_t *cluster,
                                     int32_t *threads, int32_t *elems_per_thread);
 
@@ -209,11 +215,24 @@ grape_status grape_problem_set_penalty(grape_problem_t problem, const double *di
  * owned entries rounded up to whole warps (at least 64). */
 grape_status grape_problem_set_tile(grape_problem_t problem, int32_t cluster, int32_t threads);
 
-/* Which propagation kernel the problem runs on: 0 = Hermitian cluster kernel
- * (upper triangle, states in distributed shared memory), 1 = full-matrix
- * cluster kernel, 2 = grid kernel (states in global memory, one cooperative
- * grid, for states too large for a cluster's shared memory). */
+/* Which propagation kernel the problem's full matrices need: 0 = Hermitian
+ * cluster kernel (upper triangle, states in distributed shared memory), 1 =
+ * full-matrix cluster kernel, 2 = grid kernel (states in global memory, one
+ * cooperative grid, for states too large for a cluster's shared memory).  A
+ * problem on a part of the space may run on another: grape_problem_running. */
 grape_status grape_problem_kernel(grape_problem_t problem, int32_t *kind);
+
+/* What the calls launch (see grape_problem_create): with_rho = 0, the problem
+ * that grape_gradient, the batch, the server and a grape_forward without rhoT
+ * run on; with_rho = 1, the one of a grape_forward with rhoT.  d and n_states
+ * are its dimension and number of states (a problem on blocks has more and
+ * smaller ones), kind its kernel as above, cluster and threads its tile (the
+ * grid kernel: CTAs per state), which grape_problem_set_tile and a batch or
+ * server that holds the problem change.  For tests and benchmarks; every
+ * output may be NULL. */
+grape_status grape_problem_running(grape_problem_t problem, int32_t with_rho, int32_t *d,
+                                   int32_t *n_states, int32_t *kind, int32_t *cluster,
+                                   int32_t *threads);
 
 /* Waits for the device and reports whether a bounded wait of the
  * problem's kernels gave up since the last check (GRAPE_ETIMEOUT; the

@@ -60,7 +60,7 @@ EXPORTS = ["grape_problem_create", "grape_problem_destroy", "grape_forward", "gr
            "grape_problem_set_penalty", "grape_set_profiling",
            "grape_phase_times", "grape_gradient_launches", "grape_gradient_static",
            "grape_batch_create", "grape_batch_destroy", "grape_batch_gradient", "grape_batch_info",
-           "grape_problem_kernel", "grape_problem_status", "grape_server_create",
+           "grape_problem_kernel", "grape_problem_running", "grape_problem_status", "grape_server_create",
            "grape_server_destroy", "grape_submit", "grape_poll",
            "grape_fma_peak", "grape_last_error", "grape_version"]
 
@@ -107,6 +107,8 @@ def load(build_if_missing: bool = True):
     lib.grape_poll.restype = c_int32
     lib.grape_problem_kernel.argtypes = [c_void_p, P(c_int32)]
     lib.grape_problem_kernel.restype = c_int32
+    lib.grape_problem_running.argtypes = [c_void_p, c_int32] + [P(c_int32)] * 5
+    lib.grape_problem_running.restype = c_int32
     lib.grape_problem_status.argtypes = [c_void_p]
     lib.grape_problem_status.restype = c_int32
     lib.grape_batch_create.argtypes = [P(c_void_p), c_int32, c_int32, P(c_void_p)]
@@ -240,6 +242,14 @@ def grape_problem_kernel(h) -> str:
     k = c_int32()
     check(load().grape_problem_kernel(h, ctypes.byref(k)), "grape_problem_kernel")
     return KERNEL_NAMES[int(k.value)]
+
+
+def grape_problem_running(h, with_rho: bool = False):
+    """(d, states, kernel, cluster, threads) of the problem that the calls launch."""
+    v = [c_int32() for _ in range(5)]
+    check(load().grape_problem_running(h, int(with_rho), *[ctypes.byref(x) for x in v]), "grape_problem_running")
+    d, ns, kind, cluster, threads = [int(x.value) for x in v]
+    return d, ns, KERNEL_NAMES[kind], cluster, threads
 
 
 def grape_problem_status(h) -> None:

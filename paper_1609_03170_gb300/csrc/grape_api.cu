@@ -692,6 +692,9 @@ grape_problem *grad_problem(grape_problem *P) {
     return P && P->split ? P->split : P;
 }
 
+// 0 Hermitian cluster, 1 full-matrix cluster, 2 grid kernel
+int32_t kernel_kind(const grape_problem *P) { return P->grid ? 2 : ((P->variant & 2) ? 0 : 1); }
+
 template <typename T>
 grape_status upload(grape_problem *P, const std::vector<T> &h, T **out) {
     *out = static_cast<T *>(P->alloc(h.size() * sizeof(T)));
@@ -2566,7 +2569,19 @@ grape_status grape_problem_status(grape_problem_t P) {
 
 grape_status grape_problem_kernel(grape_problem_t P, int32_t *kind) {
     if (!P || !kind) return fail(GRAPE_EINVAL, "NULL argument");
-    *kind = P->grid ? 2 : ((P->variant & 2) ? 0 : 1);
+    *kind = kernel_kind(P);
+    return GRAPE_OK;
+}
+
+grape_status grape_problem_running(grape_problem_t P, int32_t with_rho, int32_t *d, int32_t *n_states,
+                                   int32_t *kind, int32_t *cluster, int32_t *threads) {
+    if (!P) return fail(GRAPE_EINVAL, "NULL problem");
+    const grape_problem *A = with_rho ? active(P) : grad_problem(P);
+    if (d) *d = A->d;
+    if (n_states) *n_states = A->ns;
+    if (kind) *kind = kernel_kind(A);
+    if (cluster) *cluster = A->ncl;
+    if (threads) *threads = A->threads;
     return GRAPE_OK;
 }
 

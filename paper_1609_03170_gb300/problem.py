@@ -202,8 +202,13 @@ class GrapeProblem:
         return _lib.grape_gradient_launches(self._h)
 
     def kernel(self) -> str:
-        """hermitian-cluster, full-cluster or grid."""
+        """hermitian-cluster, full-cluster or grid: what the full matrices need."""
         return _lib.grape_problem_kernel(self._h)
+
+    def running(self, want_rho: bool = False):
+        """(d, states, kernel, cluster, threads) of what the gradient, or a
+        forward that returns rho(T), launches: the whole problem or its parts."""
+        return _lib.grape_problem_running(self._h, want_rho)
 
     def status(self) -> None:
         """Raise GrapeError(GRAPE_ETIMEOUT) if a grid barrier gave up."""
