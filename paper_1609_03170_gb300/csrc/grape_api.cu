@@ -3686,10 +3686,10 @@ int job_sm_demand(const grape_server *S, const ServerJob *j) {
     return P->grid ? S->n_sms : std::max(1, P->ns * P->ncl);
 }
 
-bool problem_busy(const grape_server *S, const grape_problem *P) {
-    for (const ServerJob *a : S->active)
-        if (a->P == P) return true;
-    return false;
+// a job of P runs or is about to (admitted in this pass)
+bool problem_busy(const grape_server *S, const std::vector<ServerJob *> &admit, const grape_problem *P) {
+    auto same = [P](const ServerJob *a) { return a->P == P; };
+    return std::any_of(S->active.begin(), S->active.end(), same) || std::any_of(admit.begin(), admit.end(), same);
 }
 
 void server_loop(grape_server *S) {
@@ -3706,7 +3706,7 @@ void server_loop(grape_server *S) {
             // admission: FIFO while slots are free and the estimated footprint fits
             while (!S->queue.empty() && (int)(S->active.size() + admit.size()) < S->max_slots) {
                 ServerJob *j = S->queue.front();
-                if (problem_busy(S, j->P)) break;
+                if (problem_busy(S, admit, j->P)) break;
                 // a grid-kernel job occupies every SM with one cooperative grid: it runs alone
                 bool grid_running = false;
                 for (const ServerJob *a : S->active) grid_running = grid_running || a->P->grid;
