@@ -656,7 +656,7 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
     using V = typename Num::val;
     using R = typename Num::real_t;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_err;
+    __shared__ int s_err, s_peer;
     const int d = p.d, d2 = d * d;
     const int NU = d * (d + 1) / 2;
     const int nbd = p.tab.nb * d;
@@ -704,6 +704,7 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
         mbar_init(mbar_sa + 8, 1u + (uint32_t)blockDim.x);
         mbar_init_fence();
     }
+    if (clu && threadIdx.x == 32) s_peer = __ldg(&p.htab[p.htab_len + rank]);   // window slots peers write each stage
     for (int i = threadIdx.x; i < p.htab_len; i += nth) tab[i] = __ldg(&p.htab[i]);
     const V vzero = Num::zero();
     for (int i = threadIdx.x; i < 2 * wst; i += nth) buf0[i] = Num::store(vzero);
@@ -784,9 +785,9 @@ __global__ void __launch_bounds__(GRAPE_PROP_THREADS, 1) prop_h_kernel(const Pro
         }
         e[0] = (uint32_t)n;
     }
-    // bytes peers push into this CTA's window each stage
-    const uint32_t expect = (uint32_t)__ldg(&p.htab[p.htab_len + rank]) * (uint32_t)sizeof(S);
     cluster_sync_all();   // every CTA runs, windows zeroed, mbarriers initialised, tables built
+    // bytes peers push into this CTA's window each stage
+    const uint32_t expect = (uint32_t)s_peer * (uint32_t)sizeof(S);
     const long long limit = 1LL << 31;          // SM cycles a window wait may take
     const uint32_t boff1 = (uint32_t)(wst * (int)sizeof(S));
 
@@ -1029,7 +1030,7 @@ __global__ void __launch_bounds__(EPT == 2 ? GRAPE_TWO_THREADS : GRAPE_PROP_THRE
     static_assert(NBR % 2 == 0 && NBC > 0 && NRP <= 3, "band row");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint64_t mbar[2];
-    __shared__ int s_err;
+    __shared__ int s_err, s_peer;
     __shared__ R s_uc[GRAPE_MAXR];                // the next slice's controls
     const int d = p.d, d2 = d * d;
     const int NU = d * (d + 1) / 2;
@@ -1072,6 +1073,7 @@ __global__ void __launch_bounds__(EPT == 2 ? GRAPE_TWO_THREADS : GRAPE_PROP_THRE
         mbar_init(mbar_sa + 8, 1u + (uint32_t)(nth >> 5));
         mbar_init_fence();
     }
+    if (clu && tid == 32) s_peer = __ldg(&p.htab[p.htab_len + rank]);   // window slots peers write each stage
     for (int i = tid; i < p.htab_len; i += nth) tab[i] = __ldg(&p.htab[i]);
     for (int i = tid; i < wst; i += nth) {
         buf0[i] = Num::store(Num::zero());
@@ -1238,9 +1240,9 @@ __global__ void __launch_bounds__(EPT == 2 ? GRAPE_TWO_THREADS : GRAPE_PROP_THRE
     bool mirror1[EPT];                            // the entry's mirror lies in a window too
 #pragma unroll
     for (int e = 0; e < EPT; ++e) mirror1[e] = mine[e] && ij1[e].y > ij1[e].x && ij1[e].y - ij1[e].x <= hb;
-    // bytes peers push into this CTA's window each stage
-    const uint32_t expect = (uint32_t)__ldg(&p.htab[p.htab_len + rank]) * (uint32_t)sizeof(S);
     cluster_sync_all();   // every CTA runs, windows zeroed, mbarriers initialised, tables built
+    // bytes peers push into this CTA's window each stage
+    const uint32_t expect = (uint32_t)s_peer * (uint32_t)sizeof(S);
     const long long limit = 1LL << 31;            // SM cycles a window wait may take
     bool failed = false;
 
