@@ -151,7 +151,7 @@ grape_status grape_gradient(grape_problem_t problem, const double *u, double *F,
  *   g_u[j][k] = sum_n T_k[n][j] g_s[n][k],
  * which turns dPhi/ds into dPhi/du.  u, s, g_s, g_u are device float64 arrays,
  * row-major [index][control]; omega0 is a host array of n_controls values.
- * Both run on `stream` in FP64 (one thread per output, only the band of
+ * Both run on `stream` in FP64 (a group of lanes per output, only the band of
  * terms that can be non-zero: erf saturates to +-1 exactly).  Errors:
  * GRAPE_EINVAL (NULL or host data pointers, n_steps or n_sub < 1,
  * n_controls outside [1, 8], Dt, dt or an omega0 not positive and finite),
@@ -206,13 +206,16 @@ grape_status grape_problem_set_penalty(grape_problem_t problem, const double *di
  * [64, 512]).  Every entry is computed by the same arithmetic whatever CTA
  * or thread owns it, so results do not change, bit for bit; only speed and
  * the SMs a call occupies do (narrow tiles leave room for other problems,
- * see grape_batch_create).  A problem that runs on a part of the space takes the
- * tile for that part too when it fits there.  Errors: GRAPE_EINVAL (values out of range, a
+ * see grape_batch_create).  The tile is tried on the problem's full matrices,
+ * which decide whether it is refused, and then set on the parts of the space
+ * that the problem runs on, which are smaller; a part that cannot take it all
+ * the same keeps its own (grape_problem_running tells).  Errors: GRAPE_EINVAL (values out of range, a
  * grid-kernel problem, or a tile whose state window does not fit in shared
  * memory or of which no cluster can be resident; the tile is unchanged),
- * GRAPE_ECUDA.  The tile chosen at create is the one of shortest stage
- * latency: about 128 to 160 entries per CTA up to 16 CTAs, threads for the
- * owned entries rounded up to whole warps (at least 64). */
+ * GRAPE_ECUDA.  The tile chosen at create for what runs is the one of shortest
+ * stage latency: about 128 to 160 entries per CTA up to 16 CTAs, threads for
+ * the owned entries rounded up to whole warps (at least 64; half as many for
+ * 513 to 768 entries, two each). */
 grape_status grape_problem_set_tile(grape_problem_t problem, int32_t cluster, int32_t threads);
 
 /* Which propagation kernel the problem's full matrices need: 0 = Hermitian
@@ -290,11 +293,11 @@ grape_status grape_gradient_static(grape_problem_t problem, const double *u, dou
  * d (32 wide): for the bucket's largest problem it times every tile that
  * fits (cluster width x threads per CTA, see grape_problem_set_tile) on a
  * few slices of forward propagation run as concurrent copies, as many as
- * can be resident at once, and sets the tile of highest throughput on the
- * bucket's problems (their own tiles come back at grape_batch_destroy;
- * GRAPE_BATCH_TUNE=0 skips the tuning).  The problems are then spread over
- * n_lanes concurrent streams, longest
- * first to the least loaded lane; each lane owns stage storage sized for its
+ * can be resident at once and no more than the batch has problems, and sets
+ * the tile of highest throughput on the bucket's problems (their own tiles
+ * come back at grape_batch_destroy; GRAPE_BATCH_TUNE=0 skips the tuning).  The
+ * problems are then spread over n_lanes concurrent streams, longest first to
+ * the least loaded lane; each lane owns stage storage sized for its
  * largest problem (with checkpoint segments that keep every lane within an
  * equal share of 60% of the free device memory) and runs its problems one
  * after another.  The first grape_batch_gradient call captures the whole

@@ -1180,7 +1180,13 @@ grape_status plan_h(grape_problem *P, int ncl, int threads) {
 // lets both sweeps' clusters of every state be resident (eight of 16 CTAs).
 // Threads: whole warps for the owned entries, at least 64 (a warp without
 // entries still takes part in every barrier: d=60 1.56 against 1.64 ms); for
-// 513 to 768 entries half as many threads with two entries each.
+// 513 to 768 entries half as many threads with two entries each, whichever
+// kernel the tile gets.  Measured, ms per gradient on half and on 512 threads:
+// prop_s_kernel with two entries in registers d=144 2.67 (3.10), d=148 2.69
+// (3.38); its windows beyond 32 KB (data in shared memory) d=152 3.30 (3.35);
+// the run-time layout d=129 4.07 (4.11), d=138 4.27 (4.34), d=144 4.32 (4.29),
+// d=156 4.47 (4.55), in FP64 d=132 3.28 (3.61), with controlled rates d=132 6.23
+// (6.42): the same or faster, at worst 0.7 % slower.
 // A problem that is only there for its full size (geometry_only) reports 512
 // entries per CTA and 512 threads, whole warps when one CTA holds the state.
 grape_status choose_geometry_h(grape_problem *P, bool geometry_only) {
